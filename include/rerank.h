@@ -66,7 +66,10 @@ typedef struct {
   int device;                /* CUDA device ordinal */
   int precision;             /* RERANK_PREC_*; default FP32 */
   int rescore_m;             /* extra candidates kept per row before exact rescoring; default 16
-                                (an autotuner table entry may override it per instance size) */
+                                (an autotuner table entry may override it per instance size).
+                                With 16 or more the BF16 / FP8 paths keep full lists of 64
+                                candidates where memory allows; smaller values are kept as given.
+                                The exact lists are the same for any value */
   float alpha;               /* exponent of Eq. 14; default 2 */
   int aggregator;            /* RERANK_AGG_*; default SUM (Sec. 4.1); MEAN divides the k2 messages'
                                 weights by k2; MAX takes their element-wise max (Eq. 13 variants) */
@@ -252,7 +255,7 @@ rerank_status rerank_gallery_unload(rerank_ctx* ctx);
  *   refine_order  1 = refine rows cluster by cluster, 0 = in index order
  *   rescore_m     candidates kept beyond k1 (-1 = cfg.rescore_m); the lists
  *                 stay exact for any value, only the work moves between stages.
- *                 Serving always uses cfg.rescore_m. */
+ *                 Serving does not use it. */
 typedef struct {
   int sim_chunks;
   int prop_warps;
@@ -325,7 +328,8 @@ rerank_status rerank_knn_noalloc(const void* x, int64_t n, int d, int dtype, int
 /* Counters of the last rerank_run / rerank_knn call on this context. */
 typedef struct {
   int64_t n_vertices;
-  int64_t candidates_per_row;  /* K = min(k1 + m, n), m = rescore_m or the tuned margin */
+  int64_t candidates_per_row;  /* K = min(k1 + m, n), m = rescore_m or the tuned margin, or
+                                  min(64, n) where the lists are full (see rerank_config) */
   int64_t fp64_rescored;       /* candidate scores recomputed in FP64 near a tie */
   int64_t fallback_rows;       /* rows whose first candidate list could not be certified */
   int64_t exact_scan_rows;     /* rows finally redone by the exact FP32 scan of all columns */

@@ -120,6 +120,12 @@ size_t carve(Carver& c, const Shape& sh, Buffers& b, int sm_count, int precision
     b.fb3_count = c.take<int32_t>(4);
   }
   b.row_floor = c.take<int>(size_t(n));
+  if (sh.segs > 0) {
+    b.ap.xsample = c.take<char>(size_t(sh.sample) * sh.dp * (precision == RERANK_PREC_FP8 ? 1 : 2));
+    b.ap.sample_scale = c.take<float>(size_t(sh.sample));
+    b.ap.cand = c.take<int64_t>(size_t(n) * sh.segs * sh.seg_cap);
+    b.ap.seg_cnt = c.take<int32_t>(size_t(n) * sh.segs);
+  }
   b.work = c.take<int32_t>(16);
   b.nb4 = c.take<int32_t>(4 * size_t(n));
   b.label = c.take<int32_t>(size_t(n));
@@ -196,7 +202,12 @@ rerank_status ensure_workspace(rerank_ctx* ctx, size_t bytes) {
   }
   const size_t want = bytes + bytes / 8;
   const size_t alloc = (ctx->cfg.hbm_budget && want > ctx->cfg.hbm_budget) ? bytes : want;
-  RR_CUDA(cudaMalloc(&ctx->ws, alloc));
+  const cudaError_t e = cudaMalloc(&ctx->ws, alloc);
+  if (e != cudaSuccess) {
+    ctx->ws = nullptr;
+    cudaGetLastError();  // the caller may go on with a smaller plan
+    return cuda_fail(e, "cudaMalloc(workspace)");
+  }
   ctx->ws_bytes = alloc;
   return RERANK_OK;
 }
@@ -268,6 +279,8 @@ rerank_status enqueue_job(rerank_ctx* ctx, const JobRun& j, cudaStream_t s, Stag
     }
     nl += launch_normalize(sh, dq, dg, b.xhat, b.norm, b.xlow, b.xhi, b.xlo, b.xscale, b.err, b.emax, prec, status,
                            s);
+    if (sh.sample > 0 && !(phases & kPhaseSim))
+      nl += launch_sample_rows(sh, b.xlow, prec == RERANK_PREC_FP8, b.xscale, b.ap, s);
     mark("normalize");
   }
   ErrModel em;
@@ -290,7 +303,7 @@ rerank_status enqueue_job(rerank_ctx* ctx, const JobRun& j, cudaStream_t s, Stag
       nl += launch_sim_fp32_topk(sh, b.xhat, b.row_floor, b.part_s, b.part_i, ctx->sm_count, s);
     } else {
       const int r = launch_sim_tc_topk(sh, b.xlow, prec == RERANK_PREC_FP8, b.xscale, b.row_floor, b.part_s,
-                                       b.part_i, status, ctx->sm_count, s, b.work);
+                                       b.part_i, status, ctx->sm_count, s, b.work, b.ap);
       if (r < 0) return RERANK_ECUDA;
       nl += r;
     }
@@ -301,14 +314,25 @@ rerank_status enqueue_job(rerank_ctx* ctx, const JobRun& j, cudaStream_t s, Stag
     *launches += nl;
     return RERANK_OK;
   }
+  // Batched calls run the similarity launch over all instances: its selection
+  // (like the sampled rows it started from) belongs to each instance.
+  if (sh.segs > 0 && !(phases & kPhaseSim)) nl += launch_select(sh, b.ap, b.part_s, b.part_i, status, s);
   const int32_t* order = nullptr;
   if (sh.tune.refine_order) {
     nl += launch_cluster_order(sh, b.part_s, b.part_i, b.nb4, b.label, b.ord_cnt, b.ord_start, b.ord_fill, b.order,
                                s);
     order = b.order;
   }
+  // Rows passed on start the recheck with floors from this stage's lists.
+  RefineFloors fl;
+  fl.in = b.row_floor;
+  if (prec != RERANK_PREC_FP32) {
+    fl.next = b.row_floor3;
+    fl.next_K = prec == RERANK_PREC_FP8 ? sh.K3 : sh.K;
+    fl.skip = true;
+  }
   nl += launch_refine(sh, dq, dg, b.xhat, b.norm, b.part_s, b.part_i, sh.P, em, order, nullptr, true, b.knn_idx,
-                      b.knn_score, b.fb_rows, b.fb_count, status, s);
+                      b.knn_score, b.fb_rows, b.fb_count, status, s, -1, -1, fl);
   RR_CUDA(cudaGetLastError());
   mark("refine");
   const int32_t* exact_rows = b.fb_rows;
@@ -320,6 +344,7 @@ rerank_status enqueue_job(rerank_ctx* ctx, const JobRun& j, cudaStream_t s, Stag
     nl += launch_gather_rows(b.fb_rows, b.fb_count, b.xhi, b.xlo, b.ahi, b.alo, sh.n, sh.dp, s);
     const int32_t* split_rows = b.fb_rows;
     const int32_t* split_count = b.fb_count;
+    int* split_floor = b.row_floor3;
     if (prec == RERANK_PREC_FP8) {
       // FP8 leaves most rows uncertified (its bound is ~0.07): a single-product
       // BF16 stage (the hi copies, bound ~3e-3) with the longest candidate
@@ -330,28 +355,36 @@ rerank_status enqueue_job(rerank_ctx* ctx, const JobRun& j, cudaStream_t s, Stag
       Shape sh3 = sh;
       sh3.K = sh.K3;
       const int rg = launch_sim_tc_gather_topk(sh3, sh.P3g, b.ahi, b.xhi, b.fb_rows, b.fb_count, b.row_floor3,
-                                               b.part3_s, b.part3_i, status, ctx->sm_count, s);
+                                               b.part3_s, b.part3_i, status, ctx->sm_count, s, true);
       if (rg < 0) return RERANK_ECUDA;
       nl += rg;
       // the hi copy is not the FP8 copy: its own bound ||x - hi|| = ||lo + r||
       ErrModel eh = em;
       eh.kind = 3;
       eh.eps = (sh.dp / 16 + 32) * 2.0 * kU32 + 8.0 * kU32;
+      RefineFloors fm;
+      fm.in = b.row_floor3;
+      fm.next = b.row_floor;  // the first pass's floors are done with
+      fm.next_K = sh.K;
+      fm.skip = true;
       nl += launch_refine(sh3, dq, dg, b.xhat, b.norm, b.part3_s, b.part3_i, sh.P3g, eh, b.fb_rows, b.fb_count,
-                          false, b.knn_idx, b.knn_score, b.fb3_rows, b.fb3_count, status, s, -1, kStFallbackMid);
+                          false, b.knn_idx, b.knn_score, b.fb3_rows, b.fb3_count, status, s, -1, kStFallbackMid, fm);
       nl += launch_gather_rows(b.fb3_rows, b.fb3_count, b.xhi, b.xlo, b.ahi, b.alo, sh.n, sh.dp, s);
       split_rows = b.fb3_rows;
       split_count = b.fb3_count;
+      split_floor = b.row_floor;
     }
     const int r = launch_sim_tc_split_topk(sh, sh.P3, b.ahi, b.alo, b.xhi, b.xlo, split_rows, split_count,
-                                           b.row_floor3, b.part3_s, b.part3_i, status, ctx->sm_count, s);
+                                           split_floor, b.part3_s, b.part3_i, status, ctx->sm_count, s, true);
     if (r < 0) return RERANK_ECUDA;
     nl += r;
     ErrModel e3 = em;
     e3.kind = 2;
     e3.eps = (3 * (sh.dp / 16) + 32) * 2.0 * kU32 + 8.0 * kU32;
+    RefineFloors f3;
+    f3.in = split_floor;
     nl += launch_refine(sh, dq, dg, b.xhat, b.norm, b.part3_s, b.part3_i, sh.P3, e3, split_rows, split_count, false,
-                        b.knn_idx, b.knn_score, b.fb2_rows, b.fb2_count, status, s, -1, kStFallback2);
+                        b.knn_idx, b.knn_score, b.fb2_rows, b.fb2_count, status, s, -1, kStFallback2, f3);
     exact_rows = b.fb2_rows;
     exact_count = b.fb2_count;
     RR_CUDA(cudaGetLastError());
@@ -470,14 +503,31 @@ rerank_status map_status(const long long* h, int precision, rerank_info* info, i
   return RERANK_OK;
 }
 
+// The same instance planned for the list kernels of the similarity stage.
+rerank_status plan_lists(const rerank_ctx* ctx, Shape* sh) {
+  const Shape o = *sh;
+  return plan_shape(ctx, o.nq, o.ng, o.d, o.dtype, o.k1, o.k2, o.layers, o.topk, o.knn_only, o.host_in, o.host_out,
+                    o.cap_h, sh, nullptr, false);
+}
+
 // One attempt of the pipeline.  Returns OK, or the mapped device error.
 rerank_status run_once(rerank_ctx* ctx, const void* xq, const void* xg, int32_t* out_idx, float* out_dist,
                        cudaStream_t s) {
   JobRun j;
   j.sh = ctx->shape;
   Carver dry;
-  const size_t need = carve(dry, j.sh, j.b, ctx->sm_count, ctx->cfg.precision);
+  size_t need = carve(dry, j.sh, j.b, ctx->sm_count, ctx->cfg.precision);
   rerank_status st = ensure_workspace(ctx, need);
+  if ((st == RERANK_EBUDGET || st == RERANK_ENOMEM) && j.sh.segs > 0) {
+    // No room for the append pass's segments: the list kernels need less.
+    st = plan_lists(ctx, &j.sh);
+    if (st != RERANK_OK) return st;
+    ctx->shape = j.sh;
+    j.b = Buffers{};
+    Carver again;
+    need = carve(again, j.sh, j.b, ctx->sm_count, ctx->cfg.precision);
+    st = ensure_workspace(ctx, need);
+  }
   if (st != RERANK_OK) return st;
   Carver real;
   real.base = ctx->ws;
@@ -511,7 +561,7 @@ rerank_status run_once(rerank_ctx* ctx, const void* xq, const void* xg, int32_t*
 // Shape of one instance.  cap_hint: a layer capacity learned from an earlier overflow.
 rerank_status plan_shape(const rerank_ctx* ctx, int64_t nq, int64_t ng, int d, int dtype, int k1, int k2, int layers,
                          int64_t topk, bool knn_only, bool host_in, bool host_out, int64_t cap_hint, Shape* out,
-                         const Tuning* tune) {
+                         const Tuning* tune, bool append) {
   Shape sh;
   sh.nq = nq;
   sh.ng = ng;
@@ -534,7 +584,14 @@ rerank_status plan_shape(const rerank_ctx* ctx, int64_t nq, int64_t ng, int d, i
   if (k1 > RERANK_MAX_K1 || k1 > kmax) return RERANK_EUNSUPPORTED;
   sh.tune = tune ? *tune : (ctx->force_tune ? *ctx->force_tune : lookup_tuning(ctx, prec, sh.n, d));
   const int m = sh.tune.rescore_m >= 0 ? sh.tune.rescore_m : ctx->cfg.rescore_m;
-  int64_t K = std::min<int64_t>(int64_t(k1) + std::max(m, 0), sh.n);
+  // The append pass and its selection cost hardly more for a full list than
+  // for k1 + 16 places, and every row certified by its first list saves three
+  // tensor-core products over all columns in the recheck (market: 4,004 rows
+  // with 42 places, 6 with 64; recheck 0.88 -> 0.19 ms).  Smaller margins that
+  // the caller or the tuning table asks for are kept.
+  const bool may_append = tc && append && tc_append_ok(sh.np, ctx->sm_count);
+  const bool full = may_append && sh.tune.rescore_m < 0 && m >= 16;
+  int64_t K = std::min<int64_t>(full ? kmax : int64_t(k1) + std::max(m, 0), sh.n);
   K = std::min<int64_t>(K, kmax);
   sh.K = int(K);
   // P counts candidate lists per row: one per column chunk on the FP32 path; the
@@ -546,8 +603,14 @@ rerank_status plan_shape(const rerank_ctx* ctx, int64_t nq, int64_t ng, int d, i
   // take 256) times column chunks, spread over the SMs (or SM pairs).
   const int irows = tc ? tc_item_rows() : 128;
   const int units = ctx->sm_count * 128 / irows;
-  const int chunks = choose_chunks(sh.np / irows, sh.np / (tc ? 256 : 128), units, sh.tune.sim_chunks);
+  int chunks = choose_chunks(sh.np / irows, sh.np / (tc ? 256 : 128), units, sh.tune.sim_chunks);
+  // An item of the paired kernels spans at most tc_max_item_tiles() tiles.
+  if (tc) chunks = std::max<int>(chunks, int((sh.np / 256 + tc_max_item_tiles() - 1) / tc_max_item_tiles()));
   sh.P = std::min(chunks, 32 / lpc) * lpc;
+  if (may_append) {
+    tc_append_plan(sh.n, sh.np, sh.dp, sh.K, chunks, &sh.segs, &sh.seg_cap, &sh.sample);
+    sh.P = 1;
+  }
   // The recheck covers an unknown, usually small, set of rows: many short chunks keep every SM busy.
   sh.P3 = tc ? int(std::min<int64_t>(32 / lpc3, sh.np / 256)) * lpc3 : 0;
   sh.P3g = prec == RERANK_PREC_FP8 ? int(std::min<int64_t>(32 / lpc, sh.np / 256)) * lpc : 0;
@@ -657,8 +720,8 @@ uint64_t buffer_id(const void* p) {
 // workspace offset they fix everything a batched call enqueues for it.
 void shape_key(const Shape& sh, std::vector<int64_t>& k) {
   const int64_t v[] = {sh.nq, sh.ng, sh.n, sh.np, sh.d, sh.dp, sh.dtype, sh.k1, sh.k2, sh.layers, sh.K, sh.P, sh.P3,
-                       sh.P3g, sh.K3, sh.topk, sh.host_in, sh.host_out, sh.knn_only, sh.ext_feat, sh.cap_h, sh.cap_csc,
-                       sh.hash_slots, sh.rank_ctas, sh.rank_scratch_per_cta, sh.tune.sim_chunks, sh.tune.prop_warps,
+                       sh.P3g, sh.K3, sh.segs, sh.seg_cap, sh.sample, sh.topk, sh.host_in, sh.host_out, sh.knn_only,
+                       sh.ext_feat, sh.cap_h, sh.cap_csc, sh.hash_slots, sh.rank_ctas, sh.rank_scratch_per_cta, sh.tune.sim_chunks, sh.tune.prop_warps,
                        sh.tune.refine_order, sh.tune.rescore_m, sh.tune.rank_threads};
   k.insert(k.end(), std::begin(v), std::end(v));
 }
@@ -729,31 +792,41 @@ double job_cost(const Shape& sh) {
 
 rerank_status run_batch(rerank_ctx* ctx, rerank_job* jobs, int njobs, cudaStream_t s) {
   std::vector<JobRun> runs(static_cast<size_t>(njobs));
-  size_t total = 0;
   const size_t st_bytes = sizeof(long long) * kStCount;
   std::vector<size_t> off(static_cast<size_t>(njobs));
-  for (int i = 0; i < njobs; ++i) {
-    const rerank_job& jb = jobs[i];
-    const bool host_in = is_host_ptr(jb.xq) || is_host_ptr(jb.xg);
-    const bool host_out = is_host_ptr(jb.out_idx) || is_host_ptr(jb.out_dist);
-    const int64_t topk = jb.topk_out ? jb.topk_out : jb.ng;
-    rerank_status st = plan_shape(ctx, jb.nq, jb.ng, jb.d, jb.dtype, jb.k1, jb.k2, jb.layers, topk, false, host_in,
-                                  host_out, 0, &runs[size_t(i)].sh);
-    if (st != RERANK_OK) return st;
-    Carver dry;
-    const size_t need = carve(dry, runs[size_t(i)].sh, runs[size_t(i)].b, ctx->sm_count, ctx->cfg.precision);
-    total = (total + 255) & ~size_t(255);
-    off[size_t(i)] = total;
-    total += ((st_bytes + 255) & ~size_t(255)) + need;
-  }
   // Tensor-core precisions: the similarity stage of all instances runs as
   // persistent launches over many instances (their tables live here).
   const bool tc_batch = ctx->cfg.precision != RERANK_PREC_FP32;
   const size_t inst_bytes = tc_batch_inst_bytes() * size_t(njobs);
-  total = (total + 255) & ~size_t(255);
-  const size_t inst_off = total;
-  if (tc_batch) total += inst_bytes;
-  rerank_status st = ensure_workspace(ctx, total);
+  size_t inst_off = 0, total = 0;
+  rerank_status st = RERANK_OK;
+  // With the append pass's segments; without them where they do not fit.
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    bool append = false;
+    total = 0;
+    for (int i = 0; i < njobs; ++i) {
+      const rerank_job& jb = jobs[i];
+      JobRun& run = runs[size_t(i)];
+      run = JobRun{};
+      const bool host_in = is_host_ptr(jb.xq) || is_host_ptr(jb.xg);
+      const bool host_out = is_host_ptr(jb.out_idx) || is_host_ptr(jb.out_dist);
+      const int64_t topk = jb.topk_out ? jb.topk_out : jb.ng;
+      st = plan_shape(ctx, jb.nq, jb.ng, jb.d, jb.dtype, jb.k1, jb.k2, jb.layers, topk, false, host_in, host_out, 0,
+                      &run.sh, nullptr, attempt == 0);
+      if (st != RERANK_OK) return st;
+      append = append || run.sh.segs > 0;
+      Carver dry;
+      const size_t need = carve(dry, run.sh, run.b, ctx->sm_count, ctx->cfg.precision);
+      total = (total + 255) & ~size_t(255);
+      off[size_t(i)] = total;
+      total += ((st_bytes + 255) & ~size_t(255)) + need;
+    }
+    total = (total + 255) & ~size_t(255);
+    inst_off = total;
+    if (tc_batch) total += inst_bytes;
+    st = ensure_workspace(ctx, total);
+    if (!append || (st != RERANK_EBUDGET && st != RERANK_ENOMEM)) break;
+  }
   if (st != RERANK_OK) return st;
   st = ensure_streams(ctx);
   if (st != RERANK_OK) return st;
@@ -822,13 +895,13 @@ rerank_status run_batch(rerank_ctx* ctx, rerank_job* jobs, int njobs, cudaStream
         const bool fp8 = ctx->cfg.precision == RERANK_PREC_FP8;
         std::vector<TcBatchInst> group;
         size_t used = 0;
-        for (int eg = 1; eg <= 2 && r == RERANK_OK; ++eg) {
+        for (int eg = 0; eg <= 2 && r == RERANK_OK; ++eg) {  // 0: the append pass
           group.clear();
           for (size_t p = 0; p <= idx.size(); ++p) {
             const bool end = p == idx.size();
             if (!end) {
               const JobRun& j = runs[size_t(idx[p])];
-              if (tc_lists_per_chunk(j.sh.dp, 1) != eg) continue;
+              if ((j.sh.segs > 0 ? 0 : tc_lists_per_chunk(j.sh.dp, 1)) != eg) continue;
               TcBatchInst t{};
               t.xlow = j.b.xlow;
               t.n = j.sh.n;
@@ -840,6 +913,10 @@ rerank_status run_batch(rerank_ctx* ctx, rerank_job* jobs, int njobs, cudaStream
               t.row_floor = j.b.row_floor;
               t.part_s = j.b.part_s;
               t.part_i = j.b.part_i;
+              t.segs = j.sh.segs;
+              t.seg_cap = j.sh.seg_cap;
+              t.sample = j.sh.sample;
+              t.ap = j.b.ap;
               t.status = j.st;
               group.push_back(t);
             }

@@ -50,6 +50,14 @@ struct TuneEntry {
 };
 int tune_bucket(int64_t n);  // half-octave bucket of the vertex count
 
+// Buffers of the tensor-core similarity stage's append pass.
+struct TcAppend {
+  void* xsample = nullptr;       // sample x dp: sampled rows of the low-precision copy
+  float* sample_scale = nullptr; // sample: their FP8 scales
+  void* cand = nullptr;          // n x segs x seg_cap (score, vertex) pairs, 8 bytes each
+  int32_t* seg_cnt = nullptr;    // n x segs
+};
+
 // Device pointers of one pipeline run (all inside the workspace block).
 struct Buffers {
   // inputs staged from host memory, when the caller passed host buffers
@@ -76,6 +84,7 @@ struct Buffers {
   int32_t* fb3_rows = nullptr;   // n: FP8 path, rows left after the single-product BF16 recheck stage
   int32_t* fb3_count = nullptr;
   int* row_floor = nullptr;      // n, shared K-th best per row (similarity kernels)
+  TcAppend ap;                   // append pass of the similarity stage
   int32_t* nb4 = nullptr;        // 4n: best candidates per row (processing order)
   int32_t* label = nullptr;      // n
   int32_t* order = nullptr;      // n: rows grouped by cluster
@@ -135,6 +144,9 @@ struct Shape {
   int k1 = 0, k2 = 0, layers = 0, K = 0, P = 0;
   int P3 = 0;              // candidate lists per row of the hi/lo recheck
   int P3g = 0;             // FP8 path: lists per row of the single-product BF16 recheck stage
+  int segs = 0;            // append pass: segments per row (0: the list kernels)
+  int seg_cap = 0;         // entries of a segment
+  int sample = 0;          // columns sampled for its floors (0: none)
   int K3 = 0;              // FP8 path: candidates per list of that stage (the longest list the kernels hold)
   int64_t topk = 0;
   bool host_in = false, host_out = false;
@@ -229,9 +241,22 @@ int launch_gather_rows(const int32_t* rows, const int32_t* count, const __nv_bfl
 int launch_sim_fp32_topk(const Shape& sh, const float* xhat, int* row_floor, float* part_s, int32_t* part_i,
                          int sm_count, cudaStream_t s);
 // work (4 bytes, nullable): counter for the dynamic item order of the main pass.
+// With sh.segs > 0 the lists come from the append pass and its selection (one
+// list per row; `ap` holds its buffers), and a row's floor may lie above its
+// K-th best score: the refinement bounds the columns left out by the floor.
 int launch_sim_tc_topk(const Shape& sh, const void* xlow, bool fp8, const float* inv_scale, int* row_floor,
                        float* part_s, int32_t* part_i, long long* status, int sm_count, cudaStream_t s,
-                       int32_t* work = nullptr);
+                       int32_t* work = nullptr, const TcAppend& ap = TcAppend{});
+// The append pass (pairs): segments per row, their capacity and the sample's
+// size for n rows (np padded) and lists of K, from the column chunks the work
+// split wants.  tc_append_ok: whether it can run (else the list kernels do).
+bool tc_append_ok(int64_t np, int sm_count);
+void tc_append_plan(int64_t n, int64_t np, int dp, int K, int chunks, int* segs, int* cap, int* sample);
+int launch_sample_rows(const Shape& sh, const void* xlow, bool fp8, const float* inv_scale, const TcAppend& ap,
+                       cudaStream_t s);
+// The append pass's segments into one sorted list of K per row.
+int launch_select(const Shape& sh, const TcAppend& ap, float* part_s, int32_t* part_i, const long long* status,
+                  cudaStream_t s);
 // Rectangular block: rows of `a` (a_rows of them, vertices row0 ..) against the
 // columns of `b` (b_cols, vertices col0 ..); per row P lists of its best K
 // columns (vertex indices) in part_s/part_i [a_rows][P][K].  Rows and columns
@@ -240,14 +265,25 @@ int launch_sim_tc_topk(const Shape& sh, const void* xlow, bool fp8, const float*
 int launch_sim_tc_rect_topk(const Shape& sh, const void* a, int64_t a_rows, int64_t row0, const void* b,
                             int64_t b_cols, int64_t col0, int chunks, bool fp8, const float* inv_scale,
                             int* row_floor, float* part_s, int32_t* part_i, long long* status, int sm_count,
-                            cudaStream_t s);
+                            cudaStream_t s, bool seeded = false);  // seeded: row_floor holds starting floors
+// Rows 0 .. a_rows - 1 of x against all sh.n rows of x (vertices in order) by
+// the append pass, with floors from the tc_rows_append_sample() sampled rows in
+// ap.xsample / ap.sample_scale; one list of sh.K per row.  chunks: at most
+// tc_rows_append_segs() / 4; cap: tc_rows_append_cap of them.
+int launch_sim_tc_rows_append(const Shape& sh, const void* x, int64_t a_rows, int chunks, bool fp8,
+                              const float* inv_scale, int* row_floor, const TcAppend& ap, int cap, float* part_s,
+                              int32_t* part_i, long long* status, int sm_count, cudaStream_t s);
+int tc_rows_append_sample();
+int tc_rows_append_segs();
+int tc_rows_append_cap(int64_t n, int K, int chunks);
 // hi/lo split: S' = hi_i.hi_j + lo_i.hi_j + hi_i.lo_j for the rows rows[0 .. *count)
 // (their hi/lo copies gathered in ahi/alo) against every column; lists indexed by
-// position in `rows`, P3 chunks.
+// position in `rows`, P3 chunks.  seeded: row_floor holds starting floors
+// (RefineFloors::next); otherwise the launcher resets it.
 int launch_sim_tc_split_topk(const Shape& sh, int P3, const __nv_bfloat16* ahi, const __nv_bfloat16* alo,
                              const __nv_bfloat16* bhi, const __nv_bfloat16* blo, const int32_t* rows,
                              const int32_t* count, int* row_floor, float* part_s, int32_t* part_i,
-                             long long* status, int sm_count, cudaStream_t s);
+                             long long* status, int sm_count, cudaStream_t s, bool seeded = false);
 
 // One instance of a batched similarity launch: the instance's low-precision
 // copy (np x dp) against itself, P lists of K per row.
@@ -259,10 +295,12 @@ struct TcBatchInst {
   int* row_floor;
   float* part_s;
   int32_t* part_i;
+  int segs, seg_cap, sample;
+  TcAppend ap;
   long long* status;
 };
-// Up to 64 instances with the same tc_lists_per_chunk(dp, 1) in one persistent
-// launch.  insts_dev: ninst * tc_batch_inst_bytes() of device memory; staging:
+// Up to 64 instances in one persistent launch: all on the append pass, or all
+// on the list kernels with the same tc_lists_per_chunk(dp, 1).  insts_dev: ninst * tc_batch_inst_bytes() of device memory; staging:
 // as many bytes of pinned host memory, untouched until the launch has run.
 int launch_sim_tc_batch(const TcBatchInst* in, int ninst, bool fp8, void* insts_dev, void* staging, int sm_count,
                         cudaStream_t s);
@@ -274,7 +312,8 @@ int tc_stall_hook();  // nonzero while the tensor-core kernels' test stall is se
 // column's hi copy, one product: the middle stage of the FP8 path's recheck.
 int launch_sim_tc_gather_topk(const Shape& sh, int P, const __nv_bfloat16* ahi, const __nv_bfloat16* bhi,
                               const int32_t* rows, const int32_t* count, int* row_floor, float* part_s,
-                              int32_t* part_i, long long* status, int sm_count, cudaStream_t s);
+                              int32_t* part_i, long long* status, int sm_count, cudaStream_t s,
+                              bool seeded = false);
 
 // Bound on |approximate score - S_ij| used to certify a row's candidate list.
 struct ErrModel {
@@ -284,6 +323,20 @@ struct ErrModel {
   const float* emax = nullptr;
   int64_t np = 0;
 };
+// Floors around a refinement stage.  in: the floors its similarity pass used
+// (indexed like the candidate lists; null: none), which bound the columns left
+// out of a list of fewer than K entries.  next: starting floors for the stage
+// that rechecks the rows passed on (by position; null: none), for lists of
+// next_K entries: the row's next_K-th approximate score less a part of its
+// error bound.  skip: a row that its approximate scores say cannot be
+// certified is passed on without rescoring (only where another list stage
+// follows).
+struct RefineFloors {
+  const int* in = nullptr;
+  int* next = nullptr;
+  int next_K = 0;
+  bool skip = false;
+};
 // Rows: all n in index order; or rows[0 .. *count) (count == nullptr: n) in that order,
 // with the candidate lists indexed by row (part_by_row) or by position in `rows`.
 int launch_refine(const Shape& sh, const void* xq, const void* xg, const float* xhat,
@@ -291,10 +344,12 @@ int launch_refine(const Shape& sh, const void* xq, const void* xg, const float* 
                    const int32_t* rows, const int32_t* count, bool part_by_row,
                    int32_t* knn_idx, float* knn_score, int32_t* fb_rows, int32_t* fb_count,
                    long long* status, cudaStream_t s, int64_t grid_rows = -1,  // grid_rows: bound on the row count
-                   int fb_stat = -1);  // status slot counting the rows passed on (-1: by the row set)
+                   int fb_stat = -1,  // status slot counting the rows passed on (-1: by the row set)
+                   const RefineFloors& fl = RefineFloors{});
 size_t tc_smem_bytes();
 bool tc_pairs();      // main similarity pass on CTA pairs (cta_group::2)
 int tc_item_rows();   // A rows per work item of the main pass: 256 on pairs, else 128
+int tc_max_item_tiles();  // most column tiles of an item of the paired kernels
 int tc_kmax();
 // Candidate lists per row and column chunk written by the tensor-core kernels
 // (their epilogue warp groups) for K depth dp and `segs` products per k-block.
@@ -399,7 +454,8 @@ int choose_chunks(int64_t row_blocks, int64_t col_tiles, int sm_count, int force
 size_t carve(Carver& c, const Shape& sh, Buffers& b, int sm_count, int precision);
 rerank_status plan_shape(const rerank_ctx* ctx, int64_t nq, int64_t ng, int d, int dtype, int k1, int k2,
                          int layers, int64_t topk, bool knn_only, bool host_in, bool host_out, int64_t cap_hint,
-                         Shape* out, const Tuning* tune = nullptr);  // tune: override of the table lookup
+                         Shape* out, const Tuning* tune = nullptr,  // tune: override of the table lookup
+                         bool append = true);  // append: the similarity stage may take the append pass
 // copy_overlap: host outputs are copied back in parts while later queries are
 // ranked (single calls only; batched instances copy on their own stream).
 // phases: which parts to enqueue (status reset, copies in and normalisation /

@@ -26,6 +26,7 @@
 
 #include "common.cuh"
 #include "internal.hpp"
+#include "topk_heap.cuh"  // score_key / key_score
 
 namespace rr {
 namespace {
@@ -381,12 +382,26 @@ __device__ __forceinline__ double row_eps_g(const ErrModel& em, int64_t i) {
   return eps_g;
 }
 
+// Whether the row's approximate scores say that its list cannot be certified
+// (the certificate compares the k1-th exact score with B + eps_g, and an exact
+// score is far closer to its approximation than the bound eps_g).  Passing such a row
+// on is always allowed; rescoring it first would be wasted.
+__device__ __forceinline__ bool hopeless(const WarpSmem& w, int k1, float B, double eps_g) {
+  return B > -FLT_MAX && double(w.g[k1 - 1]) < double(B) + 0.9 * eps_g;
+}
+
+// Starting floor of a row passed on: about K columns reach it in the next
+// stage's scores, whose distance from this stage's is a small part of eps_g.
+__device__ __forceinline__ int next_floor(const WarpSmem& w, int cnt, int K, double eps_g) {
+  return cnt >= K ? score_key(float(double(w.g[K - 1]) - 0.125 * eps_g)) : int(0x01010101u * kFloorResetByte);
+}
+
 template <int RV>
 __global__ void __launch_bounds__(WPB * kWarp)
 k2_refine(RowIo io, int64_t n, const float* __restrict__ part_s, const int32_t* __restrict__ part_i, int P,
           int K, int k1, ErrModel em, double eps_r, const int32_t* __restrict__ rows,
           const int32_t* __restrict__ count, bool part_by_row, int32_t* fb_rows, int32_t* fb_count,
-          int fb_stat) {
+          int fb_stat, RefineFloors fl) {
   __shared__ WarpSmem sm[WPB];
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t limit = (rows && count) ? int64_t(*count) : n;
@@ -403,13 +418,16 @@ k2_refine(RowIo io, int64_t n, const float* __restrict__ part_s, const int32_t* 
     // exact stage as one with no candidates.
     const bool aborted = (io.status[kStErr] & kErrTimeout) != 0;
     const int cnt = aborted ? 0 : merge_lists(w, part_s + base, part_i + base, P, K, n, lane, B);
+    if (cnt < K && fl.in) B = key_score(fl.in[part_by_row ? i : f]);
     if (cnt == n) B = -FLT_MAX;  // every column is a candidate
     // Fewer than k1 candidates (only after an aborted similarity stage): the
     // row goes to the next, exact stage like an uncertified one.
-    const bool ok = cnt >= k1 && refine_warp<RV>(w, cnt, i, k1, B, eps_g, eps_r, io, false, lane);
+    const bool ok = cnt >= k1 && !(fl.skip && hopeless(w, k1, B, eps_g)) &&
+                    refine_warp<RV>(w, cnt, i, k1, B, eps_g, eps_r, io, false, lane);
     if (!ok && lane == 0) {
       const int slot = atomicAdd(fb_count, 1);
       fb_rows[slot] = int32_t(i);
+      if (fl.next) fl.next[slot] = next_floor(w, cnt, fl.next_K, eps_g);
       atomicAdd(reinterpret_cast<unsigned long long*>(io.status + fb_stat), 1ull);
     }
     __syncwarp();
@@ -523,7 +541,7 @@ __global__ void __launch_bounds__(NW * kWarp, 48 / NW)
 k2_refine_cta(RowIo io, int64_t n, const float* __restrict__ part_s, const int32_t* __restrict__ part_i, int P,
               int Kmax, int k1, ErrModel em, double eps_r, const int32_t* __restrict__ rows,
               const int32_t* __restrict__ count, bool part_by_row, int32_t* fb_rows, int32_t* fb_count,
-              int fb_stat) {
+              int fb_stat, RefineFloors fl) {
   extern __shared__ float4 own[];  // dp / 4 float4: row i
   __shared__ WarpSmem w;
   __shared__ MergeSmem msm;
@@ -546,6 +564,7 @@ k2_refine_cta(RowIo io, int64_t n, const float* __restrict__ part_s, const int32
       } else if (!aborted && wid == 0) {
         cnt = merge_lists(w, part_s + base, part_i + base, P, Kmax, n, lane, B);
       }
+      if (cnt < Kmax && fl.in) B = key_score(fl.in[part_by_row ? i : f]);
       if (cnt == n) B = -FLT_MAX;  // every column is a candidate
       if (t == 0) {
         sh[0] = cnt;
@@ -554,7 +573,7 @@ k2_refine_cta(RowIo io, int64_t n, const float* __restrict__ part_s, const int32
     }
     __syncthreads();
     const int Kc = sh[0];
-    bool ok = Kc >= k1;
+    bool ok = Kc >= k1 && !(fl.skip && hopeless(w, k1, sB, eps_g));
     if (ok) {
       // FP32 scores of candidates [c0, c1) into w.s, two per warp at a time.
       auto rescore = [&](int c0, int c1) {
@@ -686,6 +705,7 @@ k2_refine_cta(RowIo io, int64_t n, const float* __restrict__ part_s, const int32
     if (!ok && t == 0) {
       const int slot = atomicAdd(fb_count, 1);
       fb_rows[slot] = int32_t(i);
+      if (fl.next) fl.next[slot] = next_floor(w, Kc, fl.next_K, eps_g);
       atomicAdd(reinterpret_cast<unsigned long long*>(io.status + fb_stat), 1ull);
     }
     __syncthreads();  // the shared row and lists are reused by the next row
@@ -798,7 +818,7 @@ int launch_refine(const Shape& sh, const void* xq, const void* xg, const float* 
                    const float* part_s, const int32_t* part_i, int P, const ErrModel& em, const int32_t* rows,
                    const int32_t* count, bool part_by_row, int32_t* knn_idx, float* knn_score,
                    int32_t* fb_rows, int32_t* fb_count,
-                   long long* status, cudaStream_t s, int64_t grid_rows, int fb_stat) {
+                   long long* status, cudaStream_t s, int64_t grid_rows, int fb_stat, const RefineFloors& fl) {
   RowIo io = make_io(sh, xq, xg, xhat, norm, knn_idx, knn_score, status);
   int64_t g = grid_rows > 0 && grid_rows < sh.n ? grid_rows : sh.n;
   // A gathered row set (size on the device): the kernels loop over it, so one
@@ -812,24 +832,24 @@ int launch_refine(const Shape& sh, const void* xq, const void* xg, const float* 
     if (refine_cta_warps(sh.dp) == 2)
       k2_refine_cta<2><<<unsigned(g), 2 * kWarp, smem, s>>>(io, sh.n, part_s, part_i, P, sh.K, sh.k1, em,
                                                              rescore_eps(sh.dp), rows, count, part_by_row, fb_rows,
-                                                             fb_count, stat);
+                                                             fb_count, stat, fl);
     else if (refine_cta_warps(sh.dp) == 8)
       k2_refine_cta<8><<<unsigned(g), 8 * kWarp, smem, s>>>(io, sh.n, part_s, part_i, P, sh.K, sh.k1, em,
                                                              rescore_eps(sh.dp), rows, count, part_by_row, fb_rows,
-                                                             fb_count, stat);
+                                                             fb_count, stat, fl);
     else
       k2_refine_cta<4><<<unsigned(g), 4 * kWarp, smem, s>>>(io, sh.n, part_s, part_i, P, sh.K, sh.k1, em,
                                                              rescore_eps(sh.dp), rows, count, part_by_row, fb_rows,
-                                                             fb_count, stat);
+                                                             fb_count, stat, fl);
     return 1;
   }
   // Row i in registers: 4 float4s per lane up to dp = 512, 16 up to 2048.
   if (sh.dp <= 512)
     k2_refine<4><<<blocks, WPB * kWarp, 0, s>>>(io, sh.n, part_s, part_i, P, sh.K, sh.k1, em, rescore_eps(sh.dp),
-                                                rows, count, part_by_row, fb_rows, fb_count, stat);
+                                                rows, count, part_by_row, fb_rows, fb_count, stat, fl);
   else
     k2_refine<16><<<blocks, WPB * kWarp, 0, s>>>(io, sh.n, part_s, part_i, P, sh.K, sh.k1, em, rescore_eps(sh.dp),
-                                                 rows, count, part_by_row, fb_rows, fb_count, stat);
+                                                 rows, count, part_by_row, fb_rows, fb_count, stat, fl);
   return 1;
 }
 

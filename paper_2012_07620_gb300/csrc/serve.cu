@@ -41,6 +41,7 @@
 
 #include "common.cuh"
 #include "internal.hpp"
+#include "topk_heap.cuh"  // score_key
 
 namespace rr {
 
@@ -82,7 +83,8 @@ struct Slot {
   float* emax_q = nullptr;  // 4: maxima over the queries
   int32_t* iota = nullptr;  // 0 .. S-1
   int32_t* scal = nullptr;  // [0] = Q, [1] = touched rows
-  float* pa_s = nullptr;    // S x Pa x K: query rows against X_u
+  TcAppend ap;              // query rows against X_u: append pass (when the server has it)
+  float* pa_s = nullptr;    // S x Pa x K: query rows against X_u (S x K with the append pass)
   int32_t* pa_i = nullptr;
   float* pb_s = nullptr;    // G x Pb x K: gallery rows against the queries
   int32_t* pb_i = nullptr;
@@ -140,6 +142,10 @@ struct Server {
   float* res_nbr_w = nullptr;
   int32_t* res_nbr_n = nullptr;
   std::vector<void*> res_extra;   // allocations of the above
+  int ap_chunks = 0, ap_cap = 0;  // query rows by the append pass: its chunks (0: the list kernels), segment capacity
+  int margin = -1;                // candidates beyond k1 (-1: cfg.rescore_m)
+  void* res_sample = nullptr;     // sampled gallery rows (low-precision copy) and their FP8 scales
+  float* res_sample_scale = nullptr;
   bool reuse = false;
   std::vector<Slot> slots;
   size_t resident_bytes = 0, slot_bytes = 0;
@@ -162,7 +168,7 @@ size_t slot_layout(const Server& v, Slot* sl, char* base, const Shape& shmax, in
   Carver c;
   c.base = base;
   const size_t rows = size_t(v.rowstride), dp = size_t(v.dp);
-  const int pa_max = 32, pb_max = int((v.S + 255) / 256) * tc_lists_per_chunk(v.dp, 1);
+  const int pa_max = v.ap_chunks ? 1 : 32, pb_max = int((v.S + 255) / 256) * tc_lists_per_chunk(v.dp, 1);
   Slot t;
   t.xhat = c.take<float>(rows * dp);
   t.xlow = c.take<char>(rows * dp * esize(v.prec));
@@ -178,6 +184,10 @@ size_t slot_layout(const Server& v, Slot* sl, char* base, const Shape& shmax, in
   t.scal = c.take<int32_t>(4);
   t.pa_s = c.take<float>(size_t(v.S) * pa_max * v.K);
   t.pa_i = c.take<int32_t>(size_t(v.S) * pa_max * v.K);
+  if (v.ap_chunks) {
+    t.ap.cand = c.take<int64_t>(size_t(v.S) * v.ap_chunks * 4 * v.ap_cap);
+    t.ap.seg_cnt = c.take<int32_t>(size_t(v.S) * v.ap_chunks * 4);
+  }
   t.pb_s = c.take<float>(size_t(v.G) * pb_max * v.K);
   t.pb_i = c.take<int32_t>(size_t(v.G) * pb_max * v.K);
   t.pm_s = c.take<float>(size_t(v.G) * v.K);
@@ -280,6 +290,24 @@ __global__ void k_serve_prep(const float* __restrict__ err_q, int64_t Q, float* 
   if (r == 0) scal[0] = int32_t(Q);
 }
 
+// Starting floors of the gallery rows against a request's queries: a query
+// column matters to row g only when its score reaches the K-th best of the
+// row's resident list (then it may be among the K best of the union) or can be
+// close enough to the k1-th neighbour to change the exact list (the test of
+// k_serve_assemble); nearly every list is then empty.
+__global__ void k_serve_floors(int64_t G, int64_t Q, int K, int k1, const float* __restrict__ res_s,
+                               const float* __restrict__ res_knn_score, const float* __restrict__ err_u,
+                               const float* __restrict__ emax_q, double eps_acc, double eps_r,
+                               int* __restrict__ floor_b) {
+  const int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (g >= G) return;
+  const double ei = err_u[Q + g], eq = emax_q[0];
+  const double eps_q = eps_acc + ei + eq + ei * eq;
+  const double sk = res_knn_score[size_t(g) * k1 + k1 - 1];
+  const float hit = nextafterf(float(sk - eps_r - eps_q), -INFINITY);
+  floor_b[g] = score_key(fminf(res_s[size_t(g) * K + K - 1], hit));
+}
+
 // One warp per gallery row: keep the resident exact list, or merge the
 // candidate lists of a row that a query may enter (see step 3 above).
 constexpr int AWPB = 8;
@@ -295,7 +323,8 @@ k_serve_assemble(int64_t G, int64_t Q, int K, int k1, int Pb, const float* __res
   const int64_t g = int64_t(blockIdx.x) * AWPB + wib;
   if (g >= G) return;
   const int64_t u = Q + g;  // the row's index in X_u
-  // Best approximate score of any query column (each list is sorted, best first).
+  // Best approximate score of any query column (each list is sorted, best
+  // first; with none listed, all lie below the row's floor, too low to matter).
   float bq = -FLT_MAX;
   for (int p = 0; p < Pb; ++p) {
     const size_t o = (size_t(g) * Pb + p) * K;
@@ -412,12 +441,14 @@ rerank_status enqueue_request(Server& v, Slot& sl, const rerank_request& rq, cud
   const int64_t topk = rq.topk_out ? rq.topk_out : G;
   const bool host_out = is_host_ptr(rq.out_idx) || is_host_ptr(rq.out_dist);
   Shape sh;
-  // The resident lists were made with the context's rescore_m: requests use it too.
+  // Requests use the resident lists' margin.
   Tuning tq = lookup_tuning(ctx, v.prec, G + Q, v.d);
-  tq.rescore_m = -1;
+  tq.rescore_m = v.margin;
   rerank_status st =
-      plan_shape(ctx, Q, G, v.d, v.dtype, v.k1, v.k2, v.layers, topk, false, false, host_out, 0, &sh, &tq);
+      plan_shape(ctx, Q, G, v.d, v.dtype, v.k1, v.k2, v.layers, topk, false, false, host_out, 0, &sh, &tq,
+                 false);
   if (st != RERANK_OK) return st;
+  sh.K = v.K;
   sh.ext_feat = true;
   sh.cap_h = v.cap_h;
   const bool fp8 = v.prec == RERANK_PREC_FP8;
@@ -463,36 +494,61 @@ rerank_status enqueue_request(Server& v, Slot& sl, const rerank_request& rq, cud
   em.eps = (v.dp / 16 + 32) * 2.0 * kU32 + 8.0 * kU32;
   // 2. query rows against X_u; gallery rows against the queries
   const int lpc = tc_lists_per_chunk(v.dp, 1);
-  const int pa = std::min(choose_chunks((Q + 127) / 128, sh.np / 256, sm, sh.tune.sim_chunks), 32 / lpc);
   const int pb = int((Q + 255) / 256);  // chunks; the lists per row are lpc times as many
   char* xl = static_cast<char*>(b.xlow);
-  if (launch_sim_tc_rect_topk(sh, xl, Q, 0, xl, n, 0, pa, fp8, b.xscale, sl.floor_a, sl.pa_s, sl.pa_i, status, sm,
-                              s) < 0)
-    return RERANK_ECUDA;
+  int pa = 0;  // lists per query row
+  RefineFloors fa;
+  if (v.ap_chunks) {
+    TcAppend ap = sl.ap;
+    ap.xsample = v.res_sample;
+    ap.sample_scale = v.res_sample_scale;
+    if (launch_sim_tc_rows_append(sh, xl, Q, v.ap_chunks, fp8, b.xscale, sl.floor_a, ap, v.ap_cap, sl.pa_s, sl.pa_i,
+                                  status, sm, s) < 0)
+      return RERANK_ECUDA;
+    pa = 1;
+    fa.in = sl.floor_a;
+  } else {
+    const int irows = tc_item_rows();
+    const int chunks = std::min(
+        choose_chunks((Q + irows - 1) / irows, sh.np / 256, sm * 128 / irows, sh.tune.sim_chunks), 32 / lpc);
+    if (launch_sim_tc_rect_topk(sh, xl, Q, 0, xl, n, 0, chunks, fp8, b.xscale, sl.floor_a, sl.pa_s, sl.pa_i, status,
+                                sm, s) < 0)
+      return RERANK_ECUDA;
+    pa = chunks * lpc;
+  }
+  const double eps_r = rescore_eps(v.dp);
+  k_serve_floors<<<unsigned((G + 255) / 256), 256, 0, s>>>(G, Q, v.K, v.k1, v.res_s, v.res_knn_score, b.err, sl.emax_q,
+                                                           em.eps, eps_r, sl.floor_b);
   if (launch_sim_tc_rect_topk(sh, xl + size_t(Q) * dp * es, G, Q, xl, Q, 0, pb, fp8, b.xscale, sl.floor_b, sl.pb_s,
-                              sl.pb_i, status, sm, s) < 0)
+                              sl.pb_i, status, sm, s, true) < 0)
     return RERANK_ECUDA;
   // 3. resident or re-derived gallery lists
-  const double eps_r = rescore_eps(v.dp);
   k_serve_assemble<<<unsigned((G + AWPB - 1) / AWPB), AWPB * kWarp, 0, s>>>(
       G, Q, v.K, v.k1, pb * lpc, v.res_s, v.res_i, v.res_knn_idx, v.res_knn_score, sl.pb_s, sl.pb_i, b.err, sl.emax_q,
       em.eps, eps_r, b.knn_idx, b.knn_score, sl.pm_s, sl.pm_i, sl.touched, sl.scal + 1, status);
   // 4. refinement of the query rows and of the touched gallery rows
   const void* dg = v.xg_raw;
-  launch_refine(sh, dq, dg, b.xhat, b.norm, sl.pa_s, sl.pa_i, pa * lpc, em, sl.iota, sl.scal, true, b.knn_idx,
-                b.knn_score, b.fb_rows, b.fb_count, status, s, Q);
+  fa.next = b.row_floor3;  // rows passed on start the recheck with floors from these lists
+  fa.next_K = v.K;
+  fa.skip = true;
+  launch_refine(sh, dq, dg, b.xhat, b.norm, sl.pa_s, sl.pa_i, pa, em, sl.iota, sl.scal, true, b.knn_idx,
+                b.knn_score, b.fb_rows, b.fb_count, status, s, Q, -1, fa);
+  RefineFloors ft = fa;
+  ft.in = nullptr;
   launch_refine(sh, dq, dg, b.xhat, b.norm, sl.pm_s, sl.pm_i, 1, em, sl.touched, sl.scal + 1, false, b.knn_idx,
-                b.knn_score, b.fb_rows, b.fb_count, status, s, G);
+                b.knn_score, b.fb_rows, b.fb_count, status, s, G, -1, ft);
   // recheck of uncertified rows with the hi/lo split, then the exact scan
   launch_gather_rows(b.fb_rows, b.fb_count, b.xhi, b.xlo, b.ahi, b.alo, n, v.dp, s);
   if (launch_sim_tc_split_topk(sh, sh.P3, b.ahi, b.alo, b.xhi, b.xlo, b.fb_rows, b.fb_count, b.row_floor3,
-                               b.part3_s, b.part3_i, status, sm, s) < 0)
+                               b.part3_s, b.part3_i, status, sm, s, true) < 0)
     return RERANK_ECUDA;
+  RefineFloors f3;
+  f3.in = b.row_floor3;
   ErrModel e3 = em;
   e3.kind = 2;
   e3.eps = (3 * (v.dp / 16) + 32) * 2.0 * kU32 + 8.0 * kU32;
   launch_refine(sh, dq, dg, b.xhat, b.norm, b.part3_s, b.part3_i, sh.P3, e3, b.fb_rows, b.fb_count, false, b.knn_idx,
-                b.knn_score, b.fb2_rows, b.fb2_count, status, s);
+                b.knn_score, b.fb2_rows, b.fb2_count, status, s, -1, -1, f3);
   float* fb_s = reinterpret_cast<float*>(b.scan_tmp);
   int32_t* fb_i = reinterpret_cast<int32_t*>(fb_s + size_t(sm) * fallback_warps() * fallback_k(sh));
   launch_refine_fallback(sh, dq, dg, b.xhat, b.norm, b.knn_idx, b.knn_score, b.fb2_rows, b.fb2_count, fb_s, fb_i,
@@ -782,8 +838,9 @@ rerank_status build_resident_graph(Server& v, cudaStream_t s0, long long* gst, s
   return RERANK_OK;
 }
 
+// narrow: plan with the context's rescore_m and the list kernels only (less memory).
 rerank_status serve_load(rerank_ctx* ctx, const void* xg, int64_t ng, int d, int dtype,
-                         const rerank_serve_config* sc) {
+                         const rerank_serve_config* sc, bool narrow = false) {
   const int prec = ctx->cfg.precision;
   if (prec == RERANK_PREC_FP32) return RERANK_EUNSUPPORTED;
   if (ctx->serve) return RERANK_EUNSUPPORTED;
@@ -807,10 +864,15 @@ rerank_status serve_load(rerank_ctx* ctx, const void* xg, int64_t ng, int d, int
   v->layers = layers;
   v->prec = prec;
   // 1. the gallery's own exact neighbour lists: the rerank_knn pipeline on G
+  // Full lists (as in rerank_run) where the budget allows: a request then
+  // rechecks hardly any row.
+  const bool want_full = !narrow && ctx->cfg.rescore_m >= 16;
+  v->margin = want_full ? tc_kmax() - k1 : -1;
   Shape shg;
   Tuning tg = lookup_tuning(ctx, prec, ng, d);
-  tg.rescore_m = -1;
-  st = plan_shape(ctx, ng, 0, d, dtype, k1, 1, 0, 0, true, false, false, 0, &shg, &tg);
+  tg.rescore_m = v->margin;
+  st = plan_shape(ctx, ng, 0, d, dtype, k1, 1, 0, 0, true, false, false, 0, &shg, &tg,
+                  false);  // lists of K entries, not bounded by a floor
   if (st != RERANK_OK) {
     delete v;
     return st;
@@ -819,17 +881,18 @@ rerank_status serve_load(rerank_ctx* ctx, const void* xg, int64_t ng, int d, int
   v->K = shg.K;
   Shape shmax;
   Tuning tm = lookup_tuning(ctx, prec, S + ng, d);
-  tm.rescore_m = -1;
-  st = plan_shape(ctx, S, ng, d, dtype, k1, k2, layers, ng, false, false, true, 0, &shmax, &tm);
+  tm.rescore_m = v->margin;
+  st = plan_shape(ctx, S, ng, d, dtype, k1, k2, layers, ng, false, false, true, 0, &shmax, &tm, false);
   if (st != RERANK_OK) {
     delete v;
     return st;
   }
-  if (shmax.K != v->K) {  // both are k1 + rescore_m once ng >= k1 + rescore_m
-    delete v;
-    return RERANK_EINTERNAL;
-  }
+  shmax.K = v->K;  // a request's lists are as long as the resident ones (at most ng places)
   shmax.ext_feat = true;
+  if (!narrow && ng >= 4096 && tc_append_ok((ng + 255) / 256 * 256, ctx->sm_count)) {
+    v->ap_chunks = int(std::min<int64_t>((ng + 255) / 256, tc_rows_append_segs() / 4));
+    v->ap_cap = tc_rows_append_cap(ng + S, v->K, v->ap_chunks);
+  }
   v->cap_h = shmax.cap_h;
   Buffers bg;
   Carver dry;
@@ -842,6 +905,9 @@ rerank_status serve_load(rerank_ctx* ctx, const void* xg, int64_t ng, int d, int
   rc.take<int32_t>(size_t(ng) * k1);
   rc.take<float>(size_t(ng) * k1);
   rc.take<float>(4);
+  const size_t sample_rows = v->ap_chunks ? size_t(tc_rows_append_sample()) : 0;
+  rc.take<char>(sample_rows * size_t(v->dp) * esize(prec));
+  rc.take<float>(sample_rows);
   v->resident_bytes = rc.used;
   v->slot_bytes = slot_layout(*v, nullptr, nullptr, shmax, ctx->sm_count);
   const size_t budget = ctx->cfg.hbm_budget;
@@ -851,7 +917,7 @@ rerank_status serve_load(rerank_ctx* ctx, const void* xg, int64_t ng, int d, int
     // The gallery's temporary workspace lives until the slots hold their copies.
     if (v->resident_bytes + gws + v->slot_bytes > budget) {
       delete v;
-      return RERANK_EBUDGET;
+      return narrow ? RERANK_EBUDGET : serve_load(ctx, xg, ng, d, dtype, sc, true);
     }
     nslots = int(std::min<size_t>(size_t(nslots), (budget - v->resident_bytes - gws) / v->slot_bytes));
   }
@@ -868,6 +934,8 @@ rerank_status serve_load(rerank_ctx* ctx, const void* xg, int64_t ng, int d, int
   v->res_knn_idx = rc.take<int32_t>(size_t(ng) * k1);
   v->res_knn_score = rc.take<float>(size_t(ng) * k1);
   v->res_emax = rc.take<float>(4);
+  v->res_sample = rc.take<char>(sample_rows * size_t(v->dp) * esize(prec));
+  v->res_sample_scale = rc.take<float>(sample_rows);
   auto fail = [&](rerank_status e) {
     free_server(v);
     return e;
@@ -903,6 +971,14 @@ rerank_status serve_load(rerank_ctx* ctx, const void* xg, int64_t ng, int d, int
     k_merge_parts<<<unsigned((ng + AWPB - 1) / AWPB), AWPB * kWarp, 0, s0>>>(ng, shg.P, v->K, j.b.part_s,
                                                                               j.b.part_i, v->res_s, v->res_i);
     cudaMemcpyAsync(v->res_emax, j.b.emax, 4 * sizeof(float), cudaMemcpyDeviceToDevice, s0);
+    if (v->ap_chunks) {
+      Shape ss = shg;
+      ss.sample = tc_rows_append_sample();
+      TcAppend sa;
+      sa.xsample = v->res_sample;
+      sa.sample_scale = v->res_sample_scale;
+      launch_sample_rows(ss, j.b.xlow, prec == RERANK_PREC_FP8, j.b.xscale, sa, s0);
+    }
     cudaMemcpyAsync(hst, gst, sizeof(hst), cudaMemcpyDeviceToHost, s0);
     if (cudaStreamSynchronize(s0) != cudaSuccess) {
       res = RERANK_ECUDA;
