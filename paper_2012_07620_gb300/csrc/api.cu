@@ -126,6 +126,7 @@ size_t carve(Carver& c, const Shape& sh, Buffers& b, int sm_count, int precision
     b.ap.cand = c.take<int64_t>(size_t(n) * sh.segs * sh.seg_cap);
     b.ap.seg_cnt = c.take<int32_t>(size_t(n) * sh.segs);
   }
+  if (sh.smat) b.smat = c.take<float>(size_t(np) * np);
   b.work = c.take<int32_t>(16);
   b.nb4 = c.take<int32_t>(4 * size_t(n));
   b.label = c.take<int32_t>(size_t(n));
@@ -300,7 +301,8 @@ rerank_status enqueue_job(rerank_ctx* ctx, const JobRun& j, cudaStream_t s, Stag
   }
   if (phases & kPhaseSim) {
     if (prec == RERANK_PREC_FP32) {
-      nl += launch_sim_fp32_topk(sh, b.xhat, b.row_floor, b.part_s, b.part_i, ctx->sm_count, s);
+      nl += sh.smat ? launch_sim_sym_topk(sh, b.xhat, b.smat, b.part_s, b.part_i, s)
+                    : launch_sim_fp32_topk(sh, b.xhat, b.row_floor, b.part_s, b.part_i, ctx->sm_count, s);
     } else {
       const int r = launch_sim_tc_topk(sh, b.xlow, prec == RERANK_PREC_FP8, b.xscale, b.row_floor, b.part_s,
                                        b.part_i, status, ctx->sm_count, s, b.work, b.ap);
@@ -325,7 +327,7 @@ rerank_status enqueue_job(rerank_ctx* ctx, const JobRun& j, cudaStream_t s, Stag
   }
   // Rows passed on start the recheck with floors from this stage's lists.
   RefineFloors fl;
-  fl.in = b.row_floor;
+  fl.in = sh.smat ? nullptr : b.row_floor;
   if (prec != RERANK_PREC_FP32) {
     fl.next = b.row_floor3;
     fl.next_K = prec == RERANK_PREC_FP8 ? sh.K3 : sh.K;
@@ -518,8 +520,8 @@ rerank_status run_once(rerank_ctx* ctx, const void* xq, const void* xg, int32_t*
   Carver dry;
   size_t need = carve(dry, j.sh, j.b, ctx->sm_count, ctx->cfg.precision);
   rerank_status st = ensure_workspace(ctx, need);
-  if ((st == RERANK_EBUDGET || st == RERANK_ENOMEM) && j.sh.segs > 0) {
-    // No room for the append pass's segments: the list kernels need less.
+  if ((st == RERANK_EBUDGET || st == RERANK_ENOMEM) && (j.sh.segs > 0 || j.sh.smat)) {
+    // No room for the append pass's segments (or the matrix): the list kernels need less.
     st = plan_lists(ctx, &j.sh);
     if (st != RERANK_OK) return st;
     ctx->shape = j.sh;
@@ -557,6 +559,11 @@ rerank_status run_once(rerank_ctx* ctx, const void* xq, const void* xg, int32_t*
   if (st == RERANK_ENOMEM) ctx->cap_h_hint = std::max<int64_t>(ctx->cap_h_hint, want + want / 4 + 1024);
   return st;
 }
+
+// Largest similarity matrix that the FP32 path keeps (n up to about 65,000): a
+// twentieth of the device's memory, with the rest left to the caller's data.
+// Beyond it the streaming kernel computes the whole square.
+constexpr size_t kSymBytes = size_t(16) << 30;
 
 // Shape of one instance.  cap_hint: a layer capacity learned from an earlier overflow.
 rerank_status plan_shape(const rerank_ctx* ctx, int64_t nq, int64_t ng, int d, int dtype, int k1, int k2, int layers,
@@ -609,6 +616,10 @@ rerank_status plan_shape(const rerank_ctx* ctx, int64_t nq, int64_t ng, int d, i
   sh.P = std::min(chunks, 32 / lpc) * lpc;
   if (may_append) {
     tc_append_plan(sh.n, sh.np, sh.dp, sh.K, chunks, &sh.segs, &sh.seg_cap, &sh.sample);
+    sh.P = 1;
+  }
+  if (!tc && append && size_t(sh.np) * sh.np * 4 <= kSymBytes) {
+    sh.smat = true;
     sh.P = 1;
   }
   // The recheck covers an unknown, usually small, set of rows: many short chunks keep every SM busy.
@@ -720,7 +731,7 @@ uint64_t buffer_id(const void* p) {
 // workspace offset they fix everything a batched call enqueues for it.
 void shape_key(const Shape& sh, std::vector<int64_t>& k) {
   const int64_t v[] = {sh.nq, sh.ng, sh.n, sh.np, sh.d, sh.dp, sh.dtype, sh.k1, sh.k2, sh.layers, sh.K, sh.P, sh.P3,
-                       sh.P3g, sh.K3, sh.segs, sh.seg_cap, sh.sample, sh.topk, sh.host_in, sh.host_out, sh.knn_only,
+                       sh.P3g, sh.K3, sh.segs, sh.seg_cap, sh.sample, sh.smat, sh.topk, sh.host_in, sh.host_out, sh.knn_only,
                        sh.ext_feat, sh.cap_h, sh.cap_csc, sh.hash_slots, sh.rank_ctas, sh.rank_scratch_per_cta, sh.tune.sim_chunks, sh.tune.prop_warps,
                        sh.tune.refine_order, sh.tune.rescore_m, sh.tune.rank_threads};
   k.insert(k.end(), std::begin(v), std::end(v));
@@ -814,7 +825,7 @@ rerank_status run_batch(rerank_ctx* ctx, rerank_job* jobs, int njobs, cudaStream
       st = plan_shape(ctx, jb.nq, jb.ng, jb.d, jb.dtype, jb.k1, jb.k2, jb.layers, topk, false, host_in, host_out, 0,
                       &run.sh, nullptr, attempt == 0);
       if (st != RERANK_OK) return st;
-      append = append || run.sh.segs > 0;
+      append = append || run.sh.segs > 0 || run.sh.smat;
       Carver dry;
       const size_t need = carve(dry, run.sh, run.b, ctx->sm_count, ctx->cfg.precision);
       total = (total + 255) & ~size_t(255);

@@ -85,6 +85,7 @@ struct Buffers {
   int32_t* fb3_count = nullptr;
   int* row_floor = nullptr;      // n, shared K-th best per row (similarity kernels)
   TcAppend ap;                   // append pass of the similarity stage
+  float* smat = nullptr;         // np x np: the FP32 similarity matrix (sh.smat)
   int32_t* nb4 = nullptr;        // 4n: best candidates per row (processing order)
   int32_t* label = nullptr;      // n
   int32_t* order = nullptr;      // n: rows grouped by cluster
@@ -144,6 +145,7 @@ struct Shape {
   int k1 = 0, k2 = 0, layers = 0, K = 0, P = 0;
   int P3 = 0;              // candidate lists per row of the hi/lo recheck
   int P3g = 0;             // FP8 path: lists per row of the single-product BF16 recheck stage
+  bool smat = false;       // FP32: the similarity matrix is kept (np x np floats) and half of it computed
   int segs = 0;            // append pass: segments per row (0: the list kernels)
   int seg_cap = 0;         // entries of a segment
   int sample = 0;          // columns sampled for its floors (0: none)
@@ -240,6 +242,8 @@ int launch_gather_rows(const int32_t* rows, const int32_t* count, const __nv_bfl
 // a row share their K-th best score.
 int launch_sim_fp32_topk(const Shape& sh, const float* xhat, int* row_floor, float* part_s, int32_t* part_i,
                          int sm_count, cudaStream_t s);
+// The same lists (one per row) by way of the whole matrix S (np x np), each pair computed once.
+int launch_sim_sym_topk(const Shape& sh, const float* xhat, float* S, float* part_s, int32_t* part_i, cudaStream_t s);
 // work (4 bytes, nullable): counter for the dynamic item order of the main pass.
 // With sh.segs > 0 the lists come from the append pass and its selection (one
 // list per row; `ap` holds its buffers), and a row's floor may lie above its

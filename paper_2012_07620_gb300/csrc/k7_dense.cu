@@ -17,6 +17,7 @@
 // (a TwoSum per chunk), so a score is as accurate as a chain of 32 products
 // (about 1e-7 for unit rows) whatever d is; the norms are applied in FP64.
 #include "common.cuh"
+#include "f32x2.cuh"
 #include "internal.hpp"
 
 namespace rr {
@@ -111,28 +112,31 @@ __global__ void k7_dense_inv_norms(const float* __restrict__ h, int64_t n, int d
   if (lane == 0) inv[i] = tot > 0.0 ? 1.0 / sqrt(tot) : 0.0;
 }
 
-// Float-float accumulation: (hi, lo) += p, with Knuth's TwoSum for the rounding error.
-__device__ __forceinline__ void ff_add(float& hi, float& lo, float p) {
-  const float s = hi + p;
-  const float bb = s - hi;
-  const float err = (hi - (s - bb)) + (p - bb);
+// Float-float accumulation of two outputs at once: (hi, lo) += p, with Knuth's
+// TwoSum for the rounding error.
+__device__ __forceinline__ void ff_add(f32x2& hi, f32x2& lo, f32x2 p) {
+  const f32x2 s = add2(hi, p);
+  const f32x2 bb = sub2(s, hi);
+  const f32x2 err = add2(sub2(hi, sub2(s, bb)), sub2(p, bb));
   hi = s;
-  lo += err;
+  lo = add2(lo, err);
 }
 
-// Scores by 128 x 128 output tiles, 256 threads of 8 x 8 outputs each (rows
-// 4 ty + a and 64 + 4 ty + a, columns 4 tx + b and 64 + 4 tx + b).  Each
-// 32-deep k-chunk is an FP32 FMA chain per output in k order and is added to
-// the output's (hi, lo) pair by TwoSum, so a score does not depend on the
-// tile shape or on which thread computes it; 8 x 8 outputs per thread keep
-// the shared-memory reads at a quarter of the FMAs' operands.  The chunk sums p and
-// hi live in registers, lo in shared memory (read and written once per
-// chunk).  The operand chunks are stored k-major (lane = row when loading, so
-// the transposing stores are free of bank conflicts); the next chunk's global
-// loads are issued before the current chunk is used.
+// Scores by 128 x 128 output tiles, 256 threads of 8 x 8 outputs each (the
+// lanes of a warp form a 4 x 8 grid: 32 rows by 64 columns, so that the operand
+// loads cost five shared-memory cycles per step).  Each 32-deep k-chunk is an
+// FP32 FMA chain per output in k order and is added to the output's (hi, lo)
+// pair by TwoSum, so a score does not depend on the tile shape or on which
+// thread computes it.  All of it runs on column pairs (packed FP32: the same
+// values, half the instructions).  The chunk sums p and hi live in registers, lo
+// in shared memory (read and written once per chunk).  The operand chunks are
+// stored k-major (lane = row when loading, so the transposing stores are free of
+// bank conflicts); the next chunk's global loads are issued before the current
+// chunk is used.  Bound by the FMA pipe (32 FMAs and 7 additions per output and
+// chunk): DENSE_NOTE.
 constexpr int ST = 128;                 // output tile
 constexpr int STHREADS = 256;
-constexpr size_t SSMEM = size_t(2) * DK * ST * 4 + size_t(64) * STHREADS * 4;  // As, Bs, lo
+constexpr size_t SSMEM = size_t(2) * DK * ST * 4 + size_t(32) * STHREADS * 8;  // As, Bs, lo
 
 __global__ void __launch_bounds__(STHREADS, 1)
 k7_dense_scores(const float* __restrict__ h, int64_t nq, int64_t ng, int dp, const double* __restrict__ inv,
@@ -140,15 +144,16 @@ k7_dense_scores(const float* __restrict__ h, int64_t nq, int64_t ng, int dp, con
   extern __shared__ float4 dyn4[];
   float* As = reinterpret_cast<float*>(dyn4);  // [DK][ST]
   float* Bs = As + DK * ST;                    // [DK][ST]
-  float* lo = Bs + DK * ST;                    // [64][STHREADS]
+  f32x2* lo = reinterpret_cast<f32x2*>(Bs + DK * ST);  // [32][STHREADS]
   const int t = threadIdx.x, lane = t & 31, wq = t >> 5;
-  const int tx = t & 15, ty = t >> 4;
+  const int tr = (wq >> 1) * 32 + (lane >> 3) * 4;  // rows tr + i and tr + 16 + i, i < 4
+  const int tc = (wq & 1) * 64 + (lane & 7) * 4;    // columns tc + j and tc + 32 + j, j < 4
   const int64_t q0 = int64_t(blockIdx.y) * ST, g0 = int64_t(blockIdx.x) * ST;
-  float hi[64], p[64];
+  f32x2 hi[32], p[32];
 #pragma unroll
-  for (int j = 0; j < 64; ++j) {
-    hi[j] = 0.f;
-    lo[j * STHREADS + t] = 0.f;
+  for (int j = 0; j < 32; ++j) {
+    hi[j] = 0ull;
+    lo[j * STHREADS + t] = 0ull;
   }
   // Loader: warp wq moves k-group wq (4 consecutive k of the chunk) of rows
   // lane + 32 s, s = 0..3, for both operands.
@@ -194,36 +199,39 @@ k7_dense_scores(const float* __restrict__ h, int64_t nq, int64_t ng, int dp, con
       }
     }
 #pragma unroll
-    for (int j = 0; j < 64; ++j) p[j] = 0.f;
-#pragma unroll 4
+    for (int j = 0; j < 32; ++j) p[j] = 0ull;
+#pragma unroll 8
     for (int k = 0; k < DK; ++k) {
-      const float4 x0 = reinterpret_cast<const float4*>(As + k * ST)[ty];
-      const float4 x1 = reinterpret_cast<const float4*>(As + k * ST)[16 + ty];
-      const float4 y0 = reinterpret_cast<const float4*>(Bs + k * ST)[tx];
-      const float4 y1 = reinterpret_cast<const float4*>(Bs + k * ST)[16 + tx];
+      const float4 x0 = *reinterpret_cast<const float4*>(As + k * ST + tr);
+      const float4 x1 = *reinterpret_cast<const float4*>(As + k * ST + tr + 16);
+      const ulonglong2 y0 = *reinterpret_cast<const ulonglong2*>(Bs + k * ST + tc);
+      const ulonglong2 y1 = *reinterpret_cast<const ulonglong2*>(Bs + k * ST + tc + 32);
       const float xa[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-      const float yb[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
+      const f32x2 yb[4] = {y0.x, y0.y, y1.x, y1.y};
 #pragma unroll
-      for (int a = 0; a < 8; ++a)
+      for (int a = 0; a < 8; ++a) {
+        const f32x2 a2 = twice(xa[a]);
 #pragma unroll
-        for (int b = 0; b < 8; ++b) p[a * 8 + b] = fmaf(xa[a], yb[b], p[a * 8 + b]);
+        for (int b = 0; b < 4; ++b) p[a * 4 + b] = fma2(a2, yb[b], p[a * 4 + b]);
+      }
     }
 #pragma unroll
-    for (int j = 0; j < 64; ++j) {
-      float l = lo[j * STHREADS + t];
+    for (int j = 0; j < 32; ++j) {
+      f32x2 l = lo[j * STHREADS + t];
       ff_add(hi[j], l, p[j]);
       lo[j * STHREADS + t] = l;
     }
   }
 #pragma unroll
   for (int a = 0; a < 8; ++a) {
-    const int64_t q = q0 + (a < 4 ? 4 * ty + a : 64 + 4 * ty + (a - 4));
+    const int64_t q = q0 + tr + (a < 4 ? a : 12 + a);
     if (q >= nq) continue;
 #pragma unroll
     for (int b = 0; b < 8; ++b) {
-      const int64_t g = g0 + (b < 4 ? 4 * tx + b : 64 + 4 * tx + (b - 4));
+      const int64_t g = g0 + tc + (b < 4 ? b : 28 + b);
       if (g >= ng) continue;
-      const double dot = double(hi[a * 8 + b]) + double(lo[(a * 8 + b) * STHREADS + t]);
+      const f32x2 hv = hi[a * 4 + b / 2], lv = lo[(a * 4 + b / 2) * STHREADS + t];
+      const double dot = (b & 1) ? double(hi_of(hv)) + double(hi_of(lv)) : double(lo_of(hv)) + double(lo_of(lv));
       S[q * ng + g] = float(dot * inv[q] * inv[nq + g]);
     }
   }
