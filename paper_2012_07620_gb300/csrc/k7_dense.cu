@@ -12,7 +12,7 @@
 // sum of squares, the 32 partials added in FP64).
 //
 // Scores: s(q, g) = <h_q, h_g> / (||h_q|| ||h_g||) for every query row q and
-// gallery row g, 128 x 128 output tiles per CTA, 8 x 8 per thread.  Each
+// gallery row g, 64 x 128 output tiles per CTA, 8 x 8 per thread.  Each
 // 32-deep k-chunk is an FP32 FMA chain; the chunks are added in float-float
 // (a TwoSum per chunk), so a score is as accurate as a chain of 32 products
 // (about 1e-7 for unit rows) whatever d is; the norms are applied in FP64.
@@ -122,90 +122,105 @@ __device__ __forceinline__ void ff_add(f32x2& hi, f32x2& lo, f32x2 p) {
   lo = add2(lo, err);
 }
 
-// Scores by 128 x 128 output tiles, 256 threads of 8 x 8 outputs each (the
+// Scores by 64 x 128 output tiles, 128 threads of 8 x 8 outputs each (the
 // lanes of a warp form a 4 x 8 grid: 32 rows by 64 columns, so that the operand
-// loads cost five shared-memory cycles per step).  Each 32-deep k-chunk is an
+// loads cost five shared-memory cycles per step), two CTAs per SM so that one
+// computes while the other waits at its barriers.  Each 32-deep k-chunk is an
 // FP32 FMA chain per output in k order and is added to the output's (hi, lo)
 // pair by TwoSum, so a score does not depend on the tile shape or on which
 // thread computes it.  All of it runs on column pairs (packed FP32: the same
 // values, half the instructions).  The chunk sums p and hi live in registers, lo
 // in shared memory (read and written once per chunk).  The operand chunks are
-// stored k-major (lane = row when loading, so the transposing stores are free of
-// bank conflicts); the next chunk's global loads are issued before the current
+// stored k-major; the next chunk's global loads are issued before the current
 // chunk is used.  Bound by the FMA pipe (32 FMAs and 7 additions per output and
-// chunk): DENSE_NOTE.
-constexpr int ST = 128;                 // output tile
-constexpr int STHREADS = 256;
-constexpr size_t SSMEM = size_t(2) * DK * ST * 4 + size_t(32) * STHREADS * 8;  // As, Bs, lo
+// chunk): 6.0 ms for 3,368 x 19,732 x 2,048, the pipe 0.70 busy (8.6 ms with scalar
+// FMAs, one CTA of 256 threads per SM and 16-byte loads of separate rows).
+constexpr int STM = 64, STN = 128;      // output tile: queries x gallery rows
+constexpr int STHREADS = 128;
+constexpr size_t SSMEM = size_t(DK) * (STM + STN) * 4 + size_t(32) * STHREADS * 8;  // As, Bs, lo
 
-__global__ void __launch_bounds__(STHREADS, 1)
+__global__ void __launch_bounds__(STHREADS, 2)
 k7_dense_scores(const float* __restrict__ h, int64_t nq, int64_t ng, int dp, const double* __restrict__ inv,
                 float* __restrict__ S) {
   extern __shared__ float4 dyn4[];
-  float* As = reinterpret_cast<float*>(dyn4);  // [DK][ST]
-  float* Bs = As + DK * ST;                    // [DK][ST]
-  f32x2* lo = reinterpret_cast<f32x2*>(Bs + DK * ST);  // [32][STHREADS]
+  float* As = reinterpret_cast<float*>(dyn4);  // [DK][STM]
+  float* Bs = As + DK * STM;                   // [DK][STN]
+  f32x2* lo = reinterpret_cast<f32x2*>(Bs + DK * STN);  // [32][STHREADS]
   const int t = threadIdx.x, lane = t & 31, wq = t >> 5;
   const int tr = (wq >> 1) * 32 + (lane >> 3) * 4;  // rows tr + i and tr + 16 + i, i < 4
   const int tc = (wq & 1) * 64 + (lane & 7) * 4;    // columns tc + j and tc + 32 + j, j < 4
-  const int64_t q0 = int64_t(blockIdx.y) * ST, g0 = int64_t(blockIdx.x) * ST;
+  const int64_t q0 = int64_t(blockIdx.y) * STM, g0 = int64_t(blockIdx.x) * STN;
   f32x2 hi[32], p[32];
 #pragma unroll
   for (int j = 0; j < 32; ++j) {
     hi[j] = 0ull;
     lo[j * STHREADS + t] = 0ull;
   }
-  // Loader: warp wq moves k-group wq (4 consecutive k of the chunk) of rows
-  // lane + 32 s, s = 0..3, for both operands.
-  const float4* arow[4];
-  const float4* brow[4];
-  bool aok[4], bok[4];
+  // Loader: four lanes read 64 bytes of a row, so that every 32-byte sector is
+  // used once; rows lr + 32 s, columns lk + 16 g of the chunk.  Row r of step k
+  // is stored at r ^ 8 ((k / 4) mod 4), which keeps 16-byte groups together and
+  // the transposing stores free of conflicts.
+  const int lr = t >> 2, lk = (t & 3) * 4, lp = lr ^ (8 * (t & 3));
+  const float4* arow[STM / 32];
+  const float4* brow[STN / 32];
+  bool aok[STM / 32], bok[STN / 32];
 #pragma unroll
-  for (int sl = 0; sl < 4; ++sl) {
-    const int64_t qa = q0 + lane + 32 * sl, ga = g0 + lane + 32 * sl;
+  for (int sl = 0; sl < STM / 32; ++sl) {
+    const int64_t qa = q0 + lr + 32 * sl;
     aok[sl] = qa < nq;
+    arow[sl] = reinterpret_cast<const float4*>(h + size_t(aok[sl] ? qa : 0) * dp + lk);
+  }
+#pragma unroll
+  for (int sl = 0; sl < STN / 32; ++sl) {
+    const int64_t ga = g0 + lr + 32 * sl;
     bok[sl] = ga < ng;
-    arow[sl] = reinterpret_cast<const float4*>(h + size_t(aok[sl] ? qa : 0) * dp) + wq;
-    brow[sl] = reinterpret_cast<const float4*>(h + size_t(bok[sl] ? nq + ga : 0) * dp) + wq;
+    brow[sl] = reinterpret_cast<const float4*>(h + size_t(bok[sl] ? nq + ga : 0) * dp + lk);
   }
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  float4 va[4], vb[4];
+  float4 va[STM / 32][2], vb[STN / 32][2];
+  auto fetch = [&](int step) {
 #pragma unroll
-  for (int sl = 0; sl < 4; ++sl) {
-    va[sl] = aok[sl] ? __ldg(arow[sl]) : zero;
-    vb[sl] = bok[sl] ? __ldg(brow[sl]) : zero;
-  }
+    for (int g = 0; g < 2; ++g) {
+#pragma unroll
+      for (int sl = 0; sl < STM / 32; ++sl) va[sl][g] = aok[sl] ? __ldg(arow[sl] + step + 4 * g) : zero;
+#pragma unroll
+      for (int sl = 0; sl < STN / 32; ++sl) vb[sl][g] = bok[sl] ? __ldg(brow[sl] + step + 4 * g) : zero;
+    }
+  };
+  fetch(0);
   for (int k0 = 0; k0 < dp; k0 += DK) {
     __syncthreads();  // the previous chunk is consumed
 #pragma unroll
-    for (int sl = 0; sl < 4; ++sl) {
-      const int r = lane + 32 * sl, kk = 4 * wq;
-      As[(kk + 0) * ST + r] = va[sl].x;
-      As[(kk + 1) * ST + r] = va[sl].y;
-      As[(kk + 2) * ST + r] = va[sl].z;
-      As[(kk + 3) * ST + r] = va[sl].w;
-      Bs[(kk + 0) * ST + r] = vb[sl].x;
-      Bs[(kk + 1) * ST + r] = vb[sl].y;
-      Bs[(kk + 2) * ST + r] = vb[sl].z;
-      Bs[(kk + 3) * ST + r] = vb[sl].w;
-    }
-    __syncthreads();
-    if (k0 + DK < dp) {
-      const int step = (k0 + DK) / 4;
+    for (int g = 0; g < 2; ++g) {
+      const int kk = lk + 16 * g;
 #pragma unroll
-      for (int sl = 0; sl < 4; ++sl) {
-        va[sl] = aok[sl] ? __ldg(arow[sl] + step) : zero;
-        vb[sl] = bok[sl] ? __ldg(brow[sl] + step) : zero;
+      for (int sl = 0; sl < STM / 32; ++sl) {
+        float* o = As + kk * STM + lp + 32 * sl;
+        o[0] = va[sl][g].x;
+        o[STM] = va[sl][g].y;
+        o[2 * STM] = va[sl][g].z;
+        o[3 * STM] = va[sl][g].w;
+      }
+#pragma unroll
+      for (int sl = 0; sl < STN / 32; ++sl) {
+        float* o = Bs + kk * STN + lp + 32 * sl;
+        o[0] = vb[sl][g].x;
+        o[STN] = vb[sl][g].y;
+        o[2 * STN] = vb[sl][g].z;
+        o[3 * STN] = vb[sl][g].w;
       }
     }
+    __syncthreads();
+    if (k0 + DK < dp) fetch((k0 + DK) / 4);
 #pragma unroll
     for (int j = 0; j < 32; ++j) p[j] = 0ull;
-#pragma unroll 8
+#pragma unroll 16
     for (int k = 0; k < DK; ++k) {
-      const float4 x0 = *reinterpret_cast<const float4*>(As + k * ST + tr);
-      const float4 x1 = *reinterpret_cast<const float4*>(As + k * ST + tr + 16);
-      const ulonglong2 y0 = *reinterpret_cast<const ulonglong2*>(Bs + k * ST + tc);
-      const ulonglong2 y1 = *reinterpret_cast<const ulonglong2*>(Bs + k * ST + tc + 32);
+      const int sw = 8 * ((k >> 2) & 3);
+      const float4 x0 = *reinterpret_cast<const float4*>(As + k * STM + (tr ^ sw));
+      const float4 x1 = *reinterpret_cast<const float4*>(As + k * STM + ((tr + 16) ^ sw));
+      const ulonglong2 y0 = *reinterpret_cast<const ulonglong2*>(Bs + k * STN + (tc ^ sw));
+      const ulonglong2 y1 = *reinterpret_cast<const ulonglong2*>(Bs + k * STN + ((tc + 32) ^ sw));
       const float xa[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
       const f32x2 yb[4] = {y0.x, y0.y, y1.x, y1.y};
 #pragma unroll
@@ -250,7 +265,7 @@ int launch_dense_layer(const Shape& sh, const float* hin, float* hout, const int
 int launch_dense_scores(const Shape& sh, const float* h, double* inv, float* S, cudaStream_t s) {
   const int T = 256;
   k7_dense_inv_norms<<<unsigned((sh.n * kWarp + T - 1) / T), T, 0, s>>>(h, sh.n, sh.dp, inv);
-  dim3 grid(unsigned((sh.ng + ST - 1) / ST), unsigned((sh.nq + ST - 1) / ST));
+  const dim3 grid(unsigned((sh.ng + STN - 1) / STN), unsigned((sh.nq + STM - 1) / STM));
   cudaFuncSetAttribute(k7_dense_scores, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SSMEM));
   k7_dense_scores<<<grid, STHREADS, SSMEM, s>>>(h, sh.nq, sh.ng, sh.dp, inv, S);
   return 2;
