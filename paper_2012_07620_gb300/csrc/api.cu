@@ -169,9 +169,9 @@ size_t carve(Carver& c, const Shape& sh, Buffers& b, int sm_count, int precision
   b.rnorm = c.take<float>(size_t(n));
   b.colcnt = c.take<int32_t>(size_t(n) + 1);
   b.colptr = c.take<int64_t>(size_t(n) + 1);
-  b.csc_row = c.take<int32_t>(size_t(sh.cap_h));
-  b.csc_val = c.take<float>(size_t(sh.cap_h));
+  b.csc = c.take<int2>(size_t(sh.cap_h));
   b.rank_scratch = c.take<uint32_t>(size_t(sh.rank_ctas) * size_t(rank_scratch_words(sh.ng)));
+  b.rank_over = c.take<int32_t>(4 + size_t(sh.nq));
   if (sh.dense) {
     b.hd[0] = c.take<float>(size_t(np) * sh.dp);
     b.hd[1] = c.take<float>(size_t(np) * sh.dp);

@@ -127,9 +127,9 @@ struct Buffers {
   // K5 / K6
   int32_t* colcnt = nullptr;     // n
   int64_t* colptr = nullptr;     // n + 1
-  int32_t* csc_row = nullptr;
-  float* csc_val = nullptr;
+  int2* csc = nullptr;           // (gallery row, value bits) by column
   uint32_t* rank_scratch = nullptr;
+  int32_t* rank_over = nullptr;  // 4 + nq: queries the light ranking kernel hands on, counted in [0]
   int32_t* work = nullptr;       // 16: item counter of the similarity kernel
   // dense features (RERANK_FEAT_X)
   float* hd[2] = {nullptr, nullptr};  // np x dp each, alternating layers
@@ -413,8 +413,7 @@ int launch_rank(const Shape& sh, const Buffers& b, int src, int32_t* out_idx, fl
 // request's own lists).
 struct RankReuse {
   const int64_t* colptr = nullptr;
-  const int32_t* row = nullptr;
-  const float* val = nullptr;
+  const int2* csc = nullptr;  // (gallery row, value bits)
   const uint8_t* changed = nullptr;
   int64_t shift = 0;
 };

@@ -50,7 +50,7 @@ __global__ void k5_count(const int64_t* __restrict__ start, const int32_t* __res
 __global__ void k5_fill(const int64_t* __restrict__ start, const int32_t* __restrict__ len,
                         const int32_t* __restrict__ col, const float* __restrict__ val, const float* __restrict__ rn,
                         int64_t nq, int64_t n, const int64_t* __restrict__ colptr, int32_t* __restrict__ fill,
-                        int32_t* __restrict__ csc_row, float* __restrict__ csc_val,
+                        int2* __restrict__ csc,
                         const long long* __restrict__ status, const uint8_t* __restrict__ sel) {
   const int64_t r = nq + ((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
@@ -61,13 +61,13 @@ __global__ void k5_fill(const int64_t* __restrict__ start, const int32_t* __rest
   for (int p = lane; p < m; p += kWarp) {
     const int c = col[a + p];
     const int64_t pos = colptr[c] + atomicAdd(&fill[c], 1);
-    csc_row[pos] = int32_t(r - nq);
-    csc_val[pos] = val[a + p] * s;
+    csc[pos] = make_int2(int(r - nq), __float_as_int(val[a + p] * s));
   }
 }
 
-// Exclusive block scan of one int per thread; returns the total.
-__device__ int block_exscan(int v, int* tmp, int& excl) {
+// Exclusive block scan of one int per thread (NW warps); returns the total.
+template <int NW>
+__device__ int block_exscan_t(int v, int* tmp, int& excl) {
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   int x = v;
 #pragma unroll
@@ -78,7 +78,7 @@ __device__ int block_exscan(int v, int* tmp, int& excl) {
   if (lane == 31) tmp[w] = x;
   __syncthreads();
   if (w == 0) {
-    int s = lane < RW ? tmp[lane] : 0;
+    int s = lane < NW ? tmp[lane] : 0;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(kFull, s, o);
@@ -88,10 +88,12 @@ __device__ int block_exscan(int v, int* tmp, int& excl) {
   }
   __syncthreads();
   excl = x - v + (w ? tmp[w - 1] : 0);
-  const int total = tmp[RW - 1];
+  const int total = tmp[NW - 1];
   __syncthreads();
   return total;
 }
+
+__device__ __forceinline__ int block_exscan(int v, int* tmp, int& excl) { return block_exscan_t<RW>(v, tmp, excl); }
 
 // Stable LSD radix sort of (key, val) ascending by key, four 8-bit passes.
 // Each warp owns a contiguous segment and counts its digits; the scatter
@@ -163,8 +165,7 @@ struct RankArgs {
   const float* val;
   const float* rn;
   const int64_t* colptr;
-  const int32_t* csc_row;
-  const float* csc_val;
+  const int2* csc;
   int64_t nq, ng, topk;
   int64_t q_begin, q_end;  // queries ranked by this launch
   int32_t* out_idx;
@@ -172,6 +173,11 @@ struct RankArgs {
   uint32_t* gscratch;   // per CTA (rank_scratch_words): acc (ng) [if !acc_smem] + 4 * ng sort buffers
   int acc_smem;
   RankReuse reuse;  // resident gallery lists (colptr null: none)
+  const int32_t* qlist;    // queries to rank (null: q_begin .. q_end - 1), their number at *qcount
+  const int32_t* qcount;
+  int32_t* over;           // light kernel: queries it hands on, counted at *over_count
+  int32_t* over_count;
+  int idx_smem;            // dense lists: 16-bit gallery indices in shared memory
   int sort_cap;    // most non-zeros the shared-memory sort takes (SORT_CAP unless a test lowers it)
   int bucket_cap;  // largest bucket it takes (BUCKET_CAP unless a test lowers it)
   long long* status;
@@ -193,12 +199,300 @@ __device__ __forceinline__ int score_bucket(uint32_t x) {
 
 __device__ __forceinline__ uint64_t rank_key(uint32_t x, uint32_t g) { return (uint64_t(~x) << 32) | g; }
 
+// One column's products by a warp: add(g, x) for each of its n entries (gallery
+// row, value), x the product with v in fixed point.  Whole rounds of 128
+// entries run without bounds checks.
+template <class Add>
+__device__ __forceinline__ void add_column(const int2* __restrict__ e, int n, float v, int lane, Add add) {
+  e += lane;
+  int k = 0;
+  for (; k + 4 * kWarp <= n; k += 4 * kWarp, e += 4 * kWarp) {
+    int2 x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = __ldg(e + u * kWarp);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) add(x[u].x, __float2uint_rn(v * __int_as_float(x[u].y)), true);
+  }
+  if (k < n) {
+    const int left = n - k - lane;  // entries at or after this lane's
+    int2 x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = left > u * kWarp ? __ldg(e + u * kWarp) : make_int2(0, 0);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (k + u * kWarp < n) add(x[u].x, __float2uint_rn(v * __int_as_float(x[u].y)), left > u * kWarp);
+  }
+}
+
+// Adds query q's products into the scores, one warp per entry of its row:
+// add(g, x, in) for every gallery row g of the entry's column (lanes past its end
+// call with in = false), x the product in fixed point (2^31 is exact, so it is
+// folded into the query's value).  Warp w of nw takes entries w, w + nw, ...; the
+// next entry's column bounds are loaded while the current column is added.
+// stop(): true ends the warp's work.
+template <class Add, class Stop>
+__device__ __forceinline__ void add_products(const RankArgs& A, int64_t q, int w, int nw, int lane, Add add,
+                                             Stop stop) {
+  const int64_t a = A.start[q];
+  const int m = A.len[q];
+  const float rq = A.rn[q];
+  const int32_t* __restrict__ col = A.col + a;
+  const float* __restrict__ val = A.val + a;
+  const int64_t* __restrict__ colptr = A.colptr;
+  const int2* __restrict__ csc = A.csc;
+  int e = w;
+  float v = 0.f;
+  int64_t p0 = 0;
+  int n = 0;
+  if (e < m) {
+    const int c = col[e];
+    v = val[e] * rq * kFix;
+    p0 = colptr[c];
+    n = int(colptr[c + 1] - p0);
+  }
+  while (e < m) {
+    const int en = e + nw;
+    float vn = 0.f;
+    int64_t n0 = 0;
+    int nn = 0;
+    if (en < m) {
+      const int cn = col[en];
+      vn = val[en] * rq * kFix;
+      n0 = colptr[cn];
+      nn = int(colptr[cn + 1] - n0);
+    }
+    add_column(csc + p0, n, v, lane, add);
+    if (stop()) return;
+    e = en;
+    v = vn;
+    p0 = n0;
+    n = nn;
+  }
+  if (A.reuse.colptr) {
+    // The same over the resident lists of the columns of gallery vertices,
+    // for the gallery rows the request left unchanged.
+    const RankReuse R = A.reuse;
+    for (e = w; e < m; e += nw) {
+      const int64_t c = col[e] - R.shift;
+      if (c < 0) continue;
+      const int64_t r0 = R.colptr[c];
+      add_column(R.csc + r0, int(R.colptr[c + 1] - r0), val[e] * rq * kFix, lane,
+                 [&](int g, uint32_t x, bool in) { add(g, x, in && !R.changed[g]); });
+      if (stop()) return;
+    }
+  }
+}
+
+// The zero tail of query q: places cnt .. T - 1 hold the gallery rows without a
+// score in index order, at distance 1.  Distances: block-wide stores, 16 bytes
+// each once aligned.  Indices: warp w writes the zeros of words [w0, w1) of the
+// non-zero bitmap (32 words at a time: a warp scan of their zero counts, then
+// one coalesced store per word); `before`: zeros before word w0.
+__device__ __forceinline__ void zero_tail(const RankArgs& A, int64_t q, int cnt, const uint32_t* bits, int w0, int w1,
+                                          int64_t before, int t, int nt, int lane) {
+  const int64_t T = A.topk;
+  if (T <= cnt) return;
+  const unsigned lt = (1u << lane) - 1u;
+  float* dq = A.out_dist + q * T;
+  const int64_t head = tmin<int64_t>((4 - int((reinterpret_cast<uintptr_t>(dq + cnt) >> 2) & 3)) & 3, T - cnt);
+  if (t < head) dq[cnt + t] = 1.0f;
+  const int64_t p0 = cnt + head, nv = (T - p0) >> 2;
+  float4* dv = reinterpret_cast<float4*>(dq + p0);
+  for (int64_t v = t; v < nv; v += nt) dv[v] = make_float4(1.f, 1.f, 1.f, 1.f);
+  for (int64_t p = p0 + 4 * nv + t; p < T; p += nt) dq[p] = 1.0f;
+  int32_t* iq = A.out_idx + q * T;
+  int64_t run = int64_t(cnt) + before;
+  for (int c0 = w0; c0 < w1 && run < T; c0 += kWarp) {
+    const int nw = min(kWarp, w1 - c0);
+    uint32_t zl = 0u;
+    if (lane < nw) {
+      const int wd = c0 + lane;
+      const int valid = int(tmin<int64_t>(32, A.ng - int64_t(wd) * 32));
+      const uint32_t vm = valid == 32 ? kFull : ((1u << valid) - 1u);
+      zl = ~bits[wd] & vm;
+    }
+    const int cz = __popc(zl);
+    int incl = cz;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += y;
+    }
+    const int64_t wbase = run + (incl - cz);
+    for (int j = 0; j < nw; ++j) {
+      const uint32_t zj = __shfl_sync(kFull, zl, j);
+      const int64_t bj = __shfl_sync(kFull, wbase, j);
+      if ((zj >> lane) & 1u) {
+        const int64_t p = bj + __popc(zj & lt);
+        if (p < T) iq[p] = int32_t(int64_t(c0 + j) * 32 + lane);
+      }
+    }
+    run += __shfl_sync(kFull, incl, 31);
+  }
+}
+
+// Ranking of queries with few non-zero scores (at most the list's capacity):
+// the gallery rows whose score becomes non-zero are listed as they appear (the
+// adding atomic returns the old score), and everything after works on that list
+// instead of on all scores: bucket counts, scatter, in-bucket places, and the
+// clean-up for the next query.  The keys are the listed 16-bit indices and the
+// scores themselves, so that a gallery of up to ~19,800 rows leaves room for two
+// CTAs per SM: one writes its zero tail (7,300 cycles of HBM at the Market
+// shape) while the other computes.  Queries with more non-zeros, or with a bucket
+// too crowded for counting, are handed to k6_rank through `over`.
+// RANK_LIGHT_NOTE
+constexpr int LB = 4096;            // score buckets, 16-bit counters in pairs
+// Bucket of a non-zero score, best first: 256 per octave down to 2^-12, 64 below.
+__device__ __forceinline__ int light_bucket(uint32_t x) {
+  const int lz = __clz(x);
+  const uint32_t below = (x << lz) << 1;  // the bits after the leading one, left-aligned
+  const int pos = 31 - lz;
+  const int f = pos >= 20 ? 1024 + ((pos - 20) << 8 | int(below >> 24)) : max(pos - 4, 0) << 6 | int(pos >= 4 ? below >> 26 : 0u);
+  return LB - 1 - f;
+}
+constexpr int LCAP = 6144;          // non-zero scores of a query
+struct LightSmem {                  // followed by bits[nwords], acc[ng]
+  uint32_t hist[LB / 2];
+  uint16_t list[LCAP];
+  uint16_t sorted[LCAP];
+  int tmp[32];
+  int cnt;
+  int big;
+};
+
+template <int NTH>
+__global__ void __launch_bounds__(NTH, 1024 / NTH) k6_rank_light(RankArgs A) {
+  extern __shared__ uint32_t sm[];
+  if (A.status[kStErr] & kErrOverflow) return;
+  LightSmem& S = *reinterpret_cast<LightSmem*>(sm);
+  constexpr int NW = NTH / kWarp;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  const int ng = int(A.ng);
+  const int nwords = (ng + 31) / 32;
+  uint32_t* const bits = sm + sizeof(LightSmem) / 4;
+  uint32_t* const acc = bits + nwords;
+  const int64_t T = A.topk;
+  for (int e = t; e < nwords + ng; e += NTH) bits[e] = 0u;
+  for (int e = t; e < LB / 2; e += NTH) S.hist[e] = 0u;
+  if (t == 0) {
+    S.cnt = 0;
+    S.big = 0;
+  }
+  __syncthreads();
+  auto place = [&](int b) { return int((S.hist[b >> 1] >> (16 * (b & 1))) & 0xffffu); };
+  for (int64_t q = A.q_begin + blockIdx.x; q < A.q_end; q += gridDim.x) {
+    volatile int* const vcnt = &S.cnt;
+    add_products(
+        A, q, w, NW, lane,
+        [&](int r, uint32_t x, bool in) {
+          const bool fresh = in && x != 0u && atomicAdd(&acc[r], x) == 0u;
+          const unsigned bal = __ballot_sync(kFull, fresh);
+          if (bal) {
+            int base = 0;
+            if (lane == 0) base = atomicAdd(&S.cnt, __popc(bal));
+            base = __shfl_sync(kFull, base, 0);
+            const int at = base + __popc(bal & lt);
+            if (fresh && at < LCAP) S.list[at] = uint16_t(r);
+          }
+        },
+        [&] { return *vcnt > LCAP; });  // handed on: what follows does not count
+    __syncthreads();
+    int cnt = S.cnt;
+    bool over = cnt > LCAP;
+    if (!over) {
+      for (int i = t; i < cnt; i += NTH) {
+        const int g = S.list[i];
+        const int b = light_bucket(acc[g]);
+        atomicAdd(&S.hist[b >> 1], 1u << (16 * (b & 1)));
+        atomicOr(&bits[g >> 5], 1u << (g & 31));
+      }
+      __syncthreads();
+      // Bucket starts (eight or four buckets per thread) and the largest bucket.
+      constexpr int PT = LB / 2 / NTH;  // words per thread
+      uint32_t h[PT];
+      int part = 0, big = 0;
+#pragma unroll
+      for (int k = 0; k < PT; ++k) {
+        h[k] = S.hist[t * PT + k];
+        const int a = int(h[k] & 0xffffu), b = int(h[k] >> 16);
+        part += a + b;
+        big = max(big, max(a, b));
+      }
+      big = __reduce_max_sync(kFull, big);
+      if (lane == 0 && big > A.bucket_cap) S.big = 1;
+      int base;
+      block_exscan_t<NW>(part, S.tmp, base);  // its barriers also publish S.big
+#pragma unroll
+      for (int k = 0; k < PT; ++k) {
+        const int a = int(h[k] & 0xffffu), b = int(h[k] >> 16);
+        S.hist[t * PT + k] = uint32_t(base) | (uint32_t(base + a) << 16);
+        base += a + b;
+      }
+      over = S.big != 0;
+      __syncthreads();
+    }
+    if (!over) {
+      for (int i = t; i < cnt; i += NTH) {
+        const int g = S.list[i];
+        const int b = light_bucket(acc[g]);
+        const uint32_t old = atomicAdd(&S.hist[b >> 1], 1u << (16 * (b & 1)));
+        S.sorted[(old >> (16 * (b & 1))) & 0xffffu] = uint16_t(g);
+      }
+      __syncthreads();  // place(b) is now the end of bucket b
+      for (int p = t; p < cnt; p += NTH) {
+        const int g = S.sorted[p];
+        const uint32_t x = acc[g];
+        const int b = light_bucket(x);
+        const int b0 = b ? place(b - 1) : 0, b1 = place(b);
+        if (b0 >= T) continue;
+        int r = b0;
+        for (int j = b0; j < b1; ++j) {
+          const int gj = S.sorted[j];
+          const uint32_t xj = acc[gj];
+          r += (xj > x || (xj == x && gj < g)) ? 1 : 0;
+        }
+        if (r < T) {
+          A.out_idx[q * T + r] = g;
+          A.out_dist[q * T + r] = 1.0f - __uint2float_rn(x) * kUnfix;
+        }
+      }
+      if (T > cnt) {
+        // Warp w owns words [w0, w1): the zeros before them from a scan of the warps' counts.
+        const int wpw = (nwords + NW - 1) / NW;
+        const int w0 = min(nwords, w * wpw), w1 = min(nwords, w0 + wpw);
+        int mine = 0;
+        for (int wd = w0 + lane; wd < w1; wd += kWarp) mine += __popc(bits[wd]);
+        mine = int(__reduce_add_sync(kFull, unsigned(mine)));
+        int off;
+        block_exscan_t<NW>(lane == 0 ? mine : 0, S.tmp, off);
+        off = __shfl_sync(kFull, off, 0);
+        zero_tail(A, q, cnt, bits, w0, w1, int64_t(w0) * 32 - off, t, NTH, lane);
+      }
+      __syncthreads();
+      for (int i = t; i < cnt; i += NTH) acc[S.list[i]] = 0u;
+    } else {
+      if (t == 0) A.over[atomicAdd(A.over_count, 1)] = int32_t(q);
+      __syncthreads();
+      for (int e = t; e < ng; e += NTH) acc[e] = 0u;
+    }
+    for (int e = t; e < nwords; e += NTH) bits[e] = 0u;
+    for (int e = t; e < LB / 2; e += NTH) S.hist[e] = 0u;
+    if (t == 0) {
+      S.cnt = 0;
+      S.big = 0;
+    }
+    __syncthreads();
+  }
+}
+
 // Global scratch per ranking CTA, in 32-bit words (even, so every CTA's part
 // is 8-byte aligned): the accumulator when shared memory cannot hold it, then
 // either two 64-bit key arrays (bucket sort beyond SORT_CAP keys) or four
 // 32-bit arrays (radix sort).
 __host__ __device__ inline int64_t scratch_words(int64_t ng) { return (5 * ng + 9) & ~int64_t(1); }
 
+template <bool ACC_SMEM>
 __global__ void __launch_bounds__(RT, 1) k6_rank(RankArgs A) {
   extern __shared__ uint32_t sm[];
   if (A.status[kStErr] & kErrOverflow) return;
@@ -214,7 +508,11 @@ __global__ void __launch_bounds__(RT, 1) k6_rank(RankArgs A) {
   uint32_t* region = reinterpret_cast<uint32_t*>(kb + SORT_CAP);  // acc (when acc_smem), later sorted keys
   uint64_t* ks = reinterpret_cast<uint64_t*>(region);   // SORT_CAP sorted keys (the accumulator is dead by then)
   uint32_t* gbase = A.gscratch + size_t(blockIdx.x) * size_t(scratch_words(ng));
-  uint32_t* acc = A.acc_smem ? region : gbase;
+  // (a compile-time choice: an accumulator of unknown kind costs generic atomics)
+  uint32_t* acc;
+  if constexpr (ACC_SMEM) acc = region;
+  else acc = gbase;
+  uint16_t* sidx = reinterpret_cast<uint16_t*>(region + ng);  // dense lists: sorted gallery indices (when idx_smem)
   uint32_t* gk0 = gbase + ng;
   uint32_t* gv0 = gk0 + ng;
   uint32_t* gk1 = gv0 + ng;
@@ -223,81 +521,19 @@ __global__ void __launch_bounds__(RT, 1) k6_rank(RankArgs A) {
   uint64_t* ksg = kbg + ng;                                                       // ng sorted keys
   const int64_t T = A.topk;
 
-  for (int64_t q = A.q_begin + blockIdx.x; q < A.q_end; q += gridDim.x) {
+  const int64_t nq = A.qlist ? int64_t(*A.qcount) : A.q_end - A.q_begin;
+  for (int64_t qi = blockIdx.x; qi < nq; qi += gridDim.x) {
+    const int64_t q = A.qlist ? int64_t(A.qlist[qi]) : A.q_begin + qi;
     for (int64_t g = t; g < ng; g += RT) acc[g] = 0u;
     for (int e = t; e < NB; e += RT) hist[e] = 0u;
     if (t == 0) misc[1] = 0;
     __syncthreads();
-    const int64_t a = A.start[q];
-    const int m = A.len[q];
-    const float rq = A.rn[q];
-    // Warp w takes entries w, w + RW, ...; the next entry's column bounds are
-    // loaded while the current column is added, four column steps per round.
-    {
-      int e = w;
-      float v = 0.f;
-      int64_t p0 = 0, p1 = 0;
-      if (e < m) {
-        const int c = A.col[a + e];
-        v = A.val[a + e] * rq;
-        p0 = A.colptr[c];
-        p1 = A.colptr[c + 1];
-      }
-      while (e < m) {
-        const int en = e + RW;
-        float vn = 0.f;
-        int64_t n0 = 0, n1 = 0;
-        if (en < m) {
-          const int cn = A.col[a + en];
-          vn = A.val[a + en] * rq;
-          n0 = A.colptr[cn];
-          n1 = A.colptr[cn + 1];
-        }
-        for (int64_t p = p0 + lane; p < p1; p += 4 * kWarp) {
-          int r[4];
-          float x[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int64_t pp = p + u * kWarp;
-            r[u] = pp < p1 ? A.csc_row[pp] : -1;
-            x[u] = pp < p1 ? A.csc_val[pp] : 0.f;
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const float prod = v * x[u];
-            if (r[u] >= 0) atomicAdd(&acc[r[u]], __float2uint_rn(prod * kFix));
-          }
-        }
-        e = en;
-        v = vn;
-        p0 = n0;
-        p1 = n1;
-      }
-    }
-    if (A.reuse.colptr) {
-      // The same over the resident lists of the columns of gallery vertices,
-      // for the gallery rows the request left unchanged.
-      const RankReuse& R = A.reuse;
-      for (int e = w; e < m; e += RW) {
-        const int64_t c = A.col[a + e] - R.shift;
-        if (c < 0) continue;
-        const float v = A.val[a + e] * rq;
-        const int64_t p1 = R.colptr[c + 1];
-        for (int64_t p = R.colptr[c] + lane; p < p1; p += 4 * kWarp) {
-          int r[4];
-          float x[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int64_t pp = p + u * kWarp;
-            r[u] = pp < p1 ? R.row[pp] : -1;
-            x[u] = pp < p1 ? R.val[pp] : 0.f;
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (r[u] >= 0 && !R.changed[r[u]]) atomicAdd(&acc[r[u]], __float2uint_rn(v * x[u] * kFix));
-        }
-      }
-    }
+    add_products(
+        A, q, w, RW, lane,
+        [&](int r, uint32_t x, bool in) {
+          if (in) atomicAdd(&acc[r], x);
+        },
+        [] { return false; });
     __syncthreads();
     // Non-zero bitmap, bucket histogram and count, warp-cooperative: warp w
     // owns words [w0, w1) (32 gallery entries each, lane = entry); the ballot
@@ -418,11 +654,31 @@ __global__ void __launch_bounds__(RT, 1) k6_rank(RankArgs A) {
             for (int u = 0; u < 4; ++u) {
               if ((bal[u] >> lane) & 1u) {
                 const uint32_t pos = atomicAdd(&h2[sub_bucket(x[u])], 1u);
-                kbg[pos] = rank_key(x[u], uint32_t(int64_t(wd + u) * 32 + lane));
+                const uint32_t g = uint32_t(int64_t(wd + u) * 32 + lane);
+                if (ACC_SMEM && A.idx_smem) sidx[pos] = uint16_t(g);
+                else kbg[pos] = rank_key(x[u], g);
               }
             }
           }
           __syncthreads();  // h2[i] is now the end of sub-bucket i
+          if (ACC_SMEM && A.idx_smem) {
+            // Keys in shared memory as 16-bit indices beside the scores (the keys in
+            // global scratch missed the small L1 left: 2.9 of 3.5 ms at market_hard).
+            for (int p = t; p < cnt; p += RT) {
+              const int g = sidx[p];
+              const uint32_t x = acc[g];
+              const int i2 = sub_bucket(x);
+              const int b0 = i2 ? int(h2[i2 - 1]) : 0, b1 = int(h2[i2]);
+              int pos = b0;
+              for (int j = b0; j < b1; ++j) {
+                const int gj = sidx[j];
+                const uint32_t xj = acc[gj];
+                pos += (xj > x || (xj == x && gj < g)) ? 1 : 0;
+              }
+              A.out_idx[q * T + pos] = g;
+              A.out_dist[q * T + pos] = 1.0f - __uint2float_rn(x) * kUnfix;
+            }
+          } else
           for (int64_t p = t; p < cnt; p += RT) {
             const uint64_t key = kbg[p];
             const uint32_t x = ~uint32_t(key >> 32);
@@ -559,51 +815,7 @@ __global__ void __launch_bounds__(RT, 1) k6_rank(RankArgs A) {
         }
       }
     }
-    // The zero tail in gallery order.  Its distances are all 1: plain
-    // block-wide stores, 16 bytes each once aligned.  Its indices: warp w
-    // writes the zeros of its words (a warp scan of 32 words' zero counts,
-    // then one coalesced store per word).
-    if (T > cnt) {
-      float* dq = A.out_dist + q * T;
-      const int64_t head = tmin<int64_t>((4 - int((reinterpret_cast<uintptr_t>(dq + cnt) >> 2) & 3)) & 3, T - cnt);
-      if (t < head) dq[cnt + t] = 1.0f;
-      const int64_t p0 = cnt + head, nv = (T - p0) >> 2;
-      float4* dv = reinterpret_cast<float4*>(dq + p0);
-      for (int64_t v = t; v < nv; v += RT) dv[v] = make_float4(1.f, 1.f, 1.f, 1.f);
-      for (int64_t p = p0 + 4 * nv + t; p < T; p += RT) dq[p] = 1.0f;
-      int32_t* iq = A.out_idx + q * T;
-      // The warp's words 32 at a time: lane l takes word c0 + l, its zeros and
-      // their count; a warp scan of the counts gives every word's first place,
-      // then the warp writes the words' indices one word at a time.
-      int64_t run = int64_t(cnt) + zeros_before;
-      for (int c0 = w0; c0 < w1 && run < T; c0 += kWarp) {
-        const int nw = min(kWarp, w1 - c0);
-        uint32_t zl = 0u;
-        if (lane < nw) {
-          const int wd = c0 + lane;
-          const int valid = int(tmin<int64_t>(32, ng - int64_t(wd) * 32));
-          const uint32_t vm = valid == 32 ? kFull : ((1u << valid) - 1u);
-          zl = ~bits[wd] & vm;
-        }
-        const int cz = __popc(zl);
-        int incl = cz;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(kFull, incl, o);
-          if (lane >= o) incl += y;
-        }
-        const int64_t wbase = run + (incl - cz);
-        for (int j = 0; j < nw; ++j) {
-          const uint32_t zj = __shfl_sync(kFull, zl, j);
-          const int64_t bj = __shfl_sync(kFull, wbase, j);
-          if ((zj >> lane) & 1u) {
-            const int64_t p = bj + __popc(zj & lt);
-            if (p < T) iq[p] = int32_t(int64_t(c0 + j) * 32 + lane);
-          }
-        }
-        run += __shfl_sync(kFull, incl, 31);
-      }
-    }
+    zero_tail(A, q, cnt, bits, w0, w1, zeros_before, t, RT, lane);
     __syncthreads();
   }
 }
@@ -774,6 +986,12 @@ void rank_caps(int* sort_cap, int* bucket_cap) {
 
 int64_t rank_scratch_words(int64_t ng) { return scratch_words(ng); }
 
+constexpr size_t kSmemMax = 227 * 1024;  // shared memory of one CTA
+constexpr size_t kSmemSm = 228 * 1024;   // of an SM
+static size_t light_smem_bytes(int64_t ng) {
+  return sizeof(LightSmem) + sizeof(uint32_t) * size_t(((ng + 31) / 32 + ng + 3) & ~int64_t(3));
+}
+
 size_t rank_smem_bytes(int64_t ng, int threads) {
   (void)threads;
   const size_t fixed = rank_smem_fixed(ng);
@@ -799,7 +1017,7 @@ int launch_rank_prep(const Shape& sh, const Buffers& b, int src, long long* stat
   launch_scan(b.colcnt, n, b.colptr, s);
   cudaMemsetAsync(b.colcnt, 0, sizeof(int32_t) * (n + 1), s);
   k5_fill<<<unsigned((ng * kWarp + T - 1) / T), T, 0, s>>>(b.start[src], b.len[src], b.col[src], b.val[src], b.rnorm,
-                                                           nq, n, b.colptr, b.colcnt, b.csc_row, b.csc_val, status,
+                                                           nq, n, b.colptr, b.colcnt, b.csc, status,
                                                            rows_sel);
   return 3;
 }
@@ -817,8 +1035,7 @@ int launch_rank_queries(const Shape& sh, const Buffers& b, int src, int32_t* out
   A.val = b.val[src];
   A.rn = b.rnorm;
   A.colptr = b.colptr;
-  A.csc_row = b.csc_row;
-  A.csc_val = b.csc_val;
+  A.csc = b.csc;
   A.nq = nq;
   A.ng = ng;
   A.topk = sh.topk;
@@ -828,15 +1045,48 @@ int launch_rank_queries(const Shape& sh, const Buffers& b, int src, int32_t* out
   A.out_dist = out_dist;
   A.gscratch = b.rank_scratch;
   A.reuse = reuse ? *reuse : RankReuse{};
-  const size_t smem = rank_smem_bytes(ng, RT);
-  A.acc_smem = smem - rank_smem_fixed(ng) >= sizeof(uint32_t) * size_t(ng);
   rank_caps(&A.sort_cap, &A.bucket_cap);
   A.status = status;
-  cudaFuncSetAttribute(k6_rank, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  A.qlist = nullptr;
+  A.qcount = nullptr;
+  A.over = b.rank_over + 4;
+  A.over_count = b.rank_over;
   const int64_t nqry = q1 - q0;
+  int nl = 1;
+  // Queries with few non-zeros first, where the scores fit the light kernel's
+  // shared memory beside its lists: two CTAs of 512 threads per SM while they
+  // fit twice (up to ~19,800 gallery rows), else one of 1,024.
+  const size_t light = light_smem_bytes(ng);
+  if (light <= kSmemMax && ng <= 65536 && A.sort_cap == SORT_CAP) {
+    cudaMemsetAsync(A.over_count, 0, sizeof(int32_t), s);
+    const bool two = 2 * (light + 1024) <= kSmemSm;
+    const int64_t ctas = int64_t(sh.rank_ctas) * (two ? 2 : 1);
+    const unsigned lg = unsigned(nqry < ctas ? (nqry > 0 ? nqry : 1) : ctas);
+    if (two) {
+      cudaFuncSetAttribute(k6_rank_light<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(light));
+      k6_rank_light<512><<<lg, 512, light, s>>>(A);
+    } else {
+      cudaFuncSetAttribute(k6_rank_light<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(light));
+      k6_rank_light<1024><<<lg, 1024, light, s>>>(A);
+    }
+    A.qlist = A.over;
+    A.qcount = A.over_count;
+    ++nl;
+  }
+  size_t smem = rank_smem_bytes(ng, RT);
+  A.acc_smem = smem - rank_smem_fixed(ng) >= sizeof(uint32_t) * size_t(ng);
+  const size_t with_idx = rank_smem_fixed(ng) + sizeof(uint32_t) * size_t(ng) + ((sizeof(uint16_t) * size_t(ng) + 15) & ~size_t(15));
+  A.idx_smem = A.acc_smem && ng <= 65536 && with_idx <= kSmemMax;
+  if (A.idx_smem && with_idx > smem) smem = with_idx;
   const unsigned grid = unsigned(nqry < sh.rank_ctas ? (nqry > 0 ? nqry : 1) : sh.rank_ctas);
-  k6_rank<<<grid, RT, smem, s>>>(A);
-  return 1;
+  if (A.acc_smem) {
+    cudaFuncSetAttribute(k6_rank<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    k6_rank<true><<<grid, RT, smem, s>>>(A);
+  } else {
+    cudaFuncSetAttribute(k6_rank<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    k6_rank<false><<<grid, RT, smem, s>>>(A);
+  }
+  return nl;
 }
 
 int rank_threads() { return RT; }

@@ -136,8 +136,7 @@ struct Server {
   };
   std::vector<ResLayer> res_layers;
   int64_t* res_colptr = nullptr;  // the last layer as CSC (row norms applied): gallery columns
-  int32_t* res_csc_row = nullptr;
-  float* res_csc_val = nullptr;
+  int2* res_csc = nullptr;
   int32_t* res_nbr = nullptr;
   float* res_nbr_w = nullptr;
   int32_t* res_nbr_n = nullptr;
@@ -602,8 +601,7 @@ rerank_status enqueue_request(Server& v, Slot& sl, const rerank_request& rq, cud
     const uint8_t* last = sl.chg[v.layers & 1];
     RankReuse rr;
     rr.colptr = v.res_colptr;
-    rr.row = v.res_csc_row;
-    rr.val = v.res_csc_val;
+    rr.csc = v.res_csc;
     rr.changed = last + Q;
     rr.shift = Q;
     launch_rank_prep(sh, b, src, status, s, last);
@@ -763,8 +761,7 @@ rerank_status build_resident_graph(Server& v, cudaStream_t s0, long long* gst, s
     v.res_nbr_w = nullptr;
     v.res_nbr_n = nullptr;
     v.res_colptr = nullptr;
-    v.res_csc_row = nullptr;
-    v.res_csc_val = nullptr;
+    v.res_csc = nullptr;
     v.reuse = false;
   };
   bool ok = true;
@@ -816,13 +813,11 @@ rerank_status build_resident_graph(Server& v, cudaStream_t s0, long long* gst, s
            cudaStreamSynchronize(s0) == cudaSuccess;
     }
     if (ok) {
-      v.res_csc_row = static_cast<int32_t*>(alloc(size_t(std::max<int64_t>(nnz, 1)) * 4));
-      v.res_csc_val = static_cast<float*>(alloc(size_t(std::max<int64_t>(nnz, 1)) * 4));
-      ok = v.res_csc_row && v.res_csc_val;
+      v.res_csc = static_cast<int2*>(alloc(size_t(std::max<int64_t>(nnz, 1)) * sizeof(int2)));
+      ok = v.res_csc != nullptr;
     }
     if (ok) {
-      copy_rows(v.res_csc_row, b.csc_row, size_t(nnz) * 4, s0);
-      copy_rows(v.res_csc_val, b.csc_val, size_t(nnz) * 4, s0);
+      copy_rows(v.res_csc, b.csc, size_t(nnz) * sizeof(int2), s0);
     }
   }
   long long hst[kStCount];
