@@ -318,6 +318,138 @@ __global__ void __launch_bounds__(256) k0_normalize_vec(const float* __restrict_
   }
 }
 
+// BF16 rows and FP32 rows of odd widths (no 16-byte loads), dp <= 32 NE: as
+// k0_normalize, element for element in the same order (the same bits), with the
+// row held in registers, so that the input is read once with all its loads in
+// flight and no output is read back: 31 us for 5,118 x 2,048 BF16 (k0_normalize 48).
+template <int MODE, int NE, class T>
+__global__ void __launch_bounds__(128) k0_normalize_reg(const T* __restrict__ xq, const T* __restrict__ xg, int64_t nq,
+                                                        int64_t n, int64_t np, int d, int dp,
+                                                        float* __restrict__ xhat, double* __restrict__ norm,
+                                                        void* __restrict__ xlow, __nv_bfloat16* __restrict__ xhi,
+                                                        __nv_bfloat16* __restrict__ xlo, float* __restrict__ inv_scale,
+                                                        float* __restrict__ err, float* __restrict__ emax,
+                                                        long long* __restrict__ status) {
+  const int64_t row = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (row >= np) return;
+  float* out = xhat + row * dp + lane;
+  __nv_bfloat16* outh = MODE != 0 ? xhi + row * dp + lane : nullptr;
+  __nv_bfloat16* outl = MODE != 0 ? xlo + row * dp + lane : nullptr;
+  __nv_fp8_e4m3* out8 = MODE == 2 ? reinterpret_cast<__nv_fp8_e4m3*>(xlow) + row * dp + lane : nullptr;
+  float x[NE];
+  double tot = 0.0;
+  bool bad = false;
+  if (row < n) {
+    const T* src = (row < nq ? xq + row * int64_t(d) : xg + (row - nq) * int64_t(d)) + lane;
+#pragma unroll
+    for (int t = 0; t < NE; ++t) x[t] = lane + kWarp * t < d ? float(src[kWarp * t]) : 0.f;
+    float s = 0.f, c = 0.f;
+#pragma unroll
+    for (int t = 0; t < NE; ++t) {
+      // a zero element leaves (s, c) unchanged
+      bad |= !isfinite(x[t]);
+      const float p = x[t] * x[t];
+      const float ep = fmaf(x[t], x[t], -p);
+      float tt, e;
+      two_sum(s, p, tt, e);
+      s = tt;
+      c += e + ep;
+    }
+    tot = warp_sum(double(s) + double(c));
+    bad = __any_sync(kFull, bad);
+  }
+  if (row >= n || bad || !(tot > 0.0)) {
+    if (row < n && lane == 0) {
+      set_error(status, bad ? kErrNonFinite : kErrZeroNorm);
+      atomicMin(reinterpret_cast<unsigned long long*>(status + kStBadRow), (unsigned long long)row);
+      norm[row] = 1.0;
+    }
+    for (int k = 0; k + lane < dp; k += kWarp) {
+      out[k] = 0.f;
+      if (MODE != 0) {
+        outh[k] = __float2bfloat16_rn(0.f);
+        outl[k] = __float2bfloat16_rn(0.f);
+      }
+      if (MODE == 2) out8[k] = __nv_fp8_e4m3(0.f);
+    }
+    if (MODE != 0 && lane == 0) {
+      err[row] = 0.f;
+      err[np + row] = 0.f;
+      err[2 * np + row] = 0.f;
+      if (MODE == 2) inv_scale[row] = 0.f;
+    }
+    return;
+  }
+  const double nrm = sqrt(tot);
+  const float r32 = float(1.0 / nrm);
+  if (lane == 0) norm[row] = nrm;
+  float e_lo = 0.f, e_r = 0.f, e_main = 0.f, amax = 0.f;
+#pragma unroll
+  for (int t = 0; t < NE; ++t) {
+    if (lane + kWarp * t >= dp) continue;
+    const float v = x[t] * r32;
+    x[t] = v;
+    out[kWarp * t] = v;
+    if (MODE != 0) {
+      const __nv_bfloat16 h = __float2bfloat16_rn(v);
+      const float dh = v - __bfloat162float(h);          // exact
+      const __nv_bfloat16 l = __float2bfloat16_rn(dh);
+      const float rr = dh - __bfloat162float(l);          // exact
+      outh[kWarp * t] = h;
+      outl[kWarp * t] = l;
+      e_lo = fmaf(__bfloat162float(l), __bfloat162float(l), e_lo);
+      e_r = fmaf(rr, rr, e_r);
+      if (MODE == 1) e_main = fmaf(dh, dh, e_main);  // xlow = hi: its error is lo + r
+    }
+    if (MODE == 2) amax = fmaxf(amax, fabsf(v));
+  }
+  if (MODE == 2) {
+    amax = warp_max_f(amax);
+    const float sc = 448.0f / amax;
+    const float inv = amax / 448.0f;
+#pragma unroll
+    for (int t = 0; t < NE; ++t) {
+      if (lane + kWarp * t >= dp) continue;
+      const __nv_fp8_e4m3 q(x[t] * sc);
+      out8[kWarp * t] = q;
+      const float dv = x[t] - float(q) * inv;
+      e_main = fmaf(dv, dv, e_main);
+    }
+    if (lane == 0) inv_scale[row] = inv;
+  }
+  if (MODE != 0) {
+    const float b0 = bound_of(warp_sum(e_main));
+    const float b1 = bound_of(warp_sum(e_lo));
+    const float b2 = bound_of(warp_sum(e_r));
+    if (lane == 0) {
+      err[row] = b0;
+      err[np + row] = b1;
+      err[2 * np + row] = b2;
+      atomicMax(reinterpret_cast<int*>(emax), __float_as_int(b0));
+      atomicMax(reinterpret_cast<int*>(emax) + 1, __float_as_int(b1));
+      atomicMax(reinterpret_cast<int*>(emax) + 2, __float_as_int(b2));
+    }
+  }
+}
+
+template <class T>
+void launch_reg(const Shape& sh, const void* xq, const void* xg, float* xhat, double* norm, void* xlow,
+                __nv_bfloat16* xhi, __nv_bfloat16* xlo, float* inv_scale, float* err, float* emax, int precision,
+                long long* status, cudaStream_t s) {
+  const unsigned blocks = unsigned((sh.np * kWarp + 127) / 128);
+  const T* q = static_cast<const T*>(xq);
+  const T* g = static_cast<const T*>(xg);
+  auto go = [&](auto kernel) {
+    kernel<<<blocks, 128, 0, s>>>(q, g, sh.nq, sh.n, sh.np, sh.d, sh.dp, xhat, norm, xlow, xhi, xlo, inv_scale, err,
+                                  emax, status);
+  };
+  const bool small = sh.dp <= 512;
+  if (precision == RERANK_PREC_BF16) small ? go(k0_normalize_reg<1, 16, T>) : go(k0_normalize_reg<1, 64, T>);
+  else if (precision == RERANK_PREC_FP8) small ? go(k0_normalize_reg<2, 16, T>) : go(k0_normalize_reg<2, 64, T>);
+  else small ? go(k0_normalize_reg<0, 16, T>) : go(k0_normalize_reg<0, 64, T>);
+}
+
 }  // namespace
 
 int launch_normalize(const Shape& sh, const void* xq, const void* xg, float* xhat, double* norm, void* xlow,
@@ -343,6 +475,14 @@ int launch_normalize(const Shape& sh, const void* xq, const void* xg, float* xha
     else
       k0_normalize_vec<0><<<blocks, threads, 0, s>>>(fq, fg, sh.nq, sh.n, sh.np, sh.d, sh.dp, xhat, norm, nullptr,
                                                      nullptr, nullptr, nullptr, nullptr, nullptr, status);
+    return 1;
+  }
+  if (sh.dp <= 2048) {
+    if (precision != RERANK_PREC_FP32) cudaMemsetAsync(emax, 0, 4 * sizeof(float), s);
+    if (sh.dtype == RERANK_DTYPE_BF16)
+      launch_reg<__nv_bfloat16>(sh, xq, xg, xhat, norm, xlow, xhi, xlo, inv_scale, err, emax, precision, status, s);
+    else
+      launch_reg<float>(sh, xq, xg, xhat, norm, xlow, xhi, xlo, inv_scale, err, emax, precision, status, s);
     return 1;
   }
   if (precision == RERANK_PREC_BF16) {
