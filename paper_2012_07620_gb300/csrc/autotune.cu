@@ -180,6 +180,7 @@ rerank_status rerank_autotune(rerank_ctx* ctx, const void* xq, int64_t nq, const
   const int64_t col_tiles = (n + (prec == RERANK_PREC_FP32 ? 127 : 255)) / (prec == RERANK_PREC_FP32 ? 128 : 256);
   Tuning best = lookup_tuning(ctx, prec, n, d);
   best.sim_chunks = 0;
+  if (best.refine_order < 0) best.refine_order = 1;  // both are tried below
   double best_ms = 0.0;
   do {
     // 0. candidates kept beyond k1: more cost in the similarity epilogue and

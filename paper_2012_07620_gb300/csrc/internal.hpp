@@ -39,7 +39,7 @@ struct Carver {
 struct Tuning {
   int sim_chunks = 0;      // column chunks P of the similarity top-K kernel (0 = from the SM count)
   int prop_warps = 8;      // warps per CTA of the propagation kernel
-  int refine_order = 1;    // 1: refine rows cluster by cluster, 0: in index order
+  int refine_order = -1;   // 1: refine rows cluster by cluster, 0: in index order, -1: by the unit rows' size
   int rescore_m = -1;      // candidates kept beyond k1 (-1: the context's cfg.rescore_m)
   int rank_threads = 1024; // threads per CTA of the final ranking kernel
 };

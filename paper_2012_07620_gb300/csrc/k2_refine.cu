@@ -125,6 +125,51 @@ __device__ __forceinline__ void dot2_fp32(const float* xi, const float* y0, cons
 }
 
 
+// One sorted candidate list: entries up to the first index outside [0, n) (a
+// warp; K <= 64).  Same result as merge_lists with P = 1.
+__device__ __forceinline__ int take_list(WarpSmem& w, const float* ls, const int32_t* li, int K, int64_t n, int lane,
+                                         float& B) {
+  const int j1 = lane + kWarp;
+  const int32_t i0 = lane < K ? li[lane] : -1, i1 = j1 < K ? li[j1] : -1;
+  const float s0 = lane < K ? ls[lane] : 0.f, s1 = j1 < K ? ls[j1] : 0.f;
+  const unsigned bad0 = __ballot_sync(kFull, i0 < 0 || i0 >= n), bad1 = __ballot_sync(kFull, i1 < 0 || i1 >= n);
+  const int cnt = bad0 ? __ffs(bad0) - 1 : (bad1 ? 31 + __ffs(bad1) : 2 * kWarp);
+  if (lane < cnt) {
+    w.idx[lane] = i0;
+    w.g[lane] = s0;
+  }
+  if (j1 < cnt) {
+    w.idx[j1] = i1;
+    w.g[j1] = s1;
+  }
+  __syncwarp();
+  B = cnt == K ? w.g[K - 1] : -FLT_MAX;
+  return cnt;
+}
+
+// The candidates in near-tie runs, as bits of their sorted positions: bit q of
+// `gap` says sorted positions q and q + 1 are within 2 eps_r; q is in a run when
+// bit q - 1 or bit q is set, and the run reaches into the top-k1 when q < k1 or
+// bits k1 - 1 .. q - 1 are all set (K <= 64: each lane tests positions lane and
+// lane + 32; the result is the same in every lane).
+__device__ __forceinline__ uint64_t near_ties(const WarpSmem& w, int K, int k1, double eps_r, int lane) {
+  const int q1 = lane + kWarp;
+  const bool f0 = lane + 1 < K && double(w.s[w.ord[lane]]) - double(w.s[w.ord[lane + 1]]) <= 2.0 * eps_r;
+  const bool f1 = q1 + 1 < K && double(w.s[w.ord[q1]]) - double(w.s[w.ord[q1 + 1]]) <= 2.0 * eps_r;
+  const uint64_t gap = uint64_t(__ballot_sync(kFull, f0)) | (uint64_t(__ballot_sync(kFull, f1)) << 32);
+  if (!gap) return 0ull;
+  auto in = [&](int q) {
+    bool nd = q < K && (((gap >> q) & 1ull) || (q > 0 && ((gap >> (q - 1)) & 1ull)));
+    if (nd && q >= k1) {
+      const int span = q - (k1 - 1);  // bits k1 - 1 .. q - 1
+      const uint64_t want = span >= 64 ? ~0ull : ((1ull << span) - 1ull);
+      nd = ((gap >> (k1 - 1)) & want) == want;
+    }
+    return nd;
+  };
+  return uint64_t(__ballot_sync(kFull, in(lane))) | (uint64_t(__ballot_sync(kFull, in(q1))) << 32);
+}
+
 // P-way merge of sorted candidate lists src[p*K .. p*K+K) for p < P (P <= 32),
 // one list per lane.  Fills w.idx/w.g with the best K; returns the count and
 // the bound B on every candidate that was not taken.  An index outside
@@ -303,29 +348,22 @@ __device__ bool refine_warp(WarpSmem& w, int Kc, int64_t i, int k1, float B, dou
   if (!ok && !last) return false;
 
   // Runs of near-equal FP32 scores that reach into the top-k1.
-  if (lane == 0) {
-    int r = 0;
-    while (r < K) {
-      int r1 = r;
-      while (r1 + 1 < K && double(w.s[w.ord[r1]]) - double(w.s[w.ord[r1 + 1]]) <= 2.0 * eps_r) ++r1;
-      if (r1 > r && r < k1)
-        for (int q = r; q <= r1; ++q) w.need[w.ord[q]] = 1;
-      r = r1 + 1;
-    }
+  const uint64_t ties = near_ties(w, K, k1, eps_r, lane);
+  if (ties) {
+    for (int q = lane; q < K; q += kWarp) w.need[w.ord[q]] = (ties >> q) & 1ull;
+    __syncwarp();
   }
-  __syncwarp();
-  int nneed = 0;
-  for (int c = 0; c < K; ++c) {
-    if (!w.need[c]) continue;
+  for (uint64_t m = ties; m; m &= m - 1ull) {
+    const int c = w.ord[__ffsll(m) - 1];
     const int j = w.idx[c];
     double t = 1.0;
     if (j != i) t = dot_fp64_raw(io, i, j, lane) / (io.norm[i] * io.norm[j]);
     if (lane == 0) w.t[c] = t;
-    ++nneed;
   }
+  const int nneed = __popcll(ties);
   __syncwarp();
-  if (lane == 0) {
-    if (nneed) atomicAdd(reinterpret_cast<unsigned long long*>(io.status + kStFp64), (unsigned long long)nneed);
+  if (lane == 0 && nneed) {
+    atomicAdd(reinterpret_cast<unsigned long long*>(io.status + kStFp64), (unsigned long long)nneed);
     // Re-sort each run by (FP64 value desc, index asc); runs are maximal
     // blocks of consecutive needed positions whose gaps are <= 2 eps_r.
     int r = 0;
@@ -417,7 +455,9 @@ k2_refine(RowIo io, int64_t n, const float* __restrict__ part_s, const int32_t* 
     // bits, repeated columns): they are not read, and every row goes on to the
     // exact stage as one with no candidates.
     const bool aborted = (io.status[kStErr] & kErrTimeout) != 0;
-    const int cnt = aborted ? 0 : merge_lists(w, part_s + base, part_i + base, P, K, n, lane, B);
+    const int cnt = aborted ? 0
+                    : P == 1 ? take_list(w, part_s + base, part_i + base, K, n, lane, B)
+                             : merge_lists(w, part_s + base, part_i + base, P, K, n, lane, B);
     if (cnt < K && fl.in) B = key_score(fl.in[part_by_row ? i : f]);
     if (cnt == n) B = -FLT_MAX;  // every column is a candidate
     // Fewer than k1 candidates (only after an aborted similarity stage): the
@@ -559,7 +599,9 @@ k2_refine_cta(RowIo io, int64_t n, const float* __restrict__ part_s, const int32
       const size_t base = size_t(part_by_row ? i : f) * P * Kmax;
       const bool aborted = (io.status[kStErr] & kErrTimeout) != 0;
       int cnt = 0;
-      if (!aborted && P * Kmax <= MERGE_CAP) {
+      if (!aborted && P == 1) {
+        if (wid == 0) cnt = take_list(w, part_s + base, part_i + base, Kmax, n, lane, B);
+      } else if (!aborted && P * Kmax <= MERGE_CAP) {
         cnt = merge_lists_cta(w, msm, part_s + base, part_i + base, P, Kmax, n, t, NW * kWarp, B);
       } else if (!aborted && wid == 0) {
         cnt = merge_lists(w, part_s + base, part_i + base, P, Kmax, n, lane, B);
@@ -619,33 +661,9 @@ k2_refine_cta(RowIo io, int64_t n, const float* __restrict__ part_s, const int32
       if (wid == 0) {
         bool cert = true;
         if (K == Kc && sB > -FLT_MAX) cert = double(w.s[w.ord[k1 - 1]]) - eps_r > double(sB) + eps_g;
-        // Runs of near-equal FP32 scores that reach into the top-k1, in
-        // parallel: bit q of `gap` says sorted positions q and q + 1 are within
-        // 2 eps_r; q is in a run when bit q - 1 or bit q is set, and the run
-        // reaches into the top-k1 when q < k1 or bits k1 - 1 .. q - 1 are all
-        // set (K <= 64: each lane takes positions lane and lane + 32).
-        const int q0 = lane, q1 = lane + kWarp;
-        const bool f0 = q0 + 1 < K && double(w.s[w.ord[q0]]) - double(w.s[w.ord[q0 + 1]]) <= 2.0 * eps_r;
-        const bool f1 = q1 + 1 < K && double(w.s[w.ord[q1]]) - double(w.s[w.ord[q1 + 1]]) <= 2.0 * eps_r;
-        const uint64_t gap = uint64_t(__ballot_sync(kFull, f0)) | (uint64_t(__ballot_sync(kFull, f1)) << 32);
-        int nneed = 0;
-  #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int q = h ? q1 : q0;
-          if (q < K) {
-            const bool inrun = ((gap >> q) & 1ull) || (q > 0 && ((gap >> (q - 1)) & 1ull));
-            bool nd = inrun;
-            if (q >= k1 && inrun) {
-              const int span = q - (k1 - 1);  // bits k1 - 1 .. q - 1
-              const uint64_t want = span >= 64 ? ~0ull : ((1ull << span) - 1ull);
-              nd = ((gap >> (k1 - 1)) & want) == want;
-            }
-            nd = nd && cert;
-            w.need[w.ord[q]] = nd ? 1 : 0;
-            nneed += nd ? 1 : 0;
-          }
-        }
-        nneed = warp_sum(nneed);
+        const uint64_t ties = cert ? near_ties(w, K, k1, eps_r, lane) : 0ull;
+        for (int q = lane; q < K; q += kWarp) w.need[w.ord[q]] = (ties >> q) & 1ull;
+        const int nneed = __popcll(ties);
         if (lane == 0) {
           sh[2] = cert ? 1 : 0;
           sh[3] = nneed;
@@ -668,8 +686,8 @@ k2_refine_cta(RowIo io, int64_t n, const float* __restrict__ part_s, const int32
         }
         __syncthreads();
         if (wid == 0) {
-          if (lane == 0) {
-            if (sh[3]) atomicAdd(reinterpret_cast<unsigned long long*>(io.status + kStFp64), (unsigned long long)sh[3]);
+          if (lane == 0 && sh[3]) {
+            atomicAdd(reinterpret_cast<unsigned long long*>(io.status + kStFp64), (unsigned long long)sh[3]);
             // Re-sort each run by (FP64 value desc, index asc).
             int r = 0;
             while (r < K) {

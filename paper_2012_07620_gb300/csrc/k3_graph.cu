@@ -83,50 +83,68 @@ __global__ void k3_sort_count(const int32_t* __restrict__ knn, int64_t n, int k1
   if (lane == 0) rowcnt[i] = feature == RERANK_FEAT_A ? k1 : k1 + m - both;
 }
 
-// One thread per row: merge the two sorted lists into row i of A* (or copy A).
+// One warp per row: the sorted union of the two sorted lists as row i of A* (or
+// a copy of A).  An entry's place is its own place plus the entries of the other
+// list before it, less the common entries before it (counted once): binary
+// searches in the other list and ballots over the out-list's common entries
+// (k1 <= 64), instead of a serial merge by one thread (20 us at any size: a
+// chain of ~60 dependent loads).
 __global__ void k3_fill(const int32_t* __restrict__ out_sorted, const int32_t* __restrict__ in_sorted,
                         const int32_t* __restrict__ inptr, const int32_t* __restrict__ h0ptr, int64_t n, int k1,
                         int feature, int32_t* __restrict__ col, float* __restrict__ val,
                         int64_t* __restrict__ start, int32_t* __restrict__ len, long long* __restrict__ nnz0) {
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int64_t i = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
   if (i >= n) return;
   const int32_t* o = out_sorted + i * k1;
-  int32_t pos = h0ptr[i];
+  const int32_t pos = h0ptr[i];
+  int total = k1;
   if (feature == RERANK_FEAT_A) {
-    for (int p = 0; p < k1; ++p) {
+    for (int p = lane; p < k1; p += kWarp) {
       col[pos + p] = o[p];
       val[pos + p] = 1.0f;
     }
-    pos += k1;
   } else {
     const int32_t* in = in_sorted + inptr[i];
     const int m = inptr[i + 1] - inptr[i];
-    int p = 0, q = 0;
-    while (p < k1 || q < m) {
-      const int32_t vo = p < k1 ? o[p] : kInvalidIdx;
-      const int32_t vi = q < m ? in[q] : kInvalidIdx;
-      if (vo == vi) {
-        col[pos] = vo;
-        val[pos] = 1.0f;
-        ++p;
-        ++q;
-      } else if (vo < vi) {
-        col[pos] = vo;
-        val[pos] = 0.5f;
-        ++p;
-      } else {
-        col[pos] = vi;
-        val[pos] = 0.5f;
-        ++q;
-      }
-      ++pos;
+    int32_t v[2];
+    int lb[2];
+    bool both[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int p = lane + h * kWarp;
+      v[h] = p < k1 ? o[p] : kInvalidIdx;
+      lb[h] = p < k1 ? lower_bound(in, m, v[h]) : 0;
+      both[h] = p < k1 && lb[h] < m && in[lb[h]] == v[h];
     }
+    const uint64_t common = uint64_t(__ballot_sync(kFull, both[0])) | (uint64_t(__ballot_sync(kFull, both[1])) << 32);
+    auto before = [&](int p) { return __popcll(common & ((p < 64 ? 1ull << p : 0ull) - 1ull)); };
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int p = lane + h * kWarp;
+      if (p < k1) {
+        const int at = pos + p + lb[h] - before(p);
+        col[at] = v[h];
+        val[at] = both[h] ? 1.0f : 0.5f;
+      }
+    }
+    for (int q = lane; q < m; q += kWarp) {
+      const int32_t w = in[q];
+      const int p = lower_bound(o, k1, w);
+      if (p < k1 && o[p] == w) continue;  // common: written above
+      const int at = pos + q + p - before(p);
+      col[at] = w;
+      val[at] = 0.5f;
+    }
+    total = k1 + m - __popcll(common);
   }
-  start[i] = h0ptr[i];
-  len[i] = pos - h0ptr[i];
-  if (i == n - 1) {
-    start[n] = pos;
-    if (nnz0) *nnz0 = pos;  // nnz of h^(0)
+  if (lane == 0) {
+    start[i] = pos;
+    len[i] = total;
+    if (i == n - 1) {
+      start[n] = pos + total;
+      if (nnz0) *nnz0 = pos + total;  // nnz of h^(0)
+    }
   }
 }
 
@@ -396,7 +414,7 @@ int launch_graph(const Shape& sh, const Buffers& b, float alpha, int aggregator,
   k3_sort_count<<<unsigned((n * kWarp + T - 1) / T), T, 0, s>>>(b.knn_idx, n, sh.k1, b.inptr, b.insrc, b.out_sorted,
                                                                b.in_sorted, b.rowcnt, feature);
   launch_scan32(b.rowcnt, n, b.h0ptr, s);
-  k3_fill<<<unsigned((n + T - 1) / T), T, 0, s>>>(b.out_sorted, b.in_sorted, b.inptr, b.h0ptr, n, sh.k1, feature,
+  k3_fill<<<unsigned((n * kWarp + T - 1) / T), T, 0, s>>>(b.out_sorted, b.in_sorted, b.inptr, b.h0ptr, n, sh.k1, feature,
                                                   b.col[2], b.val[2], b.start[2], b.len[2],
                                                   status ? status + kStNnz0 : nullptr);
   k3_edges<<<unsigned((n + T - 1) / T), T, 0, s>>>(b.knn_idx, b.knn_score, n, sh.k1, sh.k2, alpha, aggregator, b.nbr,
