@@ -441,12 +441,12 @@ rerank_status enqueue_job(rerank_ctx* ctx, const JobRun& j, cudaStream_t s, Stag
     for (int l = 0; l < sh.layers; ++l) {
       const int dst = l & 1;
       nl += launch_propagate(sh, b, src, dst, ctx->cfg.aggregator, status, ctx->sm_count, sh.tune, s, nullptr,
-                             l < 8 ? status + kStNnz0 + l + 1 : nullptr);
+                             l < 8 ? status + kStNnz0 + l + 1 : nullptr, l + 1 == sh.layers ? b.rnorm : nullptr);
       src = dst;
     }
     RR_CUDA(cudaGetLastError());
     mark("propagate");
-    nl += launch_row_norms(sh, b, src, status, s);
+    if (sh.layers == 0) nl += launch_row_norms(sh, b, src, status, s);
     int32_t* oi = sh.host_out ? b.out_idx : j.out_idx;
     float* od = sh.host_out ? b.out_dist : j.out_dist;
     if (sh.host_out && copy_overlap && sh.nq >= 4 * int64_t(ctx->sm_count)) {

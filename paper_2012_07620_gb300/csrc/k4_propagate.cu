@@ -10,9 +10,10 @@
 // max is exact, so the result does not depend on the order either.  Features
 // are stored as padded CSR: row
 // i occupies [start_i, start_i + len_i) of (col, val), each column at most
-// once, in no particular order (h^(0) from K3 is ascending).  start_i is an
-// exclusive scan of ub_i = sum_j len_j, an upper bound on the output row, so
-// every row can be written without a second pass.
+// once, in no particular order (h^(0) from K3 is ascending).  A row's warp takes
+// its place from a cursor, ub_i = sum_j len_j entries (an upper bound on the
+// output row), so every row is written without a second pass and no scan
+// precedes the layer.
 //
 // Rows whose distinct columns fit three quarters of a 512-slot table (almost
 // all): one warp per row with a private open-addressing hash table in shared
@@ -44,39 +45,6 @@ constexpr int MSLOTS = 2048;  // hash slots per warp of the second pass (16 KB)
 constexpr int RWARPS = 12;    // warps of k4_spmm_rest (192 KB of tables, one CTA per SM)
 constexpr int RTHREADS = RWARPS * 32;
 constexpr int KEY_EMPTY = -1;
-
-__global__ void k4_ub(const int32_t* __restrict__ nbr, const int32_t* __restrict__ nbr_n, int k2p1,
-                      const int32_t* __restrict__ len, int64_t n, int32_t* __restrict__ ub,
-                      int32_t* __restrict__ big_rows, int32_t* __restrict__ big_count,
-                      const long long* __restrict__ status, LayerReuse reuse) {
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  if (status[kStErr] & kErrOverflow) {
-    ub[i] = 0;
-    return;
-  }
-  int64_t u = 0;
-  const int m = nbr_n[i];
-  for (int q = 0; q < m; ++q) u += len[nbr[i * k2p1 + q]];
-  if (u > n) u = n;
-  const bool copied = reuse.changed && !reuse.changed[i];
-  if (copied) u = max(u, int64_t(reuse.rlen[i - reuse.shift]));  // room for the copied row
-  ub[i] = int32_t(u);
-  if (u > WDIRECT && !copied) big_rows[atomicAdd(big_count, 1)] = int32_t(i);
-}
-
-__device__ __forceinline__ bool capacity_ok(const int64_t* dstart, int64_t n, int64_t cap, long long* status) {
-  if (status[kStErr] & kErrOverflow) return false;
-  const int64_t need = dstart[n];
-  if (need > cap) {
-    if (threadIdx.x == 0) {
-      set_error(status, kErrOverflow);
-      atomicMax(reinterpret_cast<unsigned long long*>(status + kStNeed), (unsigned long long)need);
-    }
-    return false;
-  }
-  return true;
-}
 
 // Adds v to the entry of `col` (or, with take_max, raises it to v; entries
 // start at 0 and every value is >= 0); returns true when this call created it.
@@ -154,7 +122,7 @@ __device__ __forceinline__ int next_pow2(int x) {
 constexpr int kMaxPropWarps = 24;  // 24 warps x 4 KB of tables: 96 KB per CTA
 
 // Row i through one warp's SLOTS-entry table (keys / vals: empty on entry and
-// on return).  Returns false when the row was written (lane 0 adds its length
+// on return); o: its place in the output.  Returns false when the row was written (lane 0 adds its length
 // to nnz), true when its distinct columns filled three quarters of the table:
 // then nothing is written and the caller hands the row on.
 template <int SLOTS>
@@ -162,9 +130,9 @@ __device__ bool warp_row(int64_t i, int u, volatile int* keys, float* vals, cons
                          const int32_t* __restrict__ slen, const int32_t* __restrict__ scol,
                          const float* __restrict__ sval, const int32_t* __restrict__ nbr,
                          const float* __restrict__ nbr_w, const int32_t* __restrict__ nbr_n, int k2p1,
-                         const int64_t* __restrict__ dstart, int32_t* __restrict__ dlen, int32_t* __restrict__ dcol,
-                         float* __restrict__ dval, long long* __restrict__ status, bool agg_max, int lane,
-                         unsigned long long& nnz) {
+                         int64_t o, int32_t* __restrict__ dlen, int32_t* __restrict__ dcol,
+                         float* __restrict__ dval, float* __restrict__ rn, long long* __restrict__ status,
+                         bool agg_max, int lane, unsigned long long& nnz) {
   const unsigned lt = (1u << lane) - 1u;
   // Table of at least twice the bound on distinct columns, at most SLOTS; when
   // the bound is larger the row is tried here and handed on if its distinct
@@ -284,10 +252,16 @@ __device__ bool warp_row(int64_t i, int u, volatile int* keys, float* vals, cons
   // below is independent of the order.
   const float ss = warp_sumsq_exact(vals, cnt, lane);
   const float inv = 1.0f / sqrtf(ss);
-  const int64_t o = dstart[i];
   for (int p = lane; p < cnt; p += kWarp) {
+    const float v = vals[p] * inv;
     dcol[o + p] = keys[p];
-    dval[o + p] = vals[p] * inv;
+    dval[o + p] = v;
+    vals[p] = v;
+  }
+  if (rn) {  // the last layer: 1 / ||row|| of the values as written
+    __syncwarp();
+    const float s2 = warp_sumsq_exact(vals, cnt, lane);
+    if (lane == 0) rn[i] = 1.0f / sqrtf(s2);
   }
   if (lane == 0) {
     dlen[i] = cnt;
@@ -307,16 +281,17 @@ __device__ bool warp_row(int64_t i, int u, volatile int* keys, float* vals, cons
 __global__ void __launch_bounds__(kMaxPropWarps * kWarp)
 k4_spmm_warp(const int64_t* __restrict__ sstart, const int32_t* __restrict__ slen, const int32_t* __restrict__ scol,
              const float* __restrict__ sval, const int32_t* __restrict__ nbr, const float* __restrict__ nbr_w,
-             const int32_t* __restrict__ nbr_n, int k2p1, const int32_t* __restrict__ ub,
-             const int64_t* __restrict__ dstart, int32_t* __restrict__ dlen, int32_t* __restrict__ dcol,
-             float* __restrict__ dval, int64_t n, int64_t cap, int32_t* __restrict__ big_rows,
-             int32_t* __restrict__ big_count, int32_t* __restrict__ next_row, long long* __restrict__ status,
-             bool agg_max, LayerReuse reuse, unsigned long long* __restrict__ nnz_out) {
+             const int32_t* __restrict__ nbr_n, int k2p1, int32_t* __restrict__ ub, int64_t* dstart,
+             int32_t* __restrict__ dlen, int32_t* __restrict__ dcol, float* __restrict__ dval,
+             float* __restrict__ rn, int64_t n, int64_t cap, int32_t* __restrict__ big_rows,
+             int32_t* __restrict__ big_count, int32_t* __restrict__ next_row, unsigned long long* __restrict__ cursor,
+             long long* __restrict__ status, bool agg_max, LayerReuse reuse,
+             unsigned long long* __restrict__ nnz_out) {
   extern __shared__ int smem_i[];
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* keys = smem_i + wib * WSLOTS * 2;
   float* vals = reinterpret_cast<float*>(smem_i + wib * WSLOTS * 2 + WSLOTS);
-  if (!capacity_ok(dstart, n, cap, status)) return;
+  if (status[kStErr] & kErrOverflow) return;
   for (int s = lane; s < WSLOTS; s += kWarp) {
     keys[s] = KEY_EMPTY;
     vals[s] = 0.f;
@@ -331,9 +306,39 @@ k4_spmm_warp(const int64_t* __restrict__ sstart, const int32_t* __restrict__ sle
     if (lane == 0) i = atomicAdd(next_row, 1);
     i = __shfl_sync(kFull, i, 0);
     if (i >= n) break;
-    if (reuse.changed && !reuse.changed[i]) {
+    const bool known = reuse.changed && !reuse.changed[i];
+    // The row's place: room for the sum of its messages' lengths (or the known row).
+    long long u64 = 0;
+    if (known) {
+      u64 = lane == 0 ? reuse.rlen[i - reuse.shift] : 0;
+    } else {
+      const int m = nbr_n[i];
+      for (int q = lane; q < m; q += kWarp) u64 += slen[nbr[i * k2p1 + q]];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) u64 += __shfl_xor_sync(kFull, u64, o);
+    if (u64 > n) u64 = n;
+    long long off = 0;
+    if (lane == 0) off = (long long)atomicAdd(cursor, (unsigned long long)u64);
+    off = __shfl_sync(kFull, off, 0);
+    if (off + u64 > cap) {
+      // Every row adds its bound, so the largest value asked for is the whole need.
+      if (lane == 0) {
+        dlen[i] = 0;
+        set_error(status, kErrOverflow);
+        atomicMax(reinterpret_cast<unsigned long long*>(status + kStNeed), (unsigned long long)(off + u64));
+      }
+      continue;
+    }
+    const int u = int(u64);
+    if (lane == 0) {
+      dstart[i] = off;
+      ub[i] = u;
+    }
+    __syncwarp();
+    if (known) {
       // inputs unchanged: the known row, in its own column order
-      const int64_t g = i - reuse.shift, a = reuse.rstart[g], o = dstart[i];
+      const int64_t g = i - reuse.shift, a = reuse.rstart[g], o = off;
       const int m = reuse.rlen[g];
       for (int p = lane; p < m; p += kWarp) {
         dcol[o + p] = int32_t(reuse.rcol[a + p] + reuse.shift);
@@ -345,11 +350,9 @@ k4_spmm_warp(const int64_t* __restrict__ sstart, const int32_t* __restrict__ sle
       }
       continue;
     }
-    const int u = ub[i];
-    if (u > WDIRECT) continue;
-    if (warp_row<WSLOTS>(i, u, keys, vals, sstart, slen, scol, sval, nbr, nbr_w, nbr_n, k2p1, dstart, dlen, dcol,
-                         dval, status, agg_max, lane, nnz) &&
-        lane == 0)
+    const bool handed = u > WDIRECT || warp_row<WSLOTS>(i, u, keys, vals, sstart, slen, scol, sval, nbr, nbr_w, nbr_n,
+                                                        k2p1, off, dlen, dcol, dval, rn, status, agg_max, lane, nnz);
+    if (handed && lane == 0)
       big_rows[atomicAdd(big_count, 1)] = int32_t(i);
   }
   if (nnz_out && lane == 0 && nnz) atomicAdd(nnz_out, nnz);
@@ -364,7 +367,8 @@ __device__ void cta_row(int64_t i, const int64_t* __restrict__ sstart, const int
                         const int32_t* __restrict__ nbr, const float* __restrict__ nbr_w,
                         const int32_t* __restrict__ nbr_n, int k2p1, const int64_t* __restrict__ dstart,
                         int32_t* __restrict__ dlen, int32_t* __restrict__ dcol, float* __restrict__ dval, int64_t n,
-                        float* __restrict__ acc, uint32_t* __restrict__ bm, bool agg_max, int* scan_s,
+                        float* __restrict__ rn, float* __restrict__ acc, uint32_t* __restrict__ bm, bool agg_max,
+                        int* scan_s,
                         unsigned long long* red_hi, unsigned long long* red_lo, unsigned long long& nnz) {
   const int tid = threadIdx.x;
   const int64_t nwords = (n + 31) / 32;
@@ -414,27 +418,35 @@ __device__ void cta_row(int64_t i, const int64_t* __restrict__ sstart, const int
   // The sum of squares as in warp_sumsq_exact (exact squares truncated to
   // 2^-64, added as 128-bit integers), so a row gets the same norm, bit for
   // bit, on every path; the entries are split evenly over the threads.
-  unsigned long long shi = 0, slo = 0;
-  for (int p = tid; p < total; p += RTHREADS) {
-    unsigned long long h, l;
-    sq_fixed(dval[o + p], h, l);
-    slo += l;
-    shi += h + (slo < l ? 1ull : 0ull);
-  }
-  red_hi[tid] = shi;
-  red_lo[tid] = slo;
-  __syncthreads();
-  for (int st = 256; st > 0; st >>= 1) {  // RTHREADS <= 512
-    if (tid < st && tid + st < RTHREADS) {
-      const unsigned long long nl = red_lo[tid] + red_lo[tid + st];
-      red_hi[tid] = red_hi[tid] + red_hi[tid + st] + (nl < red_lo[tid] ? 1ull : 0ull);
-      red_lo[tid] = nl;
+  auto sum_squares = [&] {
+    unsigned long long shi = 0, slo = 0;
+    for (int p = tid; p < total; p += RTHREADS) {
+      unsigned long long h, l;
+      sq_fixed(dval[o + p], h, l);
+      slo += l;
+      shi += h + (slo < l ? 1ull : 0ull);
     }
+    red_hi[tid] = shi;
+    red_lo[tid] = slo;
     __syncthreads();
-  }
-  const float ss = float(double(red_hi[0]) + double(red_lo[0]) * 5.421010862427522e-20);  // 2^-64
-  const float inv = 1.0f / sqrtf(ss);
+    for (int st = 256; st > 0; st >>= 1) {  // RTHREADS <= 512
+      if (tid < st && tid + st < RTHREADS) {
+        const unsigned long long nl = red_lo[tid] + red_lo[tid + st];
+        red_hi[tid] = red_hi[tid] + red_hi[tid + st] + (nl < red_lo[tid] ? 1ull : 0ull);
+        red_lo[tid] = nl;
+      }
+      __syncthreads();
+    }
+    const float ss = float(double(red_hi[0]) + double(red_lo[0]) * 5.421010862427522e-20);  // 2^-64
+    __syncthreads();  // the sums may be overwritten
+    return ss;
+  };
+  const float inv = 1.0f / sqrtf(sum_squares());
   for (int p = tid; p < total; p += RTHREADS) dval[o + p] *= inv;
+  if (rn) {  // the last layer: 1 / ||row|| of the values as written (a thread reads what it wrote)
+    const float s2 = sum_squares();
+    if (tid == 0) rn[i] = 1.0f / sqrtf(s2);
+  }
   if (tid == 0) {
     dlen[i] = total;
     nnz += unsigned(total);
@@ -454,13 +466,13 @@ k4_spmm_rest(const int64_t* __restrict__ sstart, const int32_t* __restrict__ sle
              const int32_t* __restrict__ nbr_n, int k2p1, const int32_t* __restrict__ ub,
              const int32_t* __restrict__ big_rows, const int32_t* __restrict__ big_count, int min_rows,
              int32_t* __restrict__ spill, const int64_t* __restrict__ dstart, int32_t* __restrict__ dlen,
-             int32_t* __restrict__ dcol, float* __restrict__ dval, int64_t n, int64_t cap, float* __restrict__ dense,
-             uint32_t* __restrict__ bits, long long* __restrict__ status, bool agg_max,
+             int32_t* __restrict__ dcol, float* __restrict__ dval, float* __restrict__ rn, int64_t n,
+             float* __restrict__ dense, uint32_t* __restrict__ bits, long long* __restrict__ status, bool agg_max,
              unsigned long long* __restrict__ nnz_out) {
   extern __shared__ int smem_i[];
   __shared__ int scan_s[RTHREADS];
   __shared__ unsigned long long red_hi[RTHREADS], red_lo[RTHREADS];
-  if (!capacity_ok(dstart, n, cap, status)) return;
+  if (status[kStErr] & kErrOverflow) return;
   const int count = *big_count;
   if (count == 0) return;
   const int tid = threadIdx.x, wib = tid >> 5, lane = tid & 31;
@@ -478,7 +490,7 @@ k4_spmm_rest(const int64_t* __restrict__ sstart, const int32_t* __restrict__ sle
     for (int64_t f = int64_t(blockIdx.x) * RWARPS + wib; f < count; f += int64_t(gridDim.x) * RWARPS) {
       const int64_t i = big_rows[f];
       const bool sp = warp_row<MSLOTS>(i, ub[i], keys, vals, sstart, slen, scol, sval, nbr, nbr_w, nbr_n, k2p1,
-                                       dstart, dlen, dcol, dval, status, agg_max, lane, nnz);
+                                       dstart[i], dlen, dcol, dval, rn, status, agg_max, lane, nnz);
       if (lane == 0) spill[f] = sp ? 1 : 0;
     }
     __syncthreads();  // this CTA's flags are written
@@ -486,7 +498,7 @@ k4_spmm_rest(const int64_t* __restrict__ sstart, const int32_t* __restrict__ sle
       for (int w = 0; w < RWARPS && f0 + w < count; ++w)
         if (spill[f0 + w])
           cta_row(big_rows[f0 + w], sstart, slen, scol, sval, nbr, nbr_w, nbr_n, k2p1, dstart, dlen, dcol, dval, n,
-                  acc, bm, agg_max, scan_s, red_hi, red_lo, nnz);
+                  rn, acc, bm, agg_max, scan_s, red_hi, red_lo, nnz);
   } else {
     // The tables are not needed: when the dense accumulator and its bitmap fit
     // the shared memory (n up to ~47,000), they live there (zeroed once; every
@@ -500,7 +512,7 @@ k4_spmm_rest(const int64_t* __restrict__ sstart, const int32_t* __restrict__ sle
       __syncthreads();
     }
     for (int64_t f = blockIdx.x; f < count; f += gridDim.x)
-      cta_row(big_rows[f], sstart, slen, scol, sval, nbr, nbr_w, nbr_n, k2p1, dstart, dlen, dcol, dval, n, a2, b2,
+      cta_row(big_rows[f], sstart, slen, scol, sval, nbr, nbr_w, nbr_n, k2p1, dstart, dlen, dcol, dval, n, rn, a2, b2,
               agg_max, scan_s, red_hi, red_lo, nnz);
   }
   if (nnz_out && lane == 0 && nnz) atomicAdd(nnz_out, nnz);
@@ -545,16 +557,13 @@ int launch_layer_compact(int64_t n, const int64_t* start, const int32_t* len, co
 int propagate_warp_slots() { return WSLOTS; }
 
 int launch_propagate(const Shape& sh, const Buffers& b, int src, int dst, int aggregator, long long* status,
-                      int sm_count, const Tuning& t, cudaStream_t s, const LayerReuse* reuse, long long* nnz_slot) {
+                      int sm_count, const Tuning& t, cudaStream_t s, const LayerReuse* reuse, long long* nnz_slot, float* rnorm) {
   unsigned long long* nnz_out = reinterpret_cast<unsigned long long*>(nnz_slot);
   const int64_t n = sh.n;
   const int k2p1 = sh.k2 + 1;
-  const int T = 256;
-  cudaMemsetAsync(b.big_count, 0, 2 * sizeof(int32_t), s);  // [0]: rows handed on, [1]: next row of the first pass
+  // [0]: rows handed on, [1]: next row of the first pass, [2, 3]: the place cursor
+  cudaMemsetAsync(b.big_count, 0, 4 * sizeof(int32_t), s);
   const LayerReuse ru = reuse ? *reuse : LayerReuse{};
-  k4_ub<<<unsigned((n + T - 1) / T), T, 0, s>>>(b.nbr, b.nbr_n, k2p1, b.len[src], n, b.ub, b.big_rows, b.big_count,
-                                                 status, ru);
-  launch_scan(b.ub, n, b.start[dst], s);
   const int warps = t.prop_warps < 1 ? 1 : (t.prop_warps > kMaxPropWarps ? kMaxPropWarps : t.prop_warps);
   const size_t smem = size_t(warps) * WSLOTS * 2 * sizeof(int);
   cudaFuncSetAttribute(k4_spmm_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
@@ -563,9 +572,10 @@ int launch_propagate(const Shape& sh, const Buffers& b, int src, int dst, int ag
   const unsigned blocks = unsigned(tmin<int64_t>(blocks_needed, int64_t(sm_count) * (per_sm > 0 ? per_sm : 1)));
   k4_spmm_warp<<<blocks, warps * kWarp, smem, s>>>(b.start[src], b.len[src], b.col[src], b.val[src], b.nbr, b.nbr_w,
                                                    b.nbr_n, k2p1, b.ub, b.start[dst], b.len[dst], b.col[dst],
-                                                   b.val[dst], n, sh.cap_h, b.big_rows, b.big_count,
-                                                   b.big_count + 1, status, aggregator == RERANK_AGG_MAX, ru,
-                                                   nnz_out);
+                                                   b.val[dst], rnorm, n, sh.cap_h, b.big_rows, b.big_count,
+                                                   b.big_count + 1,
+                                                   reinterpret_cast<unsigned long long*>(b.big_count + 2), status,
+                                                   aggregator == RERANK_AGG_MAX, ru, nnz_out);
   // The rows the first pass listed: 2,048-slot tables when there are at least
   // 4 per SM (market_hard: 21,906 rows, propagation 2.20 -> 1.13 ms), else the
   // CTA path (market: 549 rows, faster there).
@@ -578,10 +588,10 @@ int launch_propagate(const Shape& sh, const Buffers& b, int src, int dst, int ag
   cudaFuncSetAttribute(k4_spmm_rest, cudaFuncAttributeMaxDynamicSharedMemorySize, int(rsmem));
   k4_spmm_rest<<<sm_count, RTHREADS, rsmem, s>>>(
       b.start[src], b.len[src], b.col[src], b.val[src], b.nbr, b.nbr_w, b.nbr_n, k2p1, b.ub, b.big_rows, b.big_count,
-      min_rows, b.prop_spill, b.start[dst], b.len[dst], b.col[dst], b.val[dst], n, sh.cap_h, b.hash_keys_vals,
+      min_rows, b.prop_spill, b.start[dst], b.len[dst], b.col[dst], b.val[dst], rnorm, n, b.hash_keys_vals,
       reinterpret_cast<uint32_t*>(b.hash_keys_vals + size_t(sm_count) * n), status, aggregator == RERANK_AGG_MAX,
       nnz_out);
-  return 4;
+  return 2;
 }
 
 int launch_row_norms(const Shape& sh, const Buffers& b, int src, const long long* status, cudaStream_t s,

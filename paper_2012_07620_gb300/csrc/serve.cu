@@ -587,12 +587,14 @@ rerank_status enqueue_request(Server& v, Slot& sl, const rerank_request& rq, cud
       ru.rval = rl.val;
       ru.shift = Q;
     }
-    launch_propagate(sh, b, src, dst, ctx->cfg.aggregator, status, sm, sh.tune, s, v.reuse ? &ru : nullptr);
+    launch_propagate(sh, b, src, dst, ctx->cfg.aggregator, status, sm, sh.tune, s, v.reuse ? &ru : nullptr, nullptr,
+                     l + 1 == v.layers ? b.rnorm : nullptr);
     src = dst;
   }
   // With the gallery graph kept, only the rows whose last layer changed (the
-  // queries among them) need their norm: the others' are in the resident lists.
-  launch_row_norms(sh, b, src, status, s, v.reuse ? sl.chg[v.layers & 1] : nullptr);
+  // queries among them) need their norm, and the last layer has written those:
+  // the others' are in the resident lists.
+  if (v.layers == 0) launch_row_norms(sh, b, src, status, s, v.reuse ? sl.chg[v.layers & 1] : nullptr);
   int32_t* oi = host_out ? b.out_idx : rq.out_idx;
   float* od = host_out ? b.out_dist : rq.out_dist;
   if (v.reuse) {
