@@ -294,7 +294,14 @@ __global__ void k3i_count(int64_t n, int64_t Q, int k1, const int32_t* __restric
 
 // Rows of A* into the layer-0 CSR: resident rows copied (indices shifted by
 // Q), affected rows as the sorted union of out and in (1 where in both, else
-// 1/2) by one lane.
+// 1/2).  An entry's place is its place in its own list, plus the entries of
+// the other two lists below it, less the ones counted twice; the kept resident
+// in-sources are numbered by the ballots of the row's chunks of 32.  Merged by
+// one lane, an affected row's chain of dependent loads lasted longer than the
+// copy of all the others (92 us for a request of 4 queries against 40,000
+// rows); with the merges of k_serve_assemble and k_mark_h0 given to whole
+// warps too, a burst of 16 such requests (1 to 512 queries) went from 7.8 to
+// 7.2 ms.  k1 <= 64: two out-neighbours per lane.
 __global__ void k3i_fill(int64_t n, int64_t Q, int k1, const uint8_t* __restrict__ aff,
                          const uint8_t* __restrict__ src, const int32_t* __restrict__ h0ptr,
                          const int32_t* __restrict__ out_sorted, const int32_t* __restrict__ add_ptr,
@@ -323,12 +330,13 @@ __global__ void k3i_fill(int64_t n, int64_t Q, int k1, const uint8_t* __restrict
     }
     return;
   }
-  if (lane != 0) return;
   const int32_t* o = out_sorted + u * k1;
-  const int32_t a = add_ptr[u], m = add_ptr[u + 1] - a;
+  const int32_t a = add_ptr[u];
+  const int m = add_ptr[u + 1] - a;
   const int32_t* ad = add_sorted + a;
-  // The in-list in ascending order: kept resident in-sources and added sources.
-  int64_t ra = 0, rn = 0;
+  // The in-list: the resident row's kept in-sources and the added sources.
+  int64_t ra = 0;
+  int rn = 0;
   const int32_t* rout = nullptr;
   if (u >= Q) {
     const int64_t g = u - Q;
@@ -336,41 +344,74 @@ __global__ void k3i_fill(int64_t n, int64_t Q, int k1, const uint8_t* __restrict
     rn = rln[g];
     rout = res_knn + g * k1;
   }
-  int64_t rp = 0;
-  int ap = 0, op = 0;
-  int32_t pos = dst;
-  auto next_res = [&]() -> int32_t {  // next kept resident in-source (union index), or INT_MAX
-    while (rp < rn) {
-      const int32_t c = rcol[ra + rp];
-      const float v = rval[ra + rp];
-      ++rp;
-      if (res_in_kept(c, v, rout, k1, src, Q)) return c + int32_t(Q);
+  const int32_t* rc = rcol + ra;
+  auto kept_at = [&](int p) { return p < rn && res_in_kept(rc[p], rval[ra + p], rout, k1, src, Q); };
+  int32_t v[2];
+  int lr[2], la[2], below[2] = {0, 0};  // places in the resident row and the added list; kept sources below
+  bool both[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int p = lane + h * kWarp;
+    v[h] = p < k1 ? o[p] : kInvalidIdx;
+    lr[h] = p < k1 ? lower_bound(rc, rn, v[h] - int32_t(Q)) : 0;
+    la[h] = p < k1 ? lower_bound(ad, m, v[h]) : 0;
+    both[h] = p < k1 && la[h] < m && ad[la[h]] == v[h];
+  }
+  for (int c0 = 0; c0 < rn; c0 += kWarp) {
+    const uint32_t kept = __ballot_sync(kFull, kept_at(c0 + lane));
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int q = lr[h] - c0;  // the chunk's entries below v[h]
+      if (q > 0) below[h] += __popc(q < kWarp ? kept & ((1u << q) - 1u) : kept);
+      if (q >= 0 && q < kWarp && ((kept >> q) & 1u) && lane + h * kWarp < k1 && rc[lr[h]] + int32_t(Q) == v[h])
+        both[h] = true;
     }
-    return kInvalidIdx;
-  };
-  int32_t rv = next_res();
-  for (;;) {
-    const int32_t av = ap < m ? ad[ap] : kInvalidIdx;
-    const int32_t iv = rv < av ? rv : av;  // next in-source
-    const int32_t ov = op < k1 ? o[op] : kInvalidIdx;
-    if (iv == kInvalidIdx && ov == kInvalidIdx) break;
-    if (ov == iv) {
-      col[pos] = ov;
-      val[pos] = 1.0f;
-      ++op;
-    } else if (ov < iv) {
-      col[pos] = ov;
-      val[pos] = 0.5f;
-      ++op;
-      ++pos;
-      continue;
-    } else {
-      col[pos] = iv;
-      val[pos] = 0.5f;
+  }
+  const uint64_t common = uint64_t(__ballot_sync(kFull, both[0])) | (uint64_t(__ballot_sync(kFull, both[1])) << 32);
+  auto twice = [&](int p) { return __popcll(common & ((p < 64 ? 1ull << p : 0ull) - 1ull)); };
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int p = lane + h * kWarp;
+    if (p < k1) {
+      const int at = dst + p + below[h] + la[h] - twice(p);
+      col[at] = v[h];
+      val[at] = both[h] ? 1.0f : 0.5f;
     }
-    if (iv == rv) rv = next_res();
-    else ++ap;
-    ++pos;
+  }
+  // In-sources that are no out-neighbours (the common ones are written above).
+  int kb = 0;  // kept sources of the chunks before
+  for (int c0 = 0; c0 < rn; c0 += kWarp) {
+    const bool mine = kept_at(c0 + lane);
+    const uint32_t kept = __ballot_sync(kFull, mine);
+    if (mine) {
+      const int32_t w = rc[c0 + lane] + int32_t(Q);
+      const int p = lower_bound(o, k1, w);
+      if (p == k1 || o[p] != w) {
+        const int at = dst + kb + __popc(kept & ((1u << lane) - 1u)) + lower_bound(ad, m, w) + p - twice(p);
+        col[at] = w;
+        val[at] = 0.5f;
+      }
+    }
+    kb += __popc(kept);
+  }
+  for (int q0 = 0; q0 < m; q0 += kWarp) {
+    const int q = q0 + lane;
+    const int32_t w = q < m ? ad[q] : kInvalidIdx;
+    const int lw = q < m ? lower_bound(rc, rn, w - int32_t(Q)) : 0;
+    int kbelow = 0;
+    for (int c0 = 0; c0 < rn; c0 += kWarp) {
+      const uint32_t kept = __ballot_sync(kFull, kept_at(c0 + lane));
+      const int r = lw - c0;
+      if (r > 0) kbelow += __popc(r < kWarp ? kept & ((1u << r) - 1u) : kept);
+    }
+    if (q < m) {
+      const int p = lower_bound(o, k1, w);
+      if (p == k1 || o[p] != w) {
+        const int at = dst + q + kbelow + p - twice(p);
+        col[at] = w;
+        val[at] = 0.5f;
+      }
+    }
   }
 }
 

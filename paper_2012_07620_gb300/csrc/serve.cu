@@ -219,6 +219,7 @@ size_t slot_layout(const Server& v, Slot* sl, char* base, const Shape& shmax, in
 // Layer-0 marks of a request's union rows (queries first, gallery row g at
 // union row Q + g): h0 changed when the row of A* differs from the gallery
 // graph's, msgchg when the message list (sources or weights) differs.
+constexpr int kMarkLanes = 8;  // a row's k2 + 1 messages are few, its layer-0 entries some dozens
 __global__ void k_mark_h0(int64_t n, int64_t Q, const int64_t* __restrict__ st, const int32_t* __restrict__ ln,
                           const int32_t* __restrict__ cl, const float* __restrict__ vl,
                           const int64_t* __restrict__ rst, const int32_t* __restrict__ rln,
@@ -228,26 +229,31 @@ __global__ void k_mark_h0(int64_t n, int64_t Q, const int64_t* __restrict__ st, 
                           const float* __restrict__ rnbr_w, const int32_t* __restrict__ rnbr_n, int k2p1,
                           const uint8_t* __restrict__ aff, uint8_t* __restrict__ h0chg,
                           uint8_t* __restrict__ msgchg) {
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  if (i < Q) {
-    h0chg[i] = 1;
-    msgchg[i] = 1;
-    return;
+  const int sub = threadIdx.x & (kMarkLanes - 1);
+  const int64_t i = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) / kMarkLanes;
+  if (i >= n) return;  // whole groups
+  const uint32_t group = ((1u << kMarkLanes) - 1u) << (threadIdx.x & (kWarp - kMarkLanes));
+  bool hc = i < Q, mc = i < Q;
+  if (i >= Q) {
+    const int64_t g = i - Q;
+    const int m = nbr_n[i];
+    mc = m != rnbr_n[g];
+    if (!mc)
+      for (int q = sub; q < m; q += kMarkLanes)
+        mc |= nbr[i * k2p1 + q] != rnbr[g * k2p1 + q] + Q || nbr_w[i * k2p1 + q] != rnbr_w[g * k2p1 + q];
+    // Rows the incremental graph did not rebuild (aff clear) are resident copies.
+    const int len = ln[i];
+    hc = len != rln[g];
+    const int64_t a = st[i], ra = rst[g];
+    if ((!aff || aff[i]) && !hc)
+      for (int p = sub; p < len; p += kMarkLanes) hc |= cl[a + p] != rcl[ra + p] + Q || vl[a + p] != rvl[ra + p];
   }
-  const int64_t g = i - Q;
-  const int m = nbr_n[i];
-  bool mc = m != rnbr_n[g];
-  for (int q = 0; q < m && !mc; ++q)
-    mc = nbr[i * k2p1 + q] != rnbr[g * k2p1 + q] + Q || nbr_w[i * k2p1 + q] != rnbr_w[g * k2p1 + q];
-  // Rows the incremental graph did not rebuild (aff clear) are resident copies.
-  const int len = ln[i];
-  bool hc = len != rln[g];
-  const int64_t a = st[i], ra = rst[g];
-  if (!aff || aff[i])
-    for (int p = 0; p < len && !hc; ++p) hc = cl[a + p] != rcl[ra + p] + Q || vl[a + p] != rvl[ra + p];
-  h0chg[i] = hc ? 1 : 0;
-  msgchg[i] = mc ? 1 : 0;
+  hc = __any_sync(group, hc);
+  mc = __any_sync(group, mc);
+  if (sub == 0) {
+    h0chg[i] = hc ? 1 : 0;
+    msgchg[i] = mc ? 1 : 0;
+  }
 }
 
 // Marks of the next layer: a row's output changes when its message list or a
@@ -348,37 +354,53 @@ k_serve_assemble(int64_t G, int64_t Q, int K, int k1, int Pb, const float* __res
     atomicAdd(reinterpret_cast<unsigned long long*>(status + kStTouched), 1ull);
   }
   pos = __shfl_sync(kFull, pos, 0);
-  if (lane != 0) return;
-  // Merge (1 + Pb) sorted lists into the K best by (score desc, index asc).
-  int head[1 + kMaxQueryLists] = {};
+  // Merge (1 + Pb) sorted lists into the K best by (score desc, index asc): an
+  // entry's rank is its place in its own list plus the entries of the other
+  // lists before it (no index occurs twice).  A list ends at its first unused
+  // entry.  By one lane, K rounds over the heads, the merge of the few touched
+  // rows set the kernel's time (52 us for 40,000 rows; the figure after is the
+  // burst's, see k3i_fill).
   const int L = 1 + Pb;
-  for (int e = 0; e < K; ++e) {
-    int best = -1;
-    float bs = -FLT_MAX;
-    int bi = kInvalidIdx;
-    for (int l = 0; l < L; ++l) {
-      if (head[l] >= K) continue;
-      float s;
-      int c;
-      if (l == 0) {
-        s = res_s[size_t(g) * K + head[0]];
-        c = res_i[size_t(g) * K + head[0]];
-        if (c != kInvalidIdx) c += int(Q);
-      } else {
-        const size_t o = (size_t(g) * Pb + (l - 1)) * K + head[l];
-        s = pb_s[o];
-        c = pb_i[o];
-      }
-      if (c == kInvalidIdx) continue;
-      if (best < 0 || ranks_before(s, c, bs, bi)) {
-        best = l;
-        bs = s;
-        bi = c;
+  auto list_s = [&](int l) { return l == 0 ? res_s + size_t(g) * K : pb_s + (size_t(g) * Pb + (l - 1)) * K; };
+  auto list_i = [&](int l) { return l == 0 ? res_i + size_t(g) * K : pb_i + (size_t(g) * Pb + (l - 1)) * K; };
+  int total = 0;
+  for (int l = 0; l < L; ++l) {
+    const int32_t* li = list_i(l);
+    const float* ls = list_s(l);
+    for (int e0 = 0, open = 1; open && e0 < K; e0 += kWarp) {
+      const int e = e0 + lane;
+      const int32_t raw = e < K ? li[e] : kInvalidIdx;
+      const uint32_t used = __ballot_sync(kFull, raw != kInvalidIdx);
+      const int cnt = used == kFull ? kWarp : __ffs(~used) - 1;
+      open = cnt == kWarp;
+      total += cnt;
+      if (lane < cnt) {
+        const float s = ls[e];
+        const int32_t c = l == 0 ? raw + int32_t(Q) : raw;
+        int rank = e;
+        for (int o = 0; o < L && rank < K; ++o) {
+          if (o == l) continue;
+          const int32_t* oi = list_i(o);
+          const float* os = list_s(o);
+          int lo = 0, hi = K;  // the first entry of list o that is unused or not before (s, c)
+          while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            const int32_t x = oi[mid];
+            if (x != kInvalidIdx && ranks_before(os[mid], o == 0 ? x + int(Q) : x, s, c)) lo = mid + 1;
+            else hi = mid;
+          }
+          rank += lo;
+        }
+        if (rank < K) {
+          pm_s[size_t(pos) * K + rank] = s;
+          pm_i[size_t(pos) * K + rank] = c;
+        }
       }
     }
-    if (best >= 0) ++head[best];
-    pm_s[size_t(pos) * K + e] = best >= 0 ? bs : -FLT_MAX;
-    pm_i[size_t(pos) * K + e] = best >= 0 ? bi : kInvalidIdx;
+  }
+  for (int e = total + lane; e < K; e += kWarp) {
+    pm_s[size_t(pos) * K + e] = -FLT_MAX;
+    pm_i[size_t(pos) * K + e] = kInvalidIdx;
   }
 }
 
@@ -568,7 +590,7 @@ rerank_status enqueue_request(Server& v, Slot& sl, const rerank_request& rq, cud
   const unsigned mg = unsigned((n + 255) / 256);
   if (v.reuse) {
     const Server::ResLayer& r0 = v.res_layers[0];
-    k_mark_h0<<<mg, 256, 0, s>>>(n, Q, b.start[2], b.len[2], b.col[2], b.val[2], r0.start, r0.len, r0.col, r0.val,
+    k_mark_h0<<<unsigned((n * kMarkLanes + 255) / 256), 256, 0, s>>>(n, Q, b.start[2], b.len[2], b.col[2], b.val[2], r0.start, r0.len, r0.col, r0.val,
                                  b.nbr, b.nbr_w, b.nbr_n, v.res_nbr, v.res_nbr_w, v.res_nbr_n, k2p1, aff, sl.chg[0],
                                  sl.msgchg);
   }
