@@ -369,6 +369,7 @@ rerank_status enqueue_job(rerank_ctx* ctx, const JobRun& j, cudaStream_t s, Stag
       fm.next = b.row_floor;  // the first pass's floors are done with
       fm.next_K = sh.K;
       fm.skip = true;
+      fm.most_rows = true;
       nl += launch_refine(sh3, dq, dg, b.xhat, b.norm, b.part3_s, b.part3_i, sh.P3g, eh, b.fb_rows, b.fb_count,
                           false, b.knn_idx, b.knn_score, b.fb3_rows, b.fb3_count, status, s, -1, kStFallbackMid, fm);
       nl += launch_gather_rows(b.fb3_rows, b.fb3_count, b.xhi, b.xlo, b.ahi, b.alo, sh.n, sh.dp, s);

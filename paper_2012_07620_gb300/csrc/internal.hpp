@@ -334,12 +334,13 @@ struct ErrModel {
 // next_K entries: the row's next_K-th approximate score less a part of its
 // error bound.  skip: a row that its approximate scores say cannot be
 // certified is passed on without rescoring (only where another list stage
-// follows).
+// follows).  most_rows: a gathered row set that is expected to hold most rows.
 struct RefineFloors {
   const int* in = nullptr;
   int* next = nullptr;
   int next_K = 0;
   bool skip = false;
+  bool most_rows = false;
 };
 // Rows: all n in index order; or rows[0 .. *count) (count == nullptr: n) in that order,
 // with the candidate lists indexed by row (part_by_row) or by position in `rows`.

@@ -484,7 +484,7 @@ k2_refine(RowIo io, int64_t n, const float* __restrict__ part_s, const int32_t* 
 // hold little more than K entries in all), and the serial merge by one warp,
 // K rounds of shuffles behind dependent loads, is left to the rows whose lists
 // hold more than MERGE_CAP: the FP8 recheck at 19,732 x 2048 took 2.91
-// ms with it, 2.73 this way.
+// ms with it, 2.58 this way.
 constexpr int MERGE_CAP = 512;
 struct MergeSmem {
   float s[MERGE_CAP];
@@ -497,8 +497,18 @@ template <int NW>
 __device__ int merge_lists_cta(WarpSmem& w, MergeSmem& m, const float* ls, const int32_t* li, int P, int K,
                                int64_t n, int t, float& B) {
   const int wid = t >> 5, lane = t & 31;
-  // A list ends at its first index outside [0, n) (see merge_lists).
-  for (int p = wid; p < P; p += NW) {
+  // A list ends at its first index outside [0, n) (see merge_lists); most of
+  // the places for lists are not in use (the recheck takes as many chunks as
+  // its row count asks for) and are left out by their first entry.
+  const int32_t first = lane < P ? li[lane * K] : -1;
+  const uint32_t filled = __ballot_sync(kFull, first >= 0 && first < n);
+  const int lists = __popc(filled);
+  auto each_list = [&](auto f) {  // f(list, its place among the filled ones), a warp each
+    int r = 0;
+    for (uint32_t u = filled; u; u &= u - 1u, ++r)
+      if (r % NW == wid) f(__ffs(u) - 1, r);
+  };
+  each_list([&](int p, int r) {
     int L = 0;
     for (int e0 = 0; e0 < K; e0 += kWarp) {
       const int e = e0 + lane;
@@ -507,38 +517,38 @@ __device__ int merge_lists_cta(WarpSmem& w, MergeSmem& m, const float* ls, const
       L += used == kFull ? kWarp : __ffs(~used) - 1;
       if (used != kFull) break;
     }
-    if (lane == 0) m.off[p + 1] = L;
-  }
+    if (lane == 0) m.off[r + 1] = L;
+  });
   __syncthreads();
   if (wid == 0) {
-    int x = lane < P ? m.off[lane + 1] : 0;
+    int x = lane < lists ? m.off[lane + 1] : 0;
 #pragma unroll
     for (int o = 1; o < kWarp; o <<= 1) {
       const int y = __shfl_up_sync(kFull, x, o);
       if (lane >= o) x += y;
     }
-    if (lane < P) m.off[lane + 1] = x;
+    if (lane < lists) m.off[lane + 1] = x;
     if (lane == 0) m.off[0] = 0;
   }
   __syncthreads();
-  const int total = m.off[P];
+  const int total = m.off[lists];
   if (total > MERGE_CAP) return -1;
-  for (int p = wid; p < P; p += NW) {
-    const int o = m.off[p], L = m.off[p + 1] - o;
+  each_list([&](int p, int r) {
+    const int o = m.off[r], L = m.off[r + 1] - o;
     for (int e = lane; e < L; e += kWarp) {
       m.s[o + e] = ls[p * K + e];
       m.i[o + e] = li[p * K + e];
     }
-  }
+  });
   __syncthreads();
   for (int e = t; e < total; e += NW * kWarp) {
     int p = 0;  // the list of entry e: the last that starts at or before it
     for (int step = 16; step; step >>= 1)
-      if (p + step < P && m.off[p + step] <= e) p += step;
+      if (p + step < lists && m.off[p + step] <= e) p += step;
     const float sc = m.s[e];
     const int32_t ic = m.i[e];
     int rank = e - m.off[p];
-    for (int q = 0; q < P && rank < K; ++q) {
+    for (int q = 0; q < lists && rank < K; ++q) {
       if (q == p) continue;
       const int q0 = m.off[q];
       int lo = q0, hi = m.off[q + 1];
@@ -841,8 +851,8 @@ static RowIo make_io(const Shape& sh, const void* xq, const void* xg, const floa
 double rescore_eps(int dp) { return (dp / 32 + 10) * kU32 * 1.01; }
 
 // Rows a launch over a gathered row set covers at once (both kernels loop):
-// about one resident wave on 152 SMs.
-constexpr int64_t kGatheredRows = 2048;
+// one resident wave on 152 SMs (12 CTAs of four warps each).
+constexpr int64_t kGatheredRows = 152 * 12;
 
 // Warps per row of the CTA-per-row refinement (0: warp-per-row kernel).  By
 // default 4 for rows of 512 floats or more, where the warp-per-row kernel's
@@ -868,9 +878,12 @@ int launch_refine(const Shape& sh, const void* xq, const void* xg, const float* 
                    long long* status, cudaStream_t s, int64_t grid_rows, int fb_stat, const RefineFloors& fl) {
   RowIo io = make_io(sh, xq, xg, xhat, norm, knn_idx, knn_score, status);
   int64_t g = grid_rows > 0 && grid_rows < sh.n ? grid_rows : sh.n;
-  // A gathered row set (size on the device): the kernels loop over it, so one
-  // resident wave of rows is enough.
-  if (rows && count) g = std::min<int64_t>(g, kGatheredRows);
+  // A gathered row set (size on the device): the kernels loop over it, and a
+  // set that is expected to be small gets one resident wave.  A wave and a
+  // bit, over a set of nearly all rows, is the worst of grids: the CTAs of the
+  // remainder start when the first wave ends and do as many rows each (2,048
+  // CTAs for 19,732 rows of 2,048: 980 us, one CTA per row 583 us).
+  if (rows && count && !fl.most_rows) g = std::min<int64_t>(g, kGatheredRows);
   const unsigned blocks = unsigned((g + WPB - 1) / WPB);
   // First pass: uncertified rows go to the recheck; a recheck's failures go to the exact scan.
   const int stat = fb_stat >= 0 ? fb_stat : ((rows && !part_by_row) ? kStFallback2 : kStFallback);
