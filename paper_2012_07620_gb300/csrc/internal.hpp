@@ -383,16 +383,18 @@ int launch_graph_incremental(const Shape& sh, const Buffers& b, int64_t Q, const
                              const int32_t* n_touched, const int32_t* res_knn, const int64_t* rst,
                              const int32_t* rln, const int32_t* rcol, const float* rval, uint8_t* aff,
                              uint8_t* src, float alpha, int aggregator, long long* status, cudaStream_t s);
-// Rows of a layer whose output is known elsewhere are copied instead of
-// recomputed (serving: the resident gallery's own layer rows, whose inputs a
-// request left unchanged).  Row i >= shift with changed[i] == 0 copies row
-// i - shift of the compact CSR (rstart, rlen, rcol, rval), columns + shift.
+// Rows of a layer whose output is known elsewhere are neither recomputed nor
+// copied (serving: the resident gallery's own layer rows, whose inputs a
+// request left unchanged).  The rows to compute are listed in rows[0 .. *count);
+// of every other row the caller has written the length and, as a negative
+// number, the place in the resident graph's copy of the layer (~start).
+// src_col / src_val: the resident entries of the source layer's such rows,
+// columns less shift.
 struct LayerReuse {
-  const uint8_t* changed = nullptr;
-  const int64_t* rstart = nullptr;
-  const int32_t* rlen = nullptr;
-  const int32_t* rcol = nullptr;
-  const float* rval = nullptr;
+  const int32_t* rows = nullptr;
+  const int32_t* count = nullptr;
+  const int32_t* src_col = nullptr;
+  const float* src_val = nullptr;
   int64_t shift = 0;
 };
 // Compact copy of a padded-CSR layer (rows 0 .. n-1): cstart = exclusive scan

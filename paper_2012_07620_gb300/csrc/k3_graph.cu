@@ -292,9 +292,9 @@ __global__ void k3i_count(int64_t n, int64_t Q, int k1, const int32_t* __restric
   if (lane == 0) rowcnt[u] = k1 + kept + m - both;
 }
 
-// Rows of A* into the layer-0 CSR: resident rows copied (indices shifted by
-// Q), affected rows as the sorted union of out and in (1 where in both, else
-// 1/2).  An entry's place is its place in its own list, plus the entries of
+// Rows of A* into the layer-0 CSR: resident rows stay where they are (their
+// start is stored as ~rst, see LayerReuse), affected rows as the sorted union
+// of out and in (1 where in both, else 1/2).  An entry's place is its place in its own list, plus the entries of
 // the other two lists below it, less the ones counted twice; the kept resident
 // in-sources are numbered by the ballots of the row's chunks of 32.  Merged by
 // one lane, an affected row's chain of dependent loads lasted longer than the
@@ -315,21 +315,14 @@ __global__ void k3i_fill(int64_t n, int64_t Q, int k1, const uint8_t* __restrict
   if (u >= n) return;
   const int32_t dst = h0ptr[u];
   if (lane == 0) {
-    start[u] = dst;
+    start[u] = aff[u] ? int64_t(dst) : ~rst[u - Q];
     len[u] = h0ptr[u + 1] - dst;
     if (u == n - 1) {
       start[n] = h0ptr[n];
       if (nnz0) *nnz0 = h0ptr[n];
     }
   }
-  if (!aff[u]) {
-    const int64_t g = u - Q, ra = rst[g];
-    for (int p = lane; p < rln[g]; p += kWarp) {
-      col[dst + p] = rcol[ra + p] + int32_t(Q);
-      val[dst + p] = rval[ra + p];
-    }
-    return;
-  }
+  if (!aff[u]) return;
   const int32_t* o = out_sorted + u * k1;
   const int32_t a = add_ptr[u];
   const int m = add_ptr[u + 1] - a;

@@ -119,16 +119,37 @@ __device__ __forceinline__ int next_pow2(int x) {
   return p;
 }
 
+// Rows of a source layer.  With RES, a row whose start is negative lies in the
+// resident graph's copy of the layer, at ~start, its columns less `shift`.
+struct SrcRows {
+  const int64_t* start;
+  const int32_t* len;
+  const int32_t* col;
+  const float* val;
+  const int32_t* rcol;
+  const float* rval;
+  int32_t shift;
+};
+template <bool RES>
+__device__ __forceinline__ void src_entry(const SrcRows& S, int64_t a, int e, int& col, float& val) {
+  if (RES && a < 0) {
+    col = __ldg(S.rcol + ~a + e) + S.shift;
+    val = __ldg(S.rval + ~a + e);
+  } else {
+    col = S.col[a + e];
+    val = S.val[a + e];
+  }
+}
+
 constexpr int kMaxPropWarps = 24;  // 24 warps x 4 KB of tables: 96 KB per CTA
 
 // Row i through one warp's SLOTS-entry table (keys / vals: empty on entry and
 // on return); o: its place in the output.  Returns false when the row was written (lane 0 adds its length
 // to nnz), true when its distinct columns filled three quarters of the table:
 // then nothing is written and the caller hands the row on.
-template <int SLOTS>
-__device__ bool warp_row(int64_t i, int u, volatile int* keys, float* vals, const int64_t* __restrict__ sstart,
-                         const int32_t* __restrict__ slen, const int32_t* __restrict__ scol,
-                         const float* __restrict__ sval, const int32_t* __restrict__ nbr,
+template <int SLOTS, bool RES>
+__device__ bool warp_row(int64_t i, int u, volatile int* keys, float* vals, const SrcRows& S,
+                         const int32_t* __restrict__ nbr,
                          const float* __restrict__ nbr_w, const int32_t* __restrict__ nbr_n, int k2p1,
                          int64_t o, int32_t* __restrict__ dlen, int32_t* __restrict__ dcol,
                          float* __restrict__ dval, float* __restrict__ rn, long long* __restrict__ status,
@@ -154,14 +175,17 @@ __device__ bool warp_row(int64_t i, int u, volatile int* keys, float* vals, cons
     for (int q = 0; q < m && !spilled; ++q) {
       const int32_t j = nbr[i * k2p1 + q];
       const float cj = nbr_w[i * k2p1 + q];
-      const int64_t a = sstart[j];
-      const int lj = slen[j];
+      const int64_t a = S.start[j];
+      const int lj = S.len[j];
       for (int e0 = 0; e0 < lj; e0 += kWarp) {
         const int e = e0 + lane;
         bool fresh = false;
-        if (e < lj)
-          fresh = hash_add(keys, vals, mask, shift, scol[a + e], fabsf(cj) * sval[a + e], status,
-                           agg_max && cj >= 0.f);
+        if (e < lj) {
+          int c;
+          float v;
+          src_entry<RES>(S, a, e, c, v);
+          fresh = hash_add(keys, vals, mask, shift, c, fabsf(cj) * v, status, agg_max && cj >= 0.f);
+        }
         distinct += __popc(__ballot_sync(kFull, fresh));
         __syncwarp();
         if (distinct > limit) {
@@ -175,8 +199,8 @@ __device__ bool warp_row(int64_t i, int u, volatile int* keys, float* vals, cons
   if (lane < mq) {
     const int32_t j = nbr[i * k2p1 + lane];
     qc = nbr_w[i * k2p1 + lane];
-    qa = sstart[j];
-    ql = slen[j];
+    qa = S.start[j];
+    ql = S.len[j];
   }
   int q = 0, e0 = 0;
   while (q < mq && __shfl_sync(kFull, ql, q) == 0) ++q;
@@ -185,10 +209,7 @@ __device__ bool warp_row(int64_t i, int u, volatile int* keys, float* vals, cons
   if (q < mq) {
     const int64_t a = __shfl_sync(kFull, qa, q);
     const int lj = __shfl_sync(kFull, ql, q);
-    if (lane < lj) {
-      col = scol[a + lane];
-      val = sval[a + lane];
-    }
+    if (lane < lj) src_entry<RES>(S, a, lane, col, val);
   }
   while (q < mq) {
     // next step: (q, e0 + 32) or the next non-empty message
@@ -203,10 +224,7 @@ __device__ bool warp_row(int64_t i, int u, volatile int* keys, float* vals, cons
     if (nq < mq) {
       const int64_t a = __shfl_sync(kFull, qa, nq);
       const int lj = __shfl_sync(kFull, ql, nq);
-      if (ne0 + lane < lj) {
-        ncol = scol[a + ne0 + lane];
-        nval = sval[a + ne0 + lane];
-      }
+      if (ne0 + lane < lj) src_entry<RES>(S, a, ne0 + lane, ncol, nval);
     }
     const float cj = __shfl_sync(kFull, qc, q);
     bool fresh = false;
@@ -278,9 +296,9 @@ __device__ bool warp_row(int64_t i, int u, volatile int* keys, float* vals, cons
 
 // First pass: warp per row, 512-slot tables; rows that overflow them, or
 // whose bound is above WDIRECT, are listed in big_rows for k4_spmm_rest.
+template <bool RES>
 __global__ void __launch_bounds__(kMaxPropWarps * kWarp)
-k4_spmm_warp(const int64_t* __restrict__ sstart, const int32_t* __restrict__ slen, const int32_t* __restrict__ scol,
-             const float* __restrict__ sval, const int32_t* __restrict__ nbr, const float* __restrict__ nbr_w,
+k4_spmm_warp(SrcRows S, const int32_t* __restrict__ nbr, const float* __restrict__ nbr_w,
              const int32_t* __restrict__ nbr_n, int k2p1, int32_t* __restrict__ ub, int64_t* dstart,
              int32_t* __restrict__ dlen, int32_t* __restrict__ dcol, float* __restrict__ dval,
              float* __restrict__ rn, int64_t n, int64_t cap, int32_t* __restrict__ big_rows,
@@ -301,20 +319,18 @@ k4_spmm_warp(const int64_t* __restrict__ sstart, const int32_t* __restrict__ sle
   // Rows are taken one at a time from a counter: their cost varies with the
   // length of their message rows, and a static split left the busiest SM
   // with twice the average work (market, second layer).
+  // With RES only the listed rows are computed.
+  const int64_t limit = RES ? int64_t(*reuse.count) : n;
   for (;;) {
     int64_t i = 0;
     if (lane == 0) i = atomicAdd(next_row, 1);
     i = __shfl_sync(kFull, i, 0);
-    if (i >= n) break;
-    const bool known = reuse.changed && !reuse.changed[i];
-    // The row's place: room for the sum of its messages' lengths (or the known row).
+    if (i >= limit) break;
+    if (RES) i = reuse.rows[i];
+    // The row's place: room for the sum of its messages' lengths.
     long long u64 = 0;
-    if (known) {
-      u64 = lane == 0 ? reuse.rlen[i - reuse.shift] : 0;
-    } else {
-      const int m = nbr_n[i];
-      for (int q = lane; q < m; q += kWarp) u64 += slen[nbr[i * k2p1 + q]];
-    }
+    const int m = nbr_n[i];
+    for (int q = lane; q < m; q += kWarp) u64 += S.len[nbr[i * k2p1 + q]];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) u64 += __shfl_xor_sync(kFull, u64, o);
     if (u64 > n) u64 = n;
@@ -336,22 +352,8 @@ k4_spmm_warp(const int64_t* __restrict__ sstart, const int32_t* __restrict__ sle
       ub[i] = u;
     }
     __syncwarp();
-    if (known) {
-      // inputs unchanged: the known row, in its own column order
-      const int64_t g = i - reuse.shift, a = reuse.rstart[g], o = off;
-      const int m = reuse.rlen[g];
-      for (int p = lane; p < m; p += kWarp) {
-        dcol[o + p] = int32_t(reuse.rcol[a + p] + reuse.shift);
-        dval[o + p] = reuse.rval[a + p];
-      }
-      if (lane == 0) {
-        dlen[i] = m;
-        nnz += unsigned(m);
-      }
-      continue;
-    }
-    const bool handed = u > WDIRECT || warp_row<WSLOTS>(i, u, keys, vals, sstart, slen, scol, sval, nbr, nbr_w, nbr_n,
-                                                        k2p1, off, dlen, dcol, dval, rn, status, agg_max, lane, nnz);
+    const bool handed = u > WDIRECT || warp_row<WSLOTS, RES>(i, u, keys, vals, S, nbr, nbr_w, nbr_n, k2p1, off, dlen,
+                                                             dcol, dval, rn, status, agg_max, lane, nnz);
     if (handed && lane == 0)
       big_rows[atomicAdd(big_count, 1)] = int32_t(i);
   }
@@ -362,9 +364,8 @@ k4_spmm_warp(const int64_t* __restrict__ sstart, const int32_t* __restrict__ sle
 // of touched columns in this CTA's part of the global scratch; messages in
 // order (one barrier each), the bitmap scan emits the columns in ascending
 // order, and the norm is the exact fixed-point sum of warp_row.
-__device__ void cta_row(int64_t i, const int64_t* __restrict__ sstart, const int32_t* __restrict__ slen,
-                        const int32_t* __restrict__ scol, const float* __restrict__ sval,
-                        const int32_t* __restrict__ nbr, const float* __restrict__ nbr_w,
+template <bool RES>
+__device__ void cta_row(int64_t i, const SrcRows& S, const int32_t* __restrict__ nbr, const float* __restrict__ nbr_w,
                         const int32_t* __restrict__ nbr_n, int k2p1, const int64_t* __restrict__ dstart,
                         int32_t* __restrict__ dlen, int32_t* __restrict__ dcol, float* __restrict__ dval, int64_t n,
                         float* __restrict__ rn, float* __restrict__ acc, uint32_t* __restrict__ bm, bool agg_max,
@@ -378,11 +379,13 @@ __device__ void cta_row(int64_t i, const int64_t* __restrict__ sstart, const int
   for (int q = 0; q < m; ++q) {
     const int32_t j = nbr[i * k2p1 + q];
     const float cj = nbr_w[i * k2p1 + q];
-    const int64_t a = sstart[j];
-    const int lj = slen[j];
+    const int64_t a = S.start[j];
+    const int lj = S.len[j];
     for (int e = tid; e < lj; e += RTHREADS) {
-      const int c = scol[a + e];
-      const float v = fabsf(cj) * sval[a + e];
+      int c;
+      float v;
+      src_entry<RES>(S, a, e, c, v);
+      v *= fabsf(cj);
       acc[c] = (agg_max && cj >= 0.f) ? fmaxf(acc[c], v) : acc[c] + v;
       atomicOr(&bm[c >> 5], 1u << (c & 31));
     }
@@ -460,9 +463,9 @@ __device__ void cta_row(int64_t i, const int64_t* __restrict__ sstart, const int
 // could not hold (flagged in spill[], indexed like big_rows) with cta_row;
 // with fewer, every listed row goes to cta_row, which is faster for a few rows.
 // Every path gives the same values, bit for bit.
+template <bool RES>
 __global__ void __launch_bounds__(RTHREADS)
-k4_spmm_rest(const int64_t* __restrict__ sstart, const int32_t* __restrict__ slen, const int32_t* __restrict__ scol,
-             const float* __restrict__ sval, const int32_t* __restrict__ nbr, const float* __restrict__ nbr_w,
+k4_spmm_rest(SrcRows S, const int32_t* __restrict__ nbr, const float* __restrict__ nbr_w,
              const int32_t* __restrict__ nbr_n, int k2p1, const int32_t* __restrict__ ub,
              const int32_t* __restrict__ big_rows, const int32_t* __restrict__ big_count, int min_rows,
              int32_t* __restrict__ spill, const int64_t* __restrict__ dstart, int32_t* __restrict__ dlen,
@@ -489,16 +492,16 @@ k4_spmm_rest(const int64_t* __restrict__ sstart, const int32_t* __restrict__ sle
     __syncwarp();
     for (int64_t f = int64_t(blockIdx.x) * RWARPS + wib; f < count; f += int64_t(gridDim.x) * RWARPS) {
       const int64_t i = big_rows[f];
-      const bool sp = warp_row<MSLOTS>(i, ub[i], keys, vals, sstart, slen, scol, sval, nbr, nbr_w, nbr_n, k2p1,
-                                       dstart[i], dlen, dcol, dval, rn, status, agg_max, lane, nnz);
+      const bool sp = warp_row<MSLOTS, RES>(i, ub[i], keys, vals, S, nbr, nbr_w, nbr_n, k2p1, dstart[i],
+                                            dlen, dcol, dval, rn, status, agg_max, lane, nnz);
       if (lane == 0) spill[f] = sp ? 1 : 0;
     }
     __syncthreads();  // this CTA's flags are written
     for (int64_t f0 = int64_t(blockIdx.x) * RWARPS; f0 < count; f0 += int64_t(gridDim.x) * RWARPS)
       for (int w = 0; w < RWARPS && f0 + w < count; ++w)
         if (spill[f0 + w])
-          cta_row(big_rows[f0 + w], sstart, slen, scol, sval, nbr, nbr_w, nbr_n, k2p1, dstart, dlen, dcol, dval, n,
-                  rn, acc, bm, agg_max, scan_s, red_hi, red_lo, nnz);
+          cta_row<RES>(big_rows[f0 + w], S, nbr, nbr_w, nbr_n, k2p1, dstart, dlen, dcol, dval, n, rn, acc, bm,
+                       agg_max, scan_s, red_hi, red_lo, nnz);
   } else {
     // The tables are not needed: when the dense accumulator and its bitmap fit
     // the shared memory (n up to ~47,000), they live there (zeroed once; every
@@ -512,8 +515,8 @@ k4_spmm_rest(const int64_t* __restrict__ sstart, const int32_t* __restrict__ sle
       __syncthreads();
     }
     for (int64_t f = blockIdx.x; f < count; f += gridDim.x)
-      cta_row(big_rows[f], sstart, slen, scol, sval, nbr, nbr_w, nbr_n, k2p1, dstart, dlen, dcol, dval, n, rn, a2, b2,
-              agg_max, scan_s, red_hi, red_lo, nnz);
+      cta_row<RES>(big_rows[f], S, nbr, nbr_w, nbr_n, k2p1, dstart, dlen, dcol, dval, n, rn, a2, b2, agg_max, scan_s,
+                   red_hi, red_lo, nnz);
   }
   if (nnz_out && lane == 0 && nnz) atomicAdd(nnz_out, nnz);
 }
@@ -564,18 +567,13 @@ int launch_propagate(const Shape& sh, const Buffers& b, int src, int dst, int ag
   // [0]: rows handed on, [1]: next row of the first pass, [2, 3]: the place cursor
   cudaMemsetAsync(b.big_count, 0, 4 * sizeof(int32_t), s);
   const LayerReuse ru = reuse ? *reuse : LayerReuse{};
+  const SrcRows S{b.start[src], b.len[src], b.col[src], b.val[src], ru.src_col, ru.src_val, int32_t(ru.shift)};
   const int warps = t.prop_warps < 1 ? 1 : (t.prop_warps > kMaxPropWarps ? kMaxPropWarps : t.prop_warps);
   const size_t smem = size_t(warps) * WSLOTS * 2 * sizeof(int);
-  cudaFuncSetAttribute(k4_spmm_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   const int64_t blocks_needed = (n + warps - 1) / warps;
   const int per_sm = smem ? int((227 * 1024) / smem) : 1;
   const unsigned blocks = unsigned(tmin<int64_t>(blocks_needed, int64_t(sm_count) * (per_sm > 0 ? per_sm : 1)));
-  k4_spmm_warp<<<blocks, warps * kWarp, smem, s>>>(b.start[src], b.len[src], b.col[src], b.val[src], b.nbr, b.nbr_w,
-                                                   b.nbr_n, k2p1, b.ub, b.start[dst], b.len[dst], b.col[dst],
-                                                   b.val[dst], rnorm, n, sh.cap_h, b.big_rows, b.big_count,
-                                                   b.big_count + 1,
-                                                   reinterpret_cast<unsigned long long*>(b.big_count + 2), status,
-                                                   aggregator == RERANK_AGG_MAX, ru, nnz_out);
+  const bool agg_max = aggregator == RERANK_AGG_MAX;
   // The rows the first pass listed: 2,048-slot tables when there are at least
   // 4 per SM (market_hard: 21,906 rows, propagation 2.20 -> 1.13 ms), else the
   // CTA path (market: 549 rows, faster there).
@@ -585,12 +583,21 @@ int launch_propagate(const Shape& sh, const Buffers& b, int src, int dst, int ag
   }();
   const int min_rows = min_override >= 0 ? min_override : 4 * sm_count;
   const size_t rsmem = size_t(RWARPS) * MSLOTS * 2 * sizeof(int);
-  cudaFuncSetAttribute(k4_spmm_rest, cudaFuncAttributeMaxDynamicSharedMemorySize, int(rsmem));
-  k4_spmm_rest<<<sm_count, RTHREADS, rsmem, s>>>(
-      b.start[src], b.len[src], b.col[src], b.val[src], b.nbr, b.nbr_w, b.nbr_n, k2p1, b.ub, b.big_rows, b.big_count,
-      min_rows, b.prop_spill, b.start[dst], b.len[dst], b.col[dst], b.val[dst], rnorm, n, b.hash_keys_vals,
-      reinterpret_cast<uint32_t*>(b.hash_keys_vals + size_t(sm_count) * n), status, aggregator == RERANK_AGG_MAX,
-      nnz_out);
+  auto go = [&](auto first, auto rest) {
+    cudaFuncSetAttribute(first, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    first<<<blocks, warps * kWarp, smem, s>>>(S, b.nbr, b.nbr_w, b.nbr_n, k2p1, b.ub, b.start[dst], b.len[dst],
+                                              b.col[dst], b.val[dst], rnorm, n, sh.cap_h, b.big_rows, b.big_count,
+                                              b.big_count + 1,
+                                              reinterpret_cast<unsigned long long*>(b.big_count + 2), status, agg_max,
+                                              ru, nnz_out);
+    cudaFuncSetAttribute(rest, cudaFuncAttributeMaxDynamicSharedMemorySize, int(rsmem));
+    rest<<<sm_count, RTHREADS, rsmem, s>>>(
+        S, b.nbr, b.nbr_w, b.nbr_n, k2p1, b.ub, b.big_rows, b.big_count, min_rows, b.prop_spill, b.start[dst],
+        b.len[dst], b.col[dst], b.val[dst], rnorm, n, b.hash_keys_vals,
+        reinterpret_cast<uint32_t*>(b.hash_keys_vals + size_t(sm_count) * n), status, agg_max, nnz_out);
+  };
+  if (ru.rows) go(k4_spmm_warp<true>, k4_spmm_rest<true>);
+  else go(k4_spmm_warp<false>, k4_spmm_rest<false>);
   return 2;
 }
 
