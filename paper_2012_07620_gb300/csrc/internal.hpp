@@ -376,9 +376,9 @@ int launch_graph(const Shape& sh, const Buffers& b, float alpha, int aggregator,
 // A serving request's graph (A* features) from the resident gallery graph:
 // only rows whose A* row can change (the queries, the touched gallery rows
 // touched[0 .. *n_touched) and the old and new targets of their lists) are
-// built; the others are the resident rows (rst / rln / rcol / rval, gallery
-// indices) shifted by Q.  aff / src: n bytes of scratch each.  Same CSR,
-// message lists and nnz counter as launch_graph.
+// built; the others stay in the resident graph (rst / rln / rcol / rval, gallery
+// indices): their start is ~rst, see LayerReuse.  aff / src: n bytes of scratch
+// each.  Same rows, message lists and nnz counter as launch_graph.
 int launch_graph_incremental(const Shape& sh, const Buffers& b, int64_t Q, const int32_t* touched,
                              const int32_t* n_touched, const int32_t* res_knn, const int64_t* rst,
                              const int32_t* rln, const int32_t* rcol, const float* rval, uint8_t* aff,

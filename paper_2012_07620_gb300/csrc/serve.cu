@@ -58,7 +58,6 @@ double ms_between(Clock::time_point a, Clock::time_point b) {
 
 constexpr int kMaxSlots = 8;
 constexpr int64_t kMaxQuery = 1024;  // query columns of a request: at most 4 tiles of 256
-constexpr int kMaxQueryLists = 8;    // lists per gallery row against the queries: 4 chunks x 2
 constexpr int64_t kPad = 256;  // zero rows after the gallery: one full tensor-core tile
 
 struct Server;
