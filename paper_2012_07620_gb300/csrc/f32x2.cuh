@@ -18,6 +18,11 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 // a - b: the product by -1 is exact, so the rounding is the subtraction's.
 __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
   constexpr f32x2 minus_one = 0xbf800000bf800000ull;

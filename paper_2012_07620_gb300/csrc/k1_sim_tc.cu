@@ -1,6 +1,13 @@
 // K1b: similarity S = Xhat Xhat^T (Eq. 7) on the 5th-generation tensor cores
-// (BF16 or FP8-E4M3 operands, FP32 accumulation in TMEM) with a fused per-row
-// top-K (Eq. 8).  S never leaves the SM.
+// (BF16 or FP8-E4M3 operands, FP32 accumulation in TMEM) with the selection of
+// each row's K best columns (Eq. 8).  S never leaves the SM.
+//
+// The main path is three kernels.  A sampling pass scores every row against a
+// few hundred columns and keeps a rank of them as the row's floor; the append
+// pass (CTA pairs, 16 epilogue warps) computes the whole square and appends the
+// columns that reach a row's floor to its segments; k_select sorts out the K best.
+// The list kernels, whose epilogue keeps a sorted list per row, serve the
+// rechecks, a request's gallery rows, single CTAs and tight budgets:
 //
 // One persistent CTA per SM walks work items (row block of 128 rows, chunk of
 // 256-column tiles); items are ordered so that CTAs running together share
@@ -17,7 +24,9 @@
 //                        reads its 256 scores with tcgen05.ld (32 at a time),
 //                        applies the FP8 row/column scales, sets S_ii = 1 and
 //                        admits the columns that beat the row's threshold into
-//                        its sorted top-K list; then releases the accumulator.
+//                        its sorted top-K list; then releases the accumulator
+//                        (pairs: the lists are in shared memory, merged by the
+//                        whole warp).
 // The two accumulators let the MMA of tile t+1 run under the epilogue of
 // tile t.  At the end of a work item the list is written as one
 // partial candidate list per (row, chunk), merged and certified by K2.
@@ -36,6 +45,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "f32x2.cuh"
 #include "internal.hpp"
 #include "tc_ptx.cuh"
 #include "topk_heap.cuh"  // score_key / key_score
@@ -758,6 +768,8 @@ __device__ __forceinline__ bool epilogue_append(Smem& sm, const CUtensorMap* pA0
     // s >= floor, i.e. s > the float below it
     float thr = live ? nextafterf(key_score(__ldg(it.row_floor + arow)), -INFINITY) : INFINITY;
     const float rinv = (MODE == MODE_FP8 && live) ? it.inv_scale[arow] : 1.0f;
+    const f32x2 rinv2 = twice(rinv);
+    const bool wide = MODE == MODE_FP8 && (reinterpret_cast<uintptr_t>(it.inv_scale) & 15) == 0;
     const size_t seg = size_t(live ? arow : 0) * (it.chunks * AEG) + it.chunk * AEG + eg;
     const uint64_t p0 = reinterpret_cast<uint64_t>(it.cand + seg * it.cap);
     const uint64_t plast = p0 + 8u * (it.cap - 32);  // beyond it a batch might not fit
@@ -788,11 +800,29 @@ __device__ __forceinline__ bool epilogue_append(Smem& sm, const CUtensorMap* pA0
       auto fold = [&](uint32_t (&v)[32], int h) {
         const int lb = h * 32;
         if (MODE == MODE_FP8) {
+          // Both rows' scales, in packed products of two columns with the scales
+          // loaded by fours where they are aligned (a request's may not be):
+          // similarity stage at Market 0.88 -> 0.82 ms (bounding a tile's scores
+          // by its largest scale first gained nothing: most groups of four hold
+          // a candidate of some row).
           const float* si = it.inv_scale + c0 + lb;
-          const int nv = int(tmin<int64_t>(it.n - c0 - lb, 32));
+          if (!patch && wide) {
 #pragma unroll
-          for (int j = 0; j < 32; ++j)
-            v[j] = __float_as_uint(__uint_as_float(v[j]) * rinv * __ldg(j < nv ? si + j : it.inv_scale));
+            for (int j = 0; j < 32; j += 4) {
+              const ulonglong2 f = __ldg(reinterpret_cast<const ulonglong2*>(si + j));
+              const f32x2 a = mul2(mul2(f32x2(v[j]) | (f32x2(v[j + 1]) << 32), rinv2), f.x);
+              const f32x2 b = mul2(mul2(f32x2(v[j + 2]) | (f32x2(v[j + 3]) << 32), rinv2), f.y);
+              v[j] = uint32_t(a);
+              v[j + 1] = uint32_t(a >> 32);
+              v[j + 2] = uint32_t(b);
+              v[j + 3] = uint32_t(b >> 32);
+            }
+          } else {
+            const int nv = int(tmin<int64_t>(it.n - c0 - lb, 32));
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              v[j] = __float_as_uint(__uint_as_float(v[j]) * rinv * __ldg(j < nv ? si + j : it.inv_scale));
+          }
         }
         if (patch) {
           // the diagonal (S_ii = 1) and the columns past the last one

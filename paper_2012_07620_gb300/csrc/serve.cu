@@ -20,8 +20,8 @@
 //      stages, as in rerank_run, on X_u; a propagation layer recomputes only
 //      the rows whose inputs differ from the gallery's own graph (G alone,
 //      computed at load): a row whose message list and whose sources' rows of
-//      the previous layer are unchanged gets the resident row, columns shifted
-//      by Q.  Its values are those of a recomputation (each column is summed
+//      the previous layer are unchanged is the resident row, read where it lies
+//      with columns shifted by Q.  Its values are those of a recomputation (each column is summed
 //      in message order, norms are exact), only their order in the row differs.
 // Every slot owns a stream and all the buffers of one request, so requests
 // on different slots overlap on the GPU and never see each other's data.
