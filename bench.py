@@ -246,12 +246,12 @@ def _config(args, w):
             "l2": "flushed before every step (256 MiB write)", "parallelism": f"replicas x{args.gpus}"}
 
 
-# DRAM bytes (read + write) of one similarity launch, from `ncu --set full` captures
-# of the current kernel (profiles/); None where no capture of it exists.
-SIM_TRAFFIC_BYTES = {("bf16", "market"): 314.9e6}  # profiles/k1_tc2_topk_bf16_market_23k_d2048.md
-# DRAM bytes of the refinement's first pass, same source
+# DRAM bytes (read + write) of one similarity launch, from ncu captures of the
+# current kernel (profiles/); None where no capture of it exists.
+SIM_TRAFFIC_BYTES = {("bf16", "market"): 996.1e6}  # profiles/k1_tc2_append_bf16_market_23k_d2048.md
+# DRAM bytes read by the refinement's first pass, same source
 # (profiles/k2_refine_cta_bf16_market_23k_d2048.md).
-REFINE_DRAM_BYTES = {("bf16", "market"): 1.682e9}
+REFINE_DRAM_BYTES = {("bf16", "market"): 1.640e9}
 
 
 def _stage_rooflines(precision, stages, nq, ng, d, k1, k2, rescore_m, h_nnz, layers, workload):
@@ -297,10 +297,12 @@ def _stage_rooflines(precision, stages, nq, ng, d, k1, k2, rescore_m, h_nnz, lay
 
 
 def _roofline(precision, sim_ms, n, d, workload):
-    """Roofline of the dominant kernel, the similarity GEMM with its fused top-K:
-    2 n^2 d flops per launch (the full square; the kernel computes every tile)."""
+    """Roofline of the dominant stage, the similarity GEMM with the selection of
+    the K best: 2 n^2 d flops (the full square; the tensor-core kernel computes
+    every tile), for FP32 n (n + 1) d (the symmetric matrix: every pair once,
+    as long as it fits 16 GB, n <= 65,536)."""
     peaks, which = _peaks()
-    flops = 2.0 * n * n * d
+    flops = float(n) * (n + 1) * d if precision == "fp32" and n <= 65536 else 2.0 * n * n * d
     achieved = flops / (sim_ms * 1e-3) / 1e12
     if precision == "fp32":
         mhz = peaks.get("sm_max_mhz", 2070.0)
@@ -313,7 +315,7 @@ def _roofline(precision, sim_ms, n, d, workload):
                 "peak_source": f"{which} bf16 burst" + (" x2 (fp8 nominal ratio)" if precision == "fp8" else "")}
     roof["frac"] = achieved / peak
     roof["traffic"] = SIM_TRAFFIC_BYTES.get((precision, workload))
-    roof["kernel"] = "similarity_topk (k1_tc_topk / k1_sim_fp32)"
+    roof["kernel"] = "similarity_topk (k1_tc2_append + k_select / k1_sgemm_sym + k1_select_rows)"
     roof["flops_per_launch"] = flops
     return roof
 
