@@ -6,6 +6,8 @@ in place for every aggregator, feature and depth."""
 import numpy as np
 import pytest
 
+import parity
+from oracle import rerank_oracle as o
 from paper_2012_07620_gb300 import synthetic
 
 pytestmark = pytest.mark.gpu
@@ -114,3 +116,15 @@ def test_served_rows_in_place(lib, layers, aggregator, feature, k1, k2):
             assert np.abs(sd.astype(np.float64) - fd).max() <= 1e-6
             differ = si != fi
             assert np.all(np.abs(sd[differ].astype(np.float64) - fd[differ]) <= 1e-6)
+
+
+@pytest.mark.parametrize("ng", [8191, 8192, 8200])
+def test_column_lists_by_cta_equal_the_oracle(lib, ng):
+    """The gallery's column lists from 8,192 rows up are counted per CTA."""
+    spec = synthetic.WorkloadSpec("columns", 12, ng, 64, 400, 0.35, 0, None, seed=7)
+    w = synthetic.make_workload(spec)
+    ref = o.rerank(w.xq, w.xg, k1=20, k2=5, layers=2, mode="sparse")
+    with lib.Reranker(device=0, precision="bf16") as R:
+        idx, dist = R.run(torch.from_numpy(w.xq).cuda(), torch.from_numpy(w.xg).cuda(), 20, 5, 2)
+        torch.cuda.synchronize()
+    parity.assert_ranked_equal(idx.cpu().numpy(), dist.cpu().numpy(), ref.s, ref.idx)
