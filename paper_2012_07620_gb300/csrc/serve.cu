@@ -773,6 +773,7 @@ rerank_status build_resident_graph(Server& v, cudaStream_t s0, long long* gst, s
   sg.k2 = v.k2;
   sg.layers = v.layers;
   sg.cap_h = v.cap_h;
+  sg.rank_ctas = ctx->sm_count;
   sg.tune = lookup_tuning(ctx, v.prec, G, v.d);
   const size_t e1 = size_t(G) * size_t(v.k1), k2p1 = size_t(v.k2) + 1;
   copy_rows(b.knn_idx, v.res_knn_idx, e1 * 4, s0);

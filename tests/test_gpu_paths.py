@@ -128,3 +128,23 @@ def test_column_lists_by_cta_equal_the_oracle(lib, ng):
         idx, dist = R.run(torch.from_numpy(w.xq).cuda(), torch.from_numpy(w.xg).cuda(), 20, 5, 2)
         torch.cuda.synchronize()
     parity.assert_ranked_equal(idx.cpu().numpy(), dist.cpu().numpy(), ref.s, ref.idx)
+
+
+@pytest.mark.parametrize("ng", [8191, 8192])
+def test_gallery_column_lists_at_load(lib, ng):
+    """The resident graph's column lists, built at load, from 8,192 rows up per CTA."""
+    spec = synthetic.WorkloadSpec("load_columns", 0, ng, 64, 400, 0.35, 0, None, seed=9)
+    w = synthetic.make_workload(spec)
+    xg = torch.from_numpy(w.xg).cuda()
+    q = torch.from_numpy(synthetic.request_queries(w, 3, 5)).cuda()
+    with lib.Reranker(precision="bf16") as R, lib.Reranker(precision="bf16") as F:
+        R.load_gallery(xg, max_query=16, k1=20, k2=5, layers=2, slots=2)
+        t, si, sd = R.submit(q, 0)
+        assert R.wait(t, 120000) is not None
+        assert R.serve_info()["reuse_layers"] == 1
+        fi, fd = F.run(q, xg, 20, 5, 2)
+        torch.cuda.synchronize()
+        si, sd, fi, fd = (v.cpu().numpy() for v in (si, sd, fi, fd))
+    assert np.abs(sd.astype(np.float64) - fd).max() <= 1e-6
+    differ = si != fi
+    assert np.all(np.abs(sd[differ].astype(np.float64) - fd[differ]) <= 1e-6)
