@@ -282,7 +282,8 @@ __device__ __forceinline__ void add_column(const int2* __restrict__ e, int n, fl
 // call with in = false), x the product in fixed point (2^31 is exact, so it is
 // folded into the query's value).  Warp w of nw takes entries w, w + nw, ...; the
 // next entry's column bounds are loaded while the current column is added.
-// stop(): true ends the warp's work.
+// stop(): true ends the warp's work.  add() and stop() are called by whole warps
+// and vote across them, so stop() has to answer every lane of a warp alike.
 template <class Add, class Stop>
 __device__ __forceinline__ void add_products(const RankArgs& A, int64_t q, int w, int nw, int lane, Add add,
                                              Stop stop) {
@@ -437,6 +438,8 @@ __global__ void __launch_bounds__(NTH, 1024 / NTH) k6_rank_light(RankArgs A) {
   __syncthreads();
   auto place = [&](int b) { return int((S.hist[b >> 1] >> (16 * (b & 1))) & 0xffffu); };
   for (int64_t q = A.q_begin + blockIdx.x; q < A.q_end; q += gridDim.x) {
+    // Other warps raise the count while this one reads it: one lane's reading
+    // decides for the warp, or some lanes could leave the votes of add() to the others.
     volatile int* const vcnt = &S.cnt;
     add_products(
         A, q, w, NW, lane,
@@ -451,7 +454,7 @@ __global__ void __launch_bounds__(NTH, 1024 / NTH) k6_rank_light(RankArgs A) {
             if (fresh && at < LCAP) S.list[at] = uint16_t(r);
           }
         },
-        [&] { return *vcnt > LCAP; });  // handed on: what follows does not count
+        [&] { return __shfl_sync(kFull, *vcnt, 0) > LCAP; });  // handed on: what follows does not count
     __syncthreads();
     int cnt = S.cnt;
     bool over = cnt > LCAP;
