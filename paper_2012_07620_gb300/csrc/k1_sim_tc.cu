@@ -368,6 +368,14 @@ __device__ __forceinline__ int next_item(Smem& sm, const TcArgs& A, bool publish
   return it;
 }
 
+// A whole warp waits for an accumulator.  The lanes' waits run out one by one,
+// so they agree on the outcome: a lane that gave up alone would be missing from
+// the warp's TMEM loads and votes.
+template <class Smem>
+__device__ __forceinline__ bool wait_tile(Smem& sm, uint32_t ab, uint32_t phase) {
+  return __all_sync(kFull, tc::mbar_wait(&sm.tfull[ab], phase, &sm.abort, WAIT_LIMIT));
+}
+
 // One warp takes the next item from the ring (lane 0) and shares it.
 template <bool PAIR, class Smem>
 __device__ __forceinline__ int take_item(Smem& sm, const TcArgs& A, bool leader, int prev, int unit, int units,
@@ -484,7 +492,6 @@ __device__ __forceinline__ bool epilogue_pair(Smem& sm, const CUtensorMap* pA0, 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool leader = rank == 0;
   const int unit = int(blockIdx.x >> 1), units = int(gridDim.x >> 1);
-  volatile int* abort = &sm.abort;
   const int q = warp & 3;
   const int eg = (warp - 2) >> 2;
   const uint32_t tlane = tmem + (uint32_t(q * 32) << 16);
@@ -531,7 +538,7 @@ __device__ __forceinline__ bool epilogue_pair(Smem& sm, const CUtensorMap* pA0, 
     for (int ct = it.t0; ct < it.t1; ++ct) {
       const int fk = (live && ct > it.t0) ? __ldcg(it.row_floor + arow) : seen;
       const uint32_t ab = tcount & 1u, tph = (tcount >> 1) & 1u;
-      if (!tc::mbar_wait(&sm.tfull[ab], tph, abort, WAIT_LIMIT)) {
+      if (!wait_tile(sm, ab, tph)) {
         ok = false;
         break;
       }
@@ -668,7 +675,7 @@ __device__ __forceinline__ bool epilogue_sample(Smem& sm, const CUtensorMap* pA0
     for (int j = 0; j < 64; ++j) m[j] = -FLT_MAX;
     for (int ct = it.t0; ct < it.t1; ++ct) {
       const uint32_t ab = tcount & 1u, tph = (tcount >> 1) & 1u;
-      if (!tc::mbar_wait(&sm.tfull[ab], tph, &sm.abort, WAIT_LIMIT)) return false;
+      if (!wait_tile(sm, ab, tph)) return false;
       tc::tc_fence_after();
 #pragma unroll 1
       for (int cb = 0; cb < TBN / 32; cb += 2) {
@@ -777,7 +784,7 @@ __device__ __forceinline__ bool epilogue_append(Smem& sm, const CUtensorMap* pA0
     bool over = false;
     for (int ct = it.t0; ct < it.t1; ++ct) {
       const uint32_t ab = tcount & 1u, tph = (tcount >> 1) & 1u;
-      if (!tc::mbar_wait(&sm.tfull[ab], tph, &sm.abort, WAIT_LIMIT)) {
+      if (!wait_tile(sm, ab, tph)) {
         ok = false;
         break;
       }
@@ -876,7 +883,6 @@ __device__ __forceinline__ bool epilogue_single(TcSmem& sm, const CUtensorMap* p
                                                 int row_blocks, int64_t nrows, int items, int chunks) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int unit = int(blockIdx.x), units = int(gridDim.x);
-  volatile int* abort = &sm.abort;
   // Warp w may read TMEM lanes 32 (w % 4) .. + 31 (its rows); the groups split
   // the tile's columns, and each keeps its own list per row (EGROUPS lists per chunk).
   const int q = warp & 3;
@@ -918,7 +924,7 @@ __device__ __forceinline__ bool epilogue_single(TcSmem& sm, const CUtensorMap* p
     for (int ct = it.t0; ct < it.t1; ++ct) {
       const int fk = (live && ct > it.t0) ? __ldcg(it.row_floor + arow) : seen;
       const uint32_t ab = tcount & 1u, tph = (tcount >> 1) & 1u;
-      if (!tc::mbar_wait(&sm.tfull[ab], tph, abort, WAIT_LIMIT)) {
+      if (!wait_tile(sm, ab, tph)) {
         ok = false;
         break;
       }
