@@ -309,7 +309,8 @@ k4_spmm_warp(SrcRows S, const int32_t* __restrict__ nbr, const float* __restrict
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* keys = smem_i + wib * WSLOTS * 2;
   float* vals = reinterpret_cast<float*>(smem_i + wib * WSLOTS * 2 + WSLOTS);
-  if (status[kStErr] & kErrOverflow) return;
+  // Rows of this launch may set the bit meanwhile: the warp goes by one lane's reading.
+  if (__shfl_sync(kFull, int(status[kStErr]) & kErrOverflow, 0)) return;
   for (int s = lane; s < WSLOTS; s += kWarp) {
     keys[s] = KEY_EMPTY;
     vals[s] = 0.f;
