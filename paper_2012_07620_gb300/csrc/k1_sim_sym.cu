@@ -321,12 +321,8 @@ k1_select_rows(const float* __restrict__ S, int64_t ld, int64_t n, int K, float*
 }  // namespace
 
 int launch_sim_sym_topk(const Shape& sh, const float* xhat, float* S, float* part_s, int32_t* part_i, cudaStream_t s) {
-  static const bool once = [] {
-    cudaFuncSetAttribute(k1_sgemm_sym, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(SymSmem)));
-    cudaFuncSetAttribute(k1_select_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, int(RWARPS * sizeof(RowSel)));
-    return true;
-  }();
-  (void)once;
+  // Above 48 KB; the attribute belongs to the current device, so every launch sets it.
+  cudaFuncSetAttribute(k1_select_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, int(RWARPS * sizeof(RowSel)));
   const int64_t rb = sh.np / BM, cb = (sh.np + BN - 1) / BN;
   const dim3 grid(unsigned(cb * BAND), unsigned((rb + BAND - 1) / BAND));
   k1_sgemm_sym<<<grid, NT, sizeof(SymSmem), s>>>(xhat, sh.np, sh.dp, S);
