@@ -38,6 +38,7 @@
 // gathered rows being rechecked; their count is read on the device.
 #include <cuda.h>
 #include <cfloat>
+#include <atomic>
 #include <climits>
 #include <cmath>
 
@@ -1363,11 +1364,22 @@ void launch_kl(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& 
   k1_tc_topk<MODE, KL, EG><<<grid, threads_of(EG), smem, s>>>(a0, a1, b0, b1, A);
 }
 
+// Pairs of one kernel that can be resident at once, per device (-1: not asked yet).
+struct PairUnits {
+  static constexpr int kDevices = 64;
+  std::atomic<int> n[kDevices];
+  PairUnits() {
+    for (auto& v : n) v.store(-1, std::memory_order_relaxed);
+  }
+};
+
 // Launches `kernel` on pairs (clusters of two CTAs, one CTA per SM): as many as
-// there are items, at most those that can be resident at once (queried once
-// per kernel).  False when no pair can be resident or the launch fails.
+// there are items, at most those that can be resident at once.  Their number and
+// the kernel's shared-memory limit belong to a device: asked and set by the first
+// launch on each (callers and serving workers may be first at the same time; both
+// then store the same).  False when no pair can be resident or the launch fails.
 template <class Kernel, class... Args>
-bool launch_pairs(Kernel kernel, int* cached_units, size_t smem, int threads, int items, int sm_count, cudaStream_t s,
+bool launch_pairs(Kernel kernel, PairUnits& units, size_t smem, int threads, int items, int sm_count, cudaStream_t s,
                   const Args&... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(unsigned(sm_count & ~1));
@@ -1380,17 +1392,19 @@ bool launch_pairs(Kernel kernel, int* cached_units, size_t smem, int threads, in
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (*cached_units < 0) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  int n = dev < PairUnits::kDevices ? units.n[dev].load() : -1;
+  if (n < 0) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
       cudaGetLastError();
       n = 0;
     }
-    *cached_units = n;
+    if (dev < PairUnits::kDevices) units.n[dev].store(n);
   }
-  if (*cached_units < 1) return false;
-  cfg.gridDim = dim3(unsigned(2 * (items < *cached_units ? items : *cached_units)));
+  if (n < 1) return false;
+  cfg.gridDim = dim3(unsigned(2 * (items < n ? items : n)));
   cfg.stream = s;
   return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess;
 }
@@ -1398,34 +1412,34 @@ bool launch_pairs(Kernel kernel, int* cached_units, size_t smem, int threads, in
 template <int MODE, int KL, int EG>
 bool launch_kl_pair(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0, const CUtensorMap& b1,
                     const TcArgs& A, int items, int sm_count, cudaStream_t s) {
-  static int units = -1;
-  return launch_pairs(k1_tc2_topk<MODE, KL, EG>, &units, sizeof(TcSmemPair<KL, EG>) + 1024, threads_of(EG), items,
+  static PairUnits units;
+  return launch_pairs(k1_tc2_topk<MODE, KL, EG>, units, sizeof(TcSmemPair<KL, EG>) + 1024, threads_of(EG), items,
                       sm_count, s, a0, a1, b0, b1, A);
 }
 
 template <int MODE, int KR>
 bool launch_sample(const CUtensorMap& a, const CUtensorMap& b, const TcArgs& A, int items, int sm_count,
                    cudaStream_t s) {
-  static int units = -1;
-  return launch_pairs(k1_tc2_sample<MODE, KR>, &units, sizeof(TcSmemRing) + 1024, threads_of(1), items, sm_count, s, a,
+  static PairUnits units;
+  return launch_pairs(k1_tc2_sample<MODE, KR>, units, sizeof(TcSmemRing) + 1024, threads_of(1), items, sm_count, s, a,
                       b, A);
 }
 template <int MODE, int KR>
 bool launch_sample_batch(const TcMaps2& maps, const TcArgs& A, int items, int sm_count, cudaStream_t s) {
-  static int units = -1;
-  return launch_pairs(k1_tc2_sample_batch<MODE, KR>, &units, sizeof(TcSmemRing) + 1024, threads_of(1), items, sm_count,
+  static PairUnits units;
+  return launch_pairs(k1_tc2_sample_batch<MODE, KR>, units, sizeof(TcSmemRing) + 1024, threads_of(1), items, sm_count,
                       s, maps, A);
 }
 template <int MODE>
 bool launch_append(const CUtensorMap& a, const TcArgs& A, int items, int sm_count, cudaStream_t s) {
-  static int units = -1;
-  return launch_pairs(k1_tc2_append<MODE>, &units, sizeof(TcSmemRing) + 1024, threads_of(AEG), items, sm_count, s, a,
+  static PairUnits units;
+  return launch_pairs(k1_tc2_append<MODE>, units, sizeof(TcSmemRing) + 1024, threads_of(AEG), items, sm_count, s, a,
                       A);
 }
 template <int MODE>
 bool launch_append_batch(const TcMaps& maps, const TcArgs& A, int items, int sm_count, cudaStream_t s) {
-  static int units = -1;
-  return launch_pairs(k1_tc2_append_batch<MODE>, &units, sizeof(TcSmemRing) + 1024, threads_of(AEG), items, sm_count,
+  static PairUnits units;
+  return launch_pairs(k1_tc2_append_batch<MODE>, units, sizeof(TcSmemRing) + 1024, threads_of(AEG), items, sm_count,
                       s, maps, A);
 }
 

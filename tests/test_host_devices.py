@@ -20,9 +20,24 @@ def _run_on(lib, device, precision, n=1500, ng=1400):
         R.run(*a, 26, 7, 2, 0, oi, od, stream=0)
 
 
-@pytest.mark.parametrize("precision", ["fp32"])
+@pytest.mark.parametrize("precision", ["fp32", "bf16", "fp8"])
 def test_second_device_of_a_process(lib, precision):
     lib.fake.fake_reset(1 << 36)
     for device in (0, 1, 0):
         _run_on(lib, device, precision)
+    assert lib.fake.fake_count(b"refused") == 0
+
+
+@pytest.mark.parametrize("precision", ["bf16", "fp8"])
+def test_batch_and_serving_on_both_devices(lib, precision):
+    lib.fake.fake_reset(1 << 38)
+    for device in (0, 1):
+        lib.fake.cudaSetDevice(device)
+        x = fake_cuda.device(lib, (5000, 96))
+        oi, od = fake_cuda.device(lib, (64, 100), "int32"), fake_cuda.device(lib, (64, 100))
+        with lib.Reranker(device=device, precision=precision) as R:
+            job = dict(xq=x[:64], xg=x[64:], k1=26, k2=7, layers=2, topk_out=100, out_idx=oi, out_dist=od)
+            R.run_batch([job, job], stream=0)
+            R.load_gallery(x, 64, 26, 7, 2, slots=2)
+            R.wait(R.submit(x[:64], 100, oi, od, stream=0)[0])
     assert lib.fake.fake_count(b"refused") == 0
