@@ -585,7 +585,9 @@ int launch_propagate(const Shape& sh, const Buffers& b, int src, int dst, int ag
   const int min_rows = min_override >= 0 ? min_override : 4 * sm_count;
   const size_t rsmem = size_t(RWARPS) * MSLOTS * 2 * sizeof(int);
   auto go = [&](auto first, auto rest) {
-    cudaFuncSetAttribute(first, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    // (the limit of any launch of the kernel, whatever width other threads' launches have)
+    cudaFuncSetAttribute(first, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         int(kMaxPropWarps * WSLOTS * 2 * sizeof(int)));
     first<<<blocks, warps * kWarp, smem, s>>>(S, b.nbr, b.nbr_w, b.nbr_n, k2p1, b.ub, b.start[dst], b.len[dst],
                                               b.col[dst], b.val[dst], rnorm, n, sh.cap_h, b.big_rows, b.big_count,
                                               b.big_count + 1,

@@ -1047,6 +1047,12 @@ int64_t rank_scratch_words(int64_t ng) { return scratch_words(ng); }
 
 constexpr size_t kSmemMax = 227 * 1024;  // shared memory of one CTA
 constexpr size_t kSmemSm = 228 * 1024;   // of an SM
+// The limit is the kernel's, not the launch's: set to a launch's own size, it would
+// fail the larger launch that another thread is about to make.
+template <class Kernel>
+static void allow_smem(Kernel kernel) {
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemMax));
+}
 static size_t light_smem_bytes(int64_t ng) {
   return sizeof(LightSmem) + sizeof(uint32_t) * size_t(((ng + 31) / 32 + ng + 3) & ~int64_t(3));
 }
@@ -1056,7 +1062,7 @@ size_t rank_smem_bytes(int64_t ng, int threads) {
   const size_t fixed = rank_smem_fixed(ng);
   const size_t sorted = sizeof(uint64_t) * SORT_CAP;
   const size_t with_acc = fixed + (sizeof(uint32_t) * size_t(ng) > sorted ? sizeof(uint32_t) * size_t(ng) : sorted);
-  return with_acc <= 227 * 1024 ? with_acc : fixed + sorted;
+  return with_acc <= kSmemMax ? with_acc : fixed + sorted;
 }
 
 int launch_rank(const Shape& sh, const Buffers& b, int src, int32_t* out_idx, float* out_dist, long long* status,
@@ -1075,7 +1081,7 @@ int launch_rank_prep(const Shape& sh, const Buffers& b, int src, long long* stat
     const size_t smem = sizeof(uint32_t) * size_t(n);
     uint32_t* base = reinterpret_cast<uint32_t*>(b.hash_keys_vals);  // rank_ctas x n; the propagation is done with it
     auto pass = [&](auto kernel) {
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+      allow_smem(kernel);
       kernel<<<unsigned(sh.rank_ctas), K5T, smem, s>>>(b.start[src], b.len[src], b.col[src], b.val[src], b.rnorm, nq, n,
                                                        b.colptr, b.colcnt, base, b.csc, status);
     };
@@ -1135,10 +1141,10 @@ int launch_rank_queries(const Shape& sh, const Buffers& b, int src, int32_t* out
     const int64_t ctas = int64_t(sh.rank_ctas) * (two ? 2 : 1);
     const unsigned lg = unsigned(nqry < ctas ? (nqry > 0 ? nqry : 1) : ctas);
     if (two) {
-      cudaFuncSetAttribute(k6_rank_light<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(light));
+      allow_smem(k6_rank_light<512>);
       k6_rank_light<512><<<lg, 512, light, s>>>(A);
     } else {
-      cudaFuncSetAttribute(k6_rank_light<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(light));
+      allow_smem(k6_rank_light<1024>);
       k6_rank_light<1024><<<lg, 1024, light, s>>>(A);
     }
     A.qlist = A.over;
@@ -1152,10 +1158,10 @@ int launch_rank_queries(const Shape& sh, const Buffers& b, int src, int32_t* out
   if (A.idx_smem && with_idx > smem) smem = with_idx;
   const unsigned grid = unsigned(nqry < sh.rank_ctas ? (nqry > 0 ? nqry : 1) : sh.rank_ctas);
   if (A.acc_smem) {
-    cudaFuncSetAttribute(k6_rank<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    allow_smem(k6_rank<true>);
     k6_rank<true><<<grid, RT, smem, s>>>(A);
   } else {
-    cudaFuncSetAttribute(k6_rank<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    allow_smem(k6_rank<false>);
     k6_rank<false><<<grid, RT, smem, s>>>(A);
   }
   return nl;

@@ -154,7 +154,11 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
 }
 cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {
   std::lock_guard<std::mutex> lk(S().mu);
-  if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) S().shared[{f, t_dev}] = size_t(v);
+  if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) {
+    size_t& limit = S().shared[{f, t_dev}];
+    if (size_t(v) < limit) ++S().counts["lowered " + S().names[f]];
+    limit = size_t(v);
+  }
   return cudaSuccess;
 }
 cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunchConfig_t*) {

@@ -41,3 +41,13 @@ def test_batch_and_serving_on_both_devices(lib, precision):
             R.load_gallery(x, 64, 26, 7, 2, slots=2)
             R.wait(R.submit(x[:64], 100, oi, od, stream=0)[0])
     assert lib.fake.fake_count(b"refused") == 0
+
+
+def test_no_launch_lowers_a_kernels_shared_memory_limit(lib):
+    """The limit is the kernel's, not the launch's: lowering it for a small call would
+    fail the larger launch that another thread is about to make."""
+    lib.fake.fake_reset(1 << 38)
+    for precision in ("fp32", "bf16"):
+        for n, ng in ((24000, 23000), (16000, 15000), (1500, 1400)):
+            _run_on(lib, 0, precision, n, ng)
+    assert lib.fake.fake_count(b"lowered") == 0
