@@ -25,7 +25,10 @@
  *     (one stream synchronisation at the end of the call).
  *   - The caller owns every buffer it passes; the library never frees them.
  *     The context owns its device workspace, which grows on demand up to
- *     `hbm_budget` and is reused by later calls.
+ *     `hbm_budget` and is reused by later calls.  Where the budget or the
+ *     device has no room for the fastest similarity plan, a call takes one
+ *     that needs less (the same results); a size that the device had no room
+ *     for is not tried again until as much has been allocated.
  *   - Every call returns a status and never aborts the process.  A context
  *     must not be used by two host threads at once.
  */

@@ -201,16 +201,33 @@ rerank_status ensure_workspace(rerank_ctx* ctx, size_t bytes) {
     ctx->ws = nullptr;
     ctx->ws_bytes = 0;
   }
+  // An eighth to spare for the next, slightly larger call, where it fits.
   const size_t want = bytes + bytes / 8;
-  const size_t alloc = (ctx->cfg.hbm_budget && want > ctx->cfg.hbm_budget) ? bytes : want;
-  const cudaError_t e = cudaMalloc(&ctx->ws, alloc);
+  size_t alloc = (ctx->cfg.hbm_budget && want > ctx->cfg.hbm_budget) ? bytes : want;
+  cudaError_t e = cudaMalloc(&ctx->ws, alloc);
+  if (e == cudaErrorMemoryAllocation && alloc > bytes) {
+    cudaGetLastError();
+    alloc = bytes;
+    e = cudaMalloc(&ctx->ws, alloc);
+  }
   if (e != cudaSuccess) {
     ctx->ws = nullptr;
     cudaGetLastError();  // the caller may go on with a smaller plan
-    return cuda_fail(e, "cudaMalloc(workspace)");
+    const rerank_status st = cuda_fail(e, "cudaMalloc(workspace)");
+    if (st == RERANK_ENOMEM && (!ctx->no_room || bytes < ctx->no_room)) ctx->no_room = bytes;
+    return st;
   }
   ctx->ws_bytes = alloc;
+  if (bytes >= ctx->no_room) ctx->no_room = 0;  // there is room again
   return RERANK_OK;
+}
+
+// The workspace of a plan that has a smaller stand-in.  A size that the device had
+// no room for is not tried again: trying means giving up the workspace and the
+// graphs that the smaller plan's calls go on using.
+rerank_status ensure_wide_workspace(rerank_ctx* ctx, size_t bytes) {
+  if (ctx->no_room && bytes >= ctx->no_room && bytes > ctx->ws_bytes) return RERANK_ENOMEM;
+  return ensure_workspace(ctx, bytes);
 }
 
 rerank_status collect(rerank_ctx* ctx, cudaStream_t s) {
@@ -520,8 +537,9 @@ rerank_status run_once(rerank_ctx* ctx, const void* xq, const void* xg, int32_t*
   j.sh = ctx->shape;
   Carver dry;
   size_t need = carve(dry, j.sh, j.b, ctx->sm_count, ctx->cfg.precision);
-  rerank_status st = ensure_workspace(ctx, need);
-  if ((st == RERANK_EBUDGET || st == RERANK_ENOMEM) && (j.sh.segs > 0 || j.sh.smat)) {
+  const bool wide = j.sh.segs > 0 || j.sh.smat;
+  rerank_status st = wide ? ensure_wide_workspace(ctx, need) : ensure_workspace(ctx, need);
+  if (wide && (st == RERANK_EBUDGET || st == RERANK_ENOMEM)) {
     // No room for the append pass's segments (or the matrix): the list kernels need less.
     st = plan_lists(ctx, &j.sh);
     if (st != RERANK_OK) return st;
@@ -840,7 +858,7 @@ rerank_status run_batch(rerank_ctx* ctx, rerank_job* jobs, int njobs, cudaStream
     total = (total + 255) & ~size_t(255);
     inst_off = total;
     if (tc_batch) total += inst_bytes;
-    st = ensure_workspace(ctx, total);
+    st = append ? ensure_wide_workspace(ctx, total) : ensure_workspace(ctx, total);
     if (!append || (st != RERANK_EBUDGET && st != RERANK_ENOMEM)) break;
   }
   if (st != RERANK_OK) return st;

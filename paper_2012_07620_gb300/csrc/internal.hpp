@@ -193,6 +193,7 @@ struct rerank_ctx {
   size_t smem_optin = 0;
   char* ws = nullptr;          // device workspace block
   size_t ws_bytes = 0;
+  size_t no_room = 0;          // smallest workspace the device had no room for (0: none; see ensure_wide_workspace)
   long long* d_status = nullptr;  // device status block (rr::kStCount int64)
   long long* h_status = nullptr;  // pinned host copy
   std::vector<rr::TuneEntry> tune_table;  // loaded from / written to tune_path

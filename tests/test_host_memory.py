@@ -1,0 +1,74 @@
+"""Plans at the limits of device memory, on a stand-in runtime with a set capacity:
+which plan a call ends up with, and what it allocates and frees."""
+import pytest
+
+import fake_cuda
+
+MB = 1 << 20
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    return fake_cuda.load(tmp_path_factory.mktemp("fake"))
+
+
+class Case:
+    """One instance in the stand-in's memory, and what its two plans take."""
+
+    def __init__(self, lib, precision, n=20000, d=128, nq=500, jobs=1):
+        lib.fake.fake_reset(1 << 40)
+        lib.fake.cudaSetDevice(0)
+        self.lib, self.precision = lib, precision
+        x = fake_cuda.device(lib, (n, d))
+        self.x, self.nq = x, nq
+        self.jobs = [dict(xq=x[:nq], xg=x[nq:], k1=26, k2=7, layers=2, topk_out=100,
+                          out_idx=fake_cuda.device(lib, (nq, 100), "int32"),
+                          out_dist=fake_cuda.device(lib, (nq, 100))) for _ in range(jobs)]
+        self.base = lib.fake.fake_used(0)
+        with self.context() as R:
+            self.call(R)
+            self.wide = R.last_info()["workspace_bytes"] * 8 // 9  # allocations have an eighth to spare
+        with self.context(hbm_budget=self.wide - 1) as R:
+            self.call(R)
+            self.narrow = R.last_info()["workspace_bytes"]
+        assert self.narrow + 16 * MB < self.wide
+
+    def context(self, **kw):
+        return self.lib.Reranker(device=0, precision=self.precision, **kw)
+
+    def call(self, R):
+        if len(self.jobs) > 1:
+            R.run_batch(self.jobs, stream=0)
+        else:
+            j = self.jobs[0]
+            R.run(j["xq"], j["xg"], 26, 7, 2, 100, j["out_idx"], j["out_dist"], stream=0)
+
+    def room(self, nbytes):
+        self.lib.fake.fake_reset(self.base + nbytes + MB)  # the status block and the like
+
+    def allocations(self):
+        return [self.lib.fake.fake_count(w) for w in (b"cudaMalloc", b"cudaFree")]
+
+
+@pytest.mark.parametrize("precision,jobs", [("fp32", 1), ("bf16", 1), ("fp8", 1), ("fp32", 3), ("bf16", 3)])
+def test_a_plan_without_room_is_not_tried_again(lib, precision, jobs):
+    c = Case(lib, precision, jobs=jobs)
+    c.room(c.narrow)
+    with c.context() as R:
+        c.call(R)
+        first = c.allocations()
+        for _ in range(4):
+            c.call(R)
+        assert c.allocations() == first
+        if jobs > 1:  # captured by the second call and replayed, not dropped
+            assert lib.fake.fake_count(b"graph captured") == 1
+            assert lib.fake.fake_count(b"graph launched") == 4
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+def test_the_exact_size_is_tried_before_a_plan_is_given_up(lib, precision):
+    c = Case(lib, precision)
+    c.room(c.wide)
+    with c.context() as R:
+        c.call(R)
+        assert c.narrow < R.last_info()["workspace_bytes"] <= c.wide + MB
