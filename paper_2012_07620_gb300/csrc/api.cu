@@ -123,7 +123,7 @@ size_t carve(Carver& c, const Shape& sh, Buffers& b, int sm_count, int precision
   if (sh.segs > 0) {
     b.ap.xsample = c.take<char>(size_t(sh.sample) * sh.dp * (precision == RERANK_PREC_FP8 ? 1 : 2));
     b.ap.sample_scale = c.take<float>(size_t(sh.sample));
-    b.ap.cand = c.take<int64_t>(size_t(n) * sh.segs * sh.seg_cap);
+    b.ap.cand = c.take<int64_t>(size_t(sh.seg_rows) * sh.segs * sh.seg_cap);
     b.ap.seg_cnt = c.take<int32_t>(size_t(n) * sh.segs);
   }
   if (sh.smat) b.smat = c.take<float>(size_t(np) * np);
@@ -335,7 +335,7 @@ rerank_status enqueue_job(rerank_ctx* ctx, const JobRun& j, cudaStream_t s, Stag
   }
   // Batched calls run the similarity launch over all instances: its selection
   // (like the sampled rows it started from) belongs to each instance.
-  if (sh.segs > 0 && !(phases & kPhaseSim)) nl += launch_select(sh, b.ap, b.part_s, b.part_i, status, s);
+  if (sh.segs > 0 && !(phases & kPhaseSim)) nl += launch_select(sh, b.ap, 0, sh.n, b.part_s, b.part_i, status, s);
   const int32_t* order = nullptr;
   if (sh.tune.refine_order) {
     nl += launch_cluster_order(sh, b.part_s, b.part_i, b.nb4, b.label, b.ord_cnt, b.ord_start, b.ord_fill, b.order,
@@ -527,7 +527,7 @@ rerank_status map_status(const long long* h, int precision, rerank_info* info, i
 rerank_status plan_lists(const rerank_ctx* ctx, Shape* sh) {
   const Shape o = *sh;
   return plan_shape(ctx, o.nq, o.ng, o.d, o.dtype, o.k1, o.k2, o.layers, o.topk, o.knn_only, o.host_in, o.host_out,
-                    o.cap_h, sh, nullptr, false);
+                    o.cap_h, sh, nullptr, Side::kNone);
 }
 
 // One attempt of the pipeline.  Returns OK, or the mapped device error.
@@ -587,7 +587,7 @@ constexpr size_t kSymBytes = size_t(16) << 30;
 // Shape of one instance.  cap_hint: a layer capacity learned from an earlier overflow.
 rerank_status plan_shape(const rerank_ctx* ctx, int64_t nq, int64_t ng, int d, int dtype, int k1, int k2, int layers,
                          int64_t topk, bool knn_only, bool host_in, bool host_out, int64_t cap_hint, Shape* out,
-                         const Tuning* tune, bool append) {
+                         const Tuning* tune, Side side) {
   Shape sh;
   sh.nq = nq;
   sh.ng = ng;
@@ -619,7 +619,7 @@ rerank_status plan_shape(const rerank_ctx* ctx, int64_t nq, int64_t ng, int d, i
   // tensor-core products over all columns in the recheck (market: 4,004 rows
   // with 42 places, 6 with 64; recheck 0.88 -> 0.19 ms).  Smaller margins that
   // the caller or the tuning table asks for are kept.
-  const bool may_append = tc && append && tc_append_ok(sh.np, ctx->sm_count);
+  const bool may_append = tc && side != Side::kNone && tc_append_ok(sh.np, ctx->sm_count);
   const bool full = may_append && sh.tune.rescore_m < 0 && m >= 16;
   int64_t K = std::min<int64_t>(full ? kmax : int64_t(k1) + std::max(m, 0), sh.n);
   K = std::min<int64_t>(K, kmax);
@@ -639,9 +639,10 @@ rerank_status plan_shape(const rerank_ctx* ctx, int64_t nq, int64_t ng, int d, i
   sh.P = std::min(chunks, 32 / lpc) * lpc;
   if (may_append) {
     tc_append_plan(sh.n, sh.np, sh.dp, sh.K, chunks, &sh.segs, &sh.seg_cap, &sh.sample);
+    sh.seg_rows = side == Side::kBands ? tc_append_band(sh.n, sh.segs, sh.seg_cap) : sh.n;
     sh.P = 1;
   }
-  if (!tc && append && size_t(sh.np) * sh.np * 4 <= kSymBytes) {
+  if (!tc && side != Side::kNone && size_t(sh.np) * sh.np * 4 <= kSymBytes) {
     sh.smat = true;
     sh.P = 1;
   }
@@ -754,7 +755,7 @@ uint64_t buffer_id(const void* p) {
 // workspace offset they fix everything a batched call enqueues for it.
 void shape_key(const Shape& sh, std::vector<int64_t>& k) {
   const int64_t v[] = {sh.nq, sh.ng, sh.n, sh.np, sh.d, sh.dp, sh.dtype, sh.k1, sh.k2, sh.layers, sh.K, sh.P, sh.P3,
-                       sh.P3g, sh.K3, sh.segs, sh.seg_cap, sh.sample, sh.smat, sh.topk, sh.host_in, sh.host_out, sh.knn_only,
+                       sh.P3g, sh.K3, sh.segs, sh.seg_cap, sh.seg_rows, sh.sample, sh.smat, sh.topk, sh.host_in, sh.host_out, sh.knn_only,
                        sh.ext_feat, sh.cap_h, sh.cap_csc, sh.hash_slots, sh.rank_ctas, sh.rank_scratch_per_cta, sh.tune.sim_chunks, sh.tune.prop_warps,
                        sh.tune.refine_order, sh.tune.rescore_m, sh.tune.rank_threads};
   k.insert(k.end(), std::begin(v), std::end(v));
@@ -846,7 +847,7 @@ rerank_status run_batch(rerank_ctx* ctx, rerank_job* jobs, int njobs, cudaStream
       const bool host_out = is_host_ptr(jb.out_idx) || is_host_ptr(jb.out_dist);
       const int64_t topk = jb.topk_out ? jb.topk_out : jb.ng;
       st = plan_shape(ctx, jb.nq, jb.ng, jb.d, jb.dtype, jb.k1, jb.k2, jb.layers, topk, false, host_in, host_out, 0,
-                      &run.sh, nullptr, attempt == 0);
+                      &run.sh, nullptr, attempt == 0 ? Side::kWhole : Side::kNone);
       if (st != RERANK_OK) return st;
       append = append || run.sh.segs > 0 || run.sh.smat;
       Carver dry;

@@ -54,7 +54,7 @@ int tune_bucket(int64_t n);  // half-octave bucket of the vertex count
 struct TcAppend {
   void* xsample = nullptr;       // sample x dp: sampled rows of the low-precision copy
   float* sample_scale = nullptr; // sample: their FP8 scales
-  void* cand = nullptr;          // n x segs x seg_cap (score, vertex) pairs, 8 bytes each
+  void* cand = nullptr;          // seg_rows x segs x seg_cap (score, vertex) pairs, 8 bytes each
   int32_t* seg_cnt = nullptr;    // n x segs
 };
 
@@ -148,6 +148,7 @@ struct Shape {
   bool smat = false;       // FP32: the similarity matrix is kept (np x np floats) and half of it computed
   int segs = 0;            // append pass: segments per row (0: the list kernels)
   int seg_cap = 0;         // entries of a segment
+  int64_t seg_rows = 0;    // rows whose segments exist at a time (n, or the rows of a band)
   int sample = 0;          // columns sampled for its floors (0: none)
   int K3 = 0;              // FP8 path: candidates per list of that stage (the longest list the kernels hold)
   int64_t topk = 0;
@@ -257,11 +258,14 @@ int launch_sim_tc_topk(const Shape& sh, const void* xlow, bool fp8, const float*
 // split wants.  tc_append_ok: whether it can run (else the list kernels do).
 bool tc_append_ok(int64_t np, int sm_count);
 void tc_append_plan(int64_t n, int64_t np, int dp, int K, int chunks, int* segs, int* cap, int* sample);
+// Rows of a band: as many as have their segments in tc_segment_bytes(), at most n.
+int64_t tc_append_band(int64_t n, int segs, int cap);
 int launch_sample_rows(const Shape& sh, const void* xlow, bool fp8, const float* inv_scale, const TcAppend& ap,
                        cudaStream_t s);
 // The append pass's segments into one sorted list of K per row.
-int launch_select(const Shape& sh, const TcAppend& ap, float* part_s, int32_t* part_i, const long long* status,
-                  cudaStream_t s);
+// (rows [r0, r0 + rows) of them; ap.cand holds row r0's first)
+int launch_select(const Shape& sh, const TcAppend& ap, int64_t r0, int64_t rows, float* part_s, int32_t* part_i,
+                  const long long* status, cudaStream_t s);
 // Rectangular block: rows of `a` (a_rows of them, vertices row0 ..) against the
 // columns of `b` (b_cols, vertices col0 ..); per row P lists of its best K
 // columns (vertex indices) in part_s/part_i [a_rows][P][K].  Rows and columns
@@ -460,10 +464,17 @@ bool is_host_ptr(const void* p);
 size_t type_size(int dtype);
 int choose_chunks(int64_t row_blocks, int64_t col_tiles, int sm_count, int forced);
 size_t carve(Carver& c, const Shape& sh, Buffers& b, int sm_count, int precision);
+// The memory that the similarity stage may take to be faster: the append pass's
+// segments, or the FP32 matrix.
+enum class Side {
+  kNone,   // none: the list kernels
+  kBands,  // the segments of one band of rows after the other share theirs
+  kWhole   // the segments of all rows at once (batched calls: one launch over all instances)
+};
 rerank_status plan_shape(const rerank_ctx* ctx, int64_t nq, int64_t ng, int d, int dtype, int k1, int k2,
                          int layers, int64_t topk, bool knn_only, bool host_in, bool host_out, int64_t cap_hint,
                          Shape* out, const Tuning* tune = nullptr,  // tune: override of the table lookup
-                         bool append = true);  // append: the similarity stage may take the append pass
+                         Side side = Side::kBands);
 // copy_overlap: host outputs are copied back in parts while later queries are
 // ranked (single calls only; batched instances copy on their own stream).
 // phases: which parts to enqueue (status reset, copies in and normalisation /

@@ -177,6 +177,7 @@ struct TcArgs {
   uint2* cand;              // append pass: rows x (chunks * AEG) x cap admitted (score bits, vertex)
   int32_t* seg_cnt;         // append pass: entries per segment; cap + 1 when it ran over
   int cap;
+  int rb0;                  // append pass: first row block of the launch (cand holds its rows on)
   int mb_off;               // batched sampling pass: index of instance 0's sample map
   int* work;                // non-null: items are taken in order from this counter (zero at launch)
 };
@@ -229,7 +230,7 @@ __device__ __forceinline__ void get_item(const TcArgs& A, const CUtensorMap* ma0
     it.ma1 = ma1;
     it.mb0 = mb0;
     it.mb1 = mb1;
-    it.rb = item % row_blocks;
+    it.rb = A.rb0 + item % row_blocks;
     it.chunk = item / row_blocks;
     it.t0 = int(int64_t(it.chunk) * A.col_tiles / chunks);
     it.t1 = int(int64_t(it.chunk + 1) * A.col_tiles / chunks);
@@ -778,7 +779,8 @@ __device__ __forceinline__ bool epilogue_append(Smem& sm, const CUtensorMap* pA0
     const float rinv = (MODE == MODE_FP8 && live) ? it.inv_scale[arow] : 1.0f;
     const f32x2 rinv2 = twice(rinv);
     const bool wide = MODE == MODE_FP8 && (reinterpret_cast<uintptr_t>(it.inv_scale) & 15) == 0;
-    const size_t seg = size_t(live ? arow : 0) * (it.chunks * AEG) + it.chunk * AEG + eg;
+    const size_t brow = live ? size_t(arow - int64_t(A.rb0) * (2 * TBM)) : 0;  // the row's place in the band
+    const size_t seg = brow * (it.chunks * AEG) + it.chunk * AEG + eg;
     const uint64_t p0 = reinterpret_cast<uint64_t>(it.cand + seg * it.cap);
     const uint64_t plast = p0 + 8u * (it.cap - 32);  // beyond it a batch might not fit
     uint64_t p = p0;
@@ -1741,6 +1743,21 @@ void tc_append_plan(int64_t n, int64_t np, int dp, int K, int chunks, int* segs,
   *cap = segment_cap(n, K, m, *segs, most);
 }
 
+// The segments of a large instance would outgrow its lists by far (64 KB a row at
+// 16 chunks against some 2 to 3 KB of entries: 65 GB at a million rows), so they are
+// kept for bands of rows: 4 GB hold the segments of at least 65,536 rows, and a
+// launch over so many has thousands of work items for its 76 pairs.
+static size_t tc_segment_bytes() {
+  // Test hook: smaller bands on small instances.
+  const char* e = std::getenv("RERANK_TEST_SEGMENT_BYTES");
+  return e ? size_t(std::atoll(e)) : size_t(4) << 30;
+}
+int64_t tc_append_band(int64_t n, int segs, int cap) {
+  const int64_t block = 2 * TBM;  // a band is whole row blocks
+  const int64_t rows = int64_t(tc_segment_bytes() / (size_t(segs) * cap * sizeof(uint2))) / block * block;
+  return n < rows ? n : (rows < block ? (n < block ? n : block) : rows);
+}
+
 static bool launch_sample_pass(const CUtensorMap& map, const CUtensorMap& smap, const TcArgs& S, bool fp8,
                                int sm_count, cudaStream_t s) {
   const int rk = S.floor_rank, items = S.row_blocks;
@@ -1774,7 +1791,7 @@ int launch_sim_tc_topk(const Shape& sh, const void* xlow, bool fp8, const float*
   A.stall = stall_hook();
   if (sh.segs > 0) {
     A.row_blocks = int(sh.np / (2 * TBM));
-    int nl = 2;
+    int nl = 0;
     if (sh.sample > 0) {
       CUtensorMap smap;
       if (!make_map(&smap, ap.xsample, sh.sample, sh.dp, fp8)) return -1;
@@ -1792,17 +1809,21 @@ int launch_sim_tc_topk(const Shape& sh, const void* xlow, bool fp8, const float*
     }
     A.chunks = sh.segs / AEG;
     A.cand = static_cast<uint2*>(ap.cand);
-    A.seg_cnt = ap.seg_cnt;
     A.cap = sh.seg_cap;
-    if (work && tc_dynamic()) {
-      cudaMemsetAsync(work, 0, sizeof(int32_t), s);
-      A.work = work;
+    if (work && tc_dynamic()) A.work = work;
+    // A band's rows are selected before the next band takes their segments.
+    for (int64_t r0 = 0; r0 < sh.n; r0 += sh.seg_rows) {
+      const int64_t rows = sh.n - r0 < sh.seg_rows ? sh.n - r0 : sh.seg_rows;
+      A.rb0 = int(r0 / (2 * TBM));
+      A.row_blocks = int((rows + 2 * TBM - 1) / (2 * TBM));
+      A.seg_cnt = ap.seg_cnt + r0 * sh.segs;
+      if (A.work) cudaMemsetAsync(work, 0, sizeof(int32_t), s);
+      const int items = A.row_blocks * A.chunks;
+      if (!(fp8 ? launch_append<MODE_FP8>(map, A, items, sm_count, s)
+                : launch_append<MODE_BF16>(map, A, items, sm_count, s)))
+        return -1;
+      nl += 1 + launch_select(sh, ap, r0, rows, part_s, part_i, status, s);
     }
-    const int items = A.row_blocks * A.chunks;
-    if (!(fp8 ? launch_append<MODE_FP8>(map, A, items, sm_count, s)
-              : launch_append<MODE_BF16>(map, A, items, sm_count, s)))
-      return -1;
-    nl += launch_select(sh, ap, part_s, part_i, status, s) - 1;
     return nl;
   }
   cudaMemsetAsync(row_floor, kFloorResetByte, sizeof(int) * size_t(sh.n), s);
@@ -1838,10 +1859,11 @@ int launch_sample_rows(const Shape& sh, const void* xlow, bool fp8, const float*
   return 1;
 }
 
-int launch_select(const Shape& sh, const TcAppend& ap, float* part_s, int32_t* part_i, const long long* status,
-                  cudaStream_t s) {
-  k_select<<<unsigned((sh.n + SEL_WARPS - 1) / SEL_WARPS), SEL_WARPS * kWarp, 0, s>>>(
-      static_cast<const uint2*>(ap.cand), ap.seg_cnt, sh.n, sh.segs, sh.seg_cap, sh.K, part_s, part_i, status);
+int launch_select(const Shape& sh, const TcAppend& ap, int64_t r0, int64_t rows, float* part_s, int32_t* part_i,
+                  const long long* status, cudaStream_t s) {
+  k_select<<<unsigned((rows + SEL_WARPS - 1) / SEL_WARPS), SEL_WARPS * kWarp, 0, s>>>(
+      static_cast<const uint2*>(ap.cand), ap.seg_cnt + r0 * sh.segs, rows, sh.segs, sh.seg_cap, sh.K,
+      part_s + r0 * sh.K, part_i + r0 * sh.K, status);
   return 1;
 }
 
@@ -1878,10 +1900,9 @@ int launch_sim_tc_rows_append(const Shape& sh, const void* x, int64_t a_rows, in
   if (!(fp8 ? launch_append<MODE_FP8>(map, A, items, sm_count, s) : launch_append<MODE_BF16>(map, A, items, sm_count, s)))
     return -1;
   Shape rows = sh;
-  rows.n = a_rows;
   rows.segs = chunks * AEG;
   rows.seg_cap = cap;
-  return 2 + launch_select(rows, ap, part_s, part_i, status, s);
+  return 2 + launch_select(rows, ap, 0, a_rows, part_s, part_i, status, s);
 }
 
 int launch_sim_tc_rect_topk(const Shape& sh, const void* a, int64_t a_rows, int64_t row0, const void* b,

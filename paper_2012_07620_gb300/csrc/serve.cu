@@ -483,7 +483,7 @@ rerank_status enqueue_request(Server& v, Slot& sl, const rerank_request& rq, cud
   tq.rescore_m = v.margin;
   rerank_status st =
       plan_shape(ctx, Q, G, v.d, v.dtype, v.k1, v.k2, v.layers, topk, false, false, host_out, 0, &sh, &tq,
-                 false);
+                 Side::kNone);
   if (st != RERANK_OK) return st;
   sh.K = v.K;
   sh.ext_feat = true;
@@ -912,7 +912,7 @@ rerank_status serve_load(rerank_ctx* ctx, const void* xg, int64_t ng, int d, int
   Tuning tg = lookup_tuning(ctx, prec, ng, d);
   tg.rescore_m = v->margin;
   st = plan_shape(ctx, ng, 0, d, dtype, k1, 1, 0, 0, true, false, false, 0, &shg, &tg,
-                  false);  // lists of K entries, not bounded by a floor
+                  Side::kNone);  // lists of K entries, not bounded by a floor
   if (st != RERANK_OK) {
     delete v;
     return st;
@@ -922,7 +922,7 @@ rerank_status serve_load(rerank_ctx* ctx, const void* xg, int64_t ng, int d, int
   Shape shmax;
   Tuning tm = lookup_tuning(ctx, prec, S + ng, d);
   tm.rescore_m = v->margin;
-  st = plan_shape(ctx, S, ng, d, dtype, k1, k2, layers, ng, false, false, true, 0, &shmax, &tm, false);
+  st = plan_shape(ctx, S, ng, d, dtype, k1, k2, layers, ng, false, false, true, 0, &shmax, &tm, Side::kNone);
   if (st != RERANK_OK) {
     delete v;
     return st;

@@ -72,3 +72,16 @@ def test_the_exact_size_is_tried_before_a_plan_is_given_up(lib, precision):
     with c.context() as R:
         c.call(R)
         assert c.narrow < R.last_info()["workspace_bytes"] <= c.wide + MB
+
+
+@pytest.mark.parametrize("precision", ["bf16", "fp8"])
+def test_segments_of_a_large_instance_are_bounded(lib, precision):
+    """At most 4 GB beside the plan with lists (64 KB a row otherwise: 65 GB here)."""
+    lib.fake.fake_reset(1 << 40)
+    n = 1000000
+    x, oi, os = (fake_cuda.device(lib, (n, w), t) for w, t in ((64, "f4"), (26, "i4"), (26, "f4")))
+    with lib.Reranker(device=0, precision=precision) as R:
+        R.knn(x, 26, oi, os, stream=0)
+        need = R.last_info()["workspace_bytes"] * 8 // 9
+    recheck = n * 32 * 64 * 8  # its lists, the largest buffer of either plan
+    assert need < recheck + (4 << 30) + (3 << 30)  # rows, copies and the final lists
