@@ -579,10 +579,23 @@ rerank_status run_once(rerank_ctx* ctx, const void* xq, const void* xg, int32_t*
   return st;
 }
 
-// Largest similarity matrix that the FP32 path keeps (n up to about 65,000): a
-// twentieth of the device's memory, with the rest left to the caller's data.
-// Beyond it the streaming kernel computes the whole square.
-constexpr size_t kSymBytes = size_t(16) << 30;
+// Most memory that one call takes to be faster: the FP32 similarity matrix (n up to
+// about 65,000), or the matrices and segments of all instances of a batched call.
+// A twentieth of the device's memory, with the rest left to the caller's data.
+// Beyond it the streaming kernel or the list kernels compute the whole square.
+constexpr size_t kSideBytes = size_t(16) << 30;
+
+// Test hook: fewer, so that the instances of a small batch are planned both ways.
+size_t batch_side_bytes() {
+  const char* e = std::getenv("RERANK_TEST_SIDE_BYTES");
+  return e ? size_t(std::atoll(e)) : kSideBytes;
+}
+
+// What an instance takes of it.
+size_t side_bytes(const Shape& sh) {
+  if (sh.smat) return size_t(sh.np) * sh.np * 4;
+  return size_t(sh.seg_rows) * sh.segs * sh.seg_cap * 8;
+}
 
 // Shape of one instance.  cap_hint: a layer capacity learned from an earlier overflow.
 rerank_status plan_shape(const rerank_ctx* ctx, int64_t nq, int64_t ng, int d, int dtype, int k1, int k2, int layers,
@@ -642,7 +655,7 @@ rerank_status plan_shape(const rerank_ctx* ctx, int64_t nq, int64_t ng, int d, i
     sh.seg_rows = side == Side::kBands ? tc_append_band(sh.n, sh.segs, sh.seg_cap) : sh.n;
     sh.P = 1;
   }
-  if (!tc && side != Side::kNone && size_t(sh.np) * sh.np * 4 <= kSymBytes) {
+  if (!tc && side != Side::kNone && size_t(sh.np) * sh.np * 4 <= kSideBytes) {
     sh.smat = true;
     sh.P = 1;
   }
@@ -838,6 +851,7 @@ rerank_status run_batch(rerank_ctx* ctx, rerank_job* jobs, int njobs, cudaStream
   // With the append pass's segments; without them where they do not fit.
   for (int attempt = 0; attempt < 2; ++attempt) {
     bool append = false;
+    size_t side = batch_side_bytes();  // left for the instances to come
     total = 0;
     for (int i = 0; i < njobs; ++i) {
       const rerank_job& jb = jobs[i];
@@ -846,9 +860,14 @@ rerank_status run_batch(rerank_ctx* ctx, rerank_job* jobs, int njobs, cudaStream
       const bool host_in = is_host_ptr(jb.xq) || is_host_ptr(jb.xg);
       const bool host_out = is_host_ptr(jb.out_idx) || is_host_ptr(jb.out_dist);
       const int64_t topk = jb.topk_out ? jb.topk_out : jb.ng;
-      st = plan_shape(ctx, jb.nq, jb.ng, jb.d, jb.dtype, jb.k1, jb.k2, jb.layers, topk, false, host_in, host_out, 0,
-                      &run.sh, nullptr, attempt == 0 ? Side::kWhole : Side::kNone);
+      auto plan_side = [&](Side w) {
+        return plan_shape(ctx, jb.nq, jb.ng, jb.d, jb.dtype, jb.k1, jb.k2, jb.layers, topk, false, host_in, host_out,
+                          0, &run.sh, nullptr, w);
+      };
+      st = plan_side(attempt == 0 ? Side::kWhole : Side::kNone);
+      if (st == RERANK_OK && side_bytes(run.sh) > side) st = plan_side(Side::kNone);
       if (st != RERANK_OK) return st;
+      side -= side_bytes(run.sh);
       append = append || run.sh.segs > 0 || run.sh.smat;
       Carver dry;
       const size_t need = carve(dry, run.sh, run.b, ctx->sm_count, ctx->cfg.precision);

@@ -1,5 +1,6 @@
-"""The append pass over bands of rows that share their segments gives the lists of
-one pass over all rows."""
+"""Plans that share or lack the memory the fastest ones take give the same results:
+the append pass over bands of rows that share their segments, and batches whose
+later instances do without segments or matrix."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -30,3 +31,27 @@ def test_bands_equal_one_pass(lib, monkeypatch, n, d, precision):
     assert out[1][2] == out[0][2] + 2 * ((n - 1) // 256)  # an append and a selection per band
     for i, s, _ in out[1:]:
         assert torch.equal(i, out[0][0]) and torch.equal(s, out[0][1])
+
+
+@pytest.mark.parametrize("precision,nbytes", [("fp32", 50 << 20), ("bf16", 40 << 20), ("fp8", 40 << 20)])
+def test_batch_with_and_without_segments_or_matrix(lib, monkeypatch, precision, nbytes):
+    g = torch.Generator().manual_seed(4)
+    jobs = []
+    for n, d in [(2000, 64), (900, 130), (2600, 256), (3000, 64), (60, 64)]:
+        x = (torch.randn(n // 12, d, generator=g)[torch.randint(n // 12, (n,), generator=g)]
+             + 0.5 * torch.randn(n, d, generator=g)).cuda()
+        jobs.append(dict(xq=x[: n // 7].contiguous(), xg=x[n // 7:].contiguous(), k1=20, k2=6, layers=2))
+    out, need = [], []
+    for limit in (None, nbytes, 1):  # all instances, some, none
+        if limit:
+            monkeypatch.setenv("RERANK_TEST_SIDE_BYTES", str(limit))
+        with lib.Reranker(device=0, precision=precision) as R:
+            for _ in range(2):  # the second call is captured
+                res = R.run_batch(jobs)
+                torch.cuda.synchronize()
+            out.append(res)
+            need.append(R.last_info()["workspace_bytes"])
+    assert len(set(need)) == 3
+    for res in out[1:]:
+        for (i, d), (i0, d0) in zip(res, out[0]):
+            assert torch.equal(i, i0) and torch.equal(d, d0)

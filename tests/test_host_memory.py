@@ -85,3 +85,10 @@ def test_segments_of_a_large_instance_are_bounded(lib, precision):
         need = R.last_info()["workspace_bytes"] * 8 // 9
     recheck = n * 32 * 64 * 8  # its lists, the largest buffer of either plan
     assert need < recheck + (4 << 30) + (3 << 30)  # rows, copies and the final lists
+
+
+@pytest.mark.parametrize("precision,n,jobs", [("fp32", 20000, 40), ("bf16", 8000, 160)])
+def test_a_batch_takes_no_more_than_its_share_for_speed(lib, precision, n, jobs):
+    """16 GB of matrices and segments for the call, not for each instance (64 and 82 GB here)."""
+    c = Case(lib, precision, n=n, jobs=jobs)
+    assert c.wide <= c.narrow + (16 << 30) + jobs * MB
