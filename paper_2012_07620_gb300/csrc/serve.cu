@@ -32,6 +32,7 @@
 #include <condition_variable>
 #include <cstring>
 #include <deque>
+#include <memory>
 #include <mutex>
 #include <thread>
 #include <unordered_map>
@@ -213,6 +214,22 @@ size_t slot_layout(const Server& v, Slot* sl, char* base, const Shape& shmax, in
     sl->b = b;
   }
   return ((c.used + 255) & ~size_t(255)) + ws;
+}
+
+// Bytes of the resident data; with base, their places.
+size_t resident_layout(Server& v, char* base) {
+  Carver c;
+  c.base = base;
+  const size_t G = size_t(v.G), sample = v.ap_chunks ? size_t(tc_rows_append_sample()) : 0;
+  v.xg_raw = c.take<char>(G * v.d * type_size(v.dtype));
+  v.res_s = c.take<float>(G * v.K);
+  v.res_i = c.take<int32_t>(G * v.K);
+  v.res_knn_idx = c.take<int32_t>(G * v.k1);
+  v.res_knn_score = c.take<float>(G * v.k1);
+  v.res_emax = c.take<float>(4);
+  v.res_sample = c.take<char>(sample * size_t(v.dp) * esize(v.prec));
+  v.res_sample_scale = c.take<float>(sample);
+  return c.used;
 }
 
 // Layer-0 marks of a request's union rows (queries first, gallery row g at
@@ -759,8 +776,8 @@ rerank_status serve_stop(rerank_ctx* ctx) {
 // The gallery's own graph (G alone), built on slot 0's buffers at load: the
 // message lists and layers 0 .. L, kept as compact CSR.  When they do not fit
 // what the HBM budget leaves (budget_left; 0 = no budget), they are dropped
-// and requests recompute every row.  Returns a failure only for CUDA errors.
-rerank_status build_resident_graph(Server& v, cudaStream_t s0, long long* gst, size_t budget_left) {
+// (*no_room) and requests recompute every row.  Returns a failure only for CUDA errors.
+rerank_status build_resident_graph(Server& v, cudaStream_t s0, long long* gst, size_t budget_left, bool* no_room) {
   rerank_ctx* ctx = v.ctx;
   const Buffers& b = v.slots[0].b;
   const int64_t G = v.G;
@@ -786,9 +803,9 @@ rerank_status build_resident_graph(Server& v, cudaStream_t s0, long long* gst, s
   auto alloc = [&](size_t bytes) -> void* {
     void* p = nullptr;
     used += (bytes + 255) & ~size_t(255);
-    if (budget_left && used > budget_left) return nullptr;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    if ((budget_left && used > budget_left) || cudaMalloc(&p, bytes) != cudaSuccess) {
       cudaGetLastError();
+      *no_room = true;
       return nullptr;
     }
     v.res_extra.push_back(p);
@@ -878,21 +895,21 @@ rerank_status build_resident_graph(Server& v, cudaStream_t s0, long long* gst, s
   return RERANK_OK;
 }
 
-// narrow: plan with the context's rescore_m and the list kernels only (less memory).
-rerank_status serve_load(rerank_ctx* ctx, const void* xg, int64_t ng, int d, int dtype,
-                         const rerank_serve_config* sc, bool narrow = false) {
+// What a loaded gallery takes, and the shapes of its own lists and of a request.
+struct ServePlan {
+  std::unique_ptr<Server> srv;
+  Shape shg, shmax;
+  size_t gws = 0;  // the gallery's temporary workspace: it lives until the slots hold their copies
+};
+
+// narrow: with the context's rescore_m and the list kernels only (less memory).
+rerank_status serve_plan(rerank_ctx* ctx, int64_t ng, int d, int dtype, const rerank_serve_config* sc, bool narrow,
+                         ServePlan* out) {
   const int prec = ctx->cfg.precision;
-  if (prec == RERANK_PREC_FP32) return RERANK_EUNSUPPORTED;
-  if (ctx->serve) return RERANK_EUNSUPPORTED;
-  if (ctx->cfg.feature_mode == RERANK_FEAT_X) return RERANK_EUNSUPPORTED;  // dense features: rerank_run only
   const int64_t S = sc->max_query;
   const int k1 = sc->k1, k2 = sc->k2, layers = sc->layers;
-  rerank_status st = rerank_check_args(S, ng, d, dtype, k1, k2, layers, 0);
-  if (st != RERANK_OK) return st;
-  if (ng < int64_t(k1) + ctx->cfg.rescore_m || sc->slots < 0 || S > kMaxQuery) return RERANK_EINVAL;
-  RR_CUDA(cudaSetDevice(ctx->device));
-
-  Server* v = new Server();
+  out->srv.reset(new Server());
+  Server* v = out->srv.get();
   v->ctx = ctx;
   v->G = ng;
   v->S = S;
@@ -903,95 +920,81 @@ rerank_status serve_load(rerank_ctx* ctx, const void* xg, int64_t ng, int d, int
   v->k2 = k2;
   v->layers = layers;
   v->prec = prec;
-  // 1. the gallery's own exact neighbour lists: the rerank_knn pipeline on G
-  // Full lists (as in rerank_run) where the budget allows: a request then
-  // rechecks hardly any row.
+  // Full lists (as in rerank_run) where there is room: a request then rechecks
+  // hardly any row.
   const bool want_full = !narrow && ctx->cfg.rescore_m >= 16;
   v->margin = want_full ? tc_kmax() - k1 : -1;
-  Shape shg;
   Tuning tg = lookup_tuning(ctx, prec, ng, d);
   tg.rescore_m = v->margin;
-  st = plan_shape(ctx, ng, 0, d, dtype, k1, 1, 0, 0, true, false, false, 0, &shg, &tg,
-                  Side::kNone);  // lists of K entries, not bounded by a floor
-  if (st != RERANK_OK) {
-    delete v;
-    return st;
-  }
-  v->dp = shg.dp;
-  v->K = shg.K;
-  Shape shmax;
+  rerank_status st = plan_shape(ctx, ng, 0, d, dtype, k1, 1, 0, 0, true, false, false, 0, &out->shg, &tg,
+                                Side::kNone);  // lists of K entries, not bounded by a floor
+  if (st != RERANK_OK) return st;
+  v->dp = out->shg.dp;
+  v->K = out->shg.K;
   Tuning tm = lookup_tuning(ctx, prec, S + ng, d);
   tm.rescore_m = v->margin;
-  st = plan_shape(ctx, S, ng, d, dtype, k1, k2, layers, ng, false, false, true, 0, &shmax, &tm, Side::kNone);
-  if (st != RERANK_OK) {
-    delete v;
-    return st;
-  }
-  shmax.K = v->K;  // a request's lists are as long as the resident ones (at most ng places)
-  shmax.ext_feat = true;
+  st = plan_shape(ctx, S, ng, d, dtype, k1, k2, layers, ng, false, false, true, 0, &out->shmax, &tm, Side::kNone);
+  if (st != RERANK_OK) return st;
+  out->shmax.K = v->K;  // a request's lists are as long as the resident ones (at most ng places)
+  out->shmax.ext_feat = true;
   if (!narrow && ng >= 4096 && tc_append_ok((ng + 255) / 256 * 256, ctx->sm_count)) {
     v->ap_chunks = int(std::min<int64_t>((ng + 255) / 256, tc_rows_append_segs() / 4));
     v->ap_cap = tc_rows_append_cap(ng + S, v->K, v->ap_chunks);
   }
-  v->cap_h = shmax.cap_h;
+  v->cap_h = out->shmax.cap_h;
   Buffers bg;
   Carver dry;
-  const size_t gws = carve(dry, shg, bg, ctx->sm_count, prec);
-  const size_t raw = size_t(ng) * d * type_size(dtype);
-  Carver rc;
-  rc.take<char>(raw);
-  rc.take<float>(size_t(ng) * v->K);
-  rc.take<int32_t>(size_t(ng) * v->K);
-  rc.take<int32_t>(size_t(ng) * k1);
-  rc.take<float>(size_t(ng) * k1);
-  rc.take<float>(4);
-  const size_t sample_rows = v->ap_chunks ? size_t(tc_rows_append_sample()) : 0;
-  rc.take<char>(sample_rows * size_t(v->dp) * esize(prec));
-  rc.take<float>(sample_rows);
-  v->resident_bytes = rc.used;
-  v->slot_bytes = slot_layout(*v, nullptr, nullptr, shmax, ctx->sm_count);
+  out->gws = carve(dry, out->shg, bg, ctx->sm_count, prec);
+  v->resident_bytes = resident_layout(*v, nullptr);
+  v->slot_bytes = slot_layout(*v, nullptr, nullptr, out->shmax, ctx->sm_count);
+  return RERANK_OK;
+}
+
+// Slots of a plan under a budget, at most `asked`.
+int slots_in(const ServePlan& p, size_t budget, int asked) {
+  const size_t other = p.srv->resident_bytes + p.gws;
+  if (other + p.srv->slot_bytes > budget) return 0;
+  return int(std::min<size_t>(size_t(asked), (budget - other) / p.srv->slot_bytes));
+}
+
+// Whether `narrow` would hold more slots (up to nn) in the device's memory than
+// `wide` got of the nw it was to have.
+bool more_slots(const ServePlan& wide, int nw, const ServePlan& narrow, int nn) {
+  const size_t got = wide.srv->slots.size();
+  size_t free = 0, total = 0;
+  if (got >= size_t(nw) || cudaMemGetInfo(&free, &total) != cudaSuccess) return false;
+  const size_t room = free + wide.srv->resident_bytes + got * wide.srv->slot_bytes;
+  return size_t(slots_in(narrow, room, nn)) > got;
+}
+
+// Loads the gallery as planned, with up to nslots slots (fewer where the device has no
+// room for more).  *no_graph: there was no room for the resident graph.
+rerank_status serve_build(ServePlan& plan, const void* xg, int nslots, bool* no_graph) {
+  Server* v = plan.srv.get();
+  rerank_ctx* ctx = v->ctx;
+  const Shape &shg = plan.shg, &shmax = plan.shmax;
+  const int64_t ng = v->G, S = v->S;
+  const int prec = v->prec;
   const size_t budget = ctx->cfg.hbm_budget;
-  // The gallery's temporary workspace is freed before the slots are made.
-  int nslots = sc->slots ? std::min(sc->slots, kMaxSlots) : kMaxSlots;
-  if (budget) {
-    // The gallery's temporary workspace lives until the slots hold their copies.
-    if (v->resident_bytes + gws + v->slot_bytes > budget) {
-      delete v;
-      return narrow ? RERANK_EBUDGET : serve_load(ctx, xg, ng, d, dtype, sc, true);
-    }
-    nslots = int(std::min<size_t>(size_t(nslots), (budget - v->resident_bytes - gws) / v->slot_bytes));
-  }
   if (cudaMalloc(&v->res_mem, v->resident_bytes) != cudaSuccess) {
     cudaGetLastError();
-    delete v;
     return RERANK_ENOMEM;
   }
-  rc.base = v->res_mem;
-  rc.used = 0;
-  v->xg_raw = rc.take<char>(raw);
-  v->res_s = rc.take<float>(size_t(ng) * v->K);
-  v->res_i = rc.take<int32_t>(size_t(ng) * v->K);
-  v->res_knn_idx = rc.take<int32_t>(size_t(ng) * k1);
-  v->res_knn_score = rc.take<float>(size_t(ng) * k1);
-  v->res_emax = rc.take<float>(4);
-  v->res_sample = rc.take<char>(sample_rows * size_t(v->dp) * esize(prec));
-  v->res_sample_scale = rc.take<float>(sample_rows);
-  auto fail = [&](rerank_status e) {
-    free_server(v);
-    return e;
-  };
+  resident_layout(*v, v->res_mem);
   cudaStream_t s0 = nullptr;
-  if (cudaStreamCreateWithFlags(&s0, cudaStreamNonBlocking) != cudaSuccess) return fail(RERANK_ECUDA);
+  if (cudaStreamCreateWithFlags(&s0, cudaStreamNonBlocking) != cudaSuccess) return RERANK_ECUDA;
   char* gmem = nullptr;
   long long* gst = nullptr;
   long long hst[kStCount];
   rerank_status res = RERANK_OK;
   do {
-    if (cudaMemcpyAsync(v->xg_raw, xg, raw, cudaMemcpyDefault, s0) != cudaSuccess) {
+    if (cudaMemcpyAsync(v->xg_raw, xg, size_t(ng) * v->d * type_size(v->dtype), cudaMemcpyDefault, s0) != cudaSuccess) {
       res = RERANK_ECUDA;
       break;
     }
-    if (cudaMalloc(&gmem, gws) != cudaSuccess || cudaMalloc(&gst, sizeof(long long) * kStCount) != cudaSuccess) {
+    if (cudaMalloc(&gmem, plan.gws) != cudaSuccess ||
+        cudaMalloc(&gst, sizeof(long long) * kStCount) != cudaSuccess) {
+      cudaGetLastError();
       res = RERANK_ENOMEM;
       break;
     }
@@ -1071,15 +1074,50 @@ rerank_status serve_load(rerank_ctx* ctx, const void* xg, int64_t ng, int d, int
     // 3. the gallery's own graph and layers, for the rows a request leaves unchanged
     size_t left = 0;
     if (budget) {
-      const size_t spent = v->resident_bytes + gws + v->slots.size() * v->slot_bytes;
+      const size_t spent = v->resident_bytes + plan.gws + v->slots.size() * v->slot_bytes;
       left = budget > spent ? budget - spent : 1;
     }
-    res = build_resident_graph(*v, s0, gst, left);
+    res = build_resident_graph(*v, s0, gst, left, no_graph);
   } while (false);
   if (gmem) cudaFree(gmem);
   if (gst) cudaFree(gst);
   cudaStreamDestroy(s0);
-  if (res != RERANK_OK) return fail(res);
+  return res;
+}
+
+rerank_status serve_load(rerank_ctx* ctx, const void* xg, int64_t ng, int d, int dtype,
+                         const rerank_serve_config* sc) {
+  if (ctx->cfg.precision == RERANK_PREC_FP32) return RERANK_EUNSUPPORTED;
+  if (ctx->serve) return RERANK_EUNSUPPORTED;
+  if (ctx->cfg.feature_mode == RERANK_FEAT_X) return RERANK_EUNSUPPORTED;  // dense features: rerank_run only
+  rerank_status st = rerank_check_args(sc->max_query, ng, d, dtype, sc->k1, sc->k2, sc->layers, 0);
+  if (st != RERANK_OK) return st;
+  if (ng < int64_t(sc->k1) + ctx->cfg.rescore_m || sc->slots < 0 || sc->max_query > kMaxQuery) return RERANK_EINVAL;
+  RR_CUDA(cudaSetDevice(ctx->device));
+  ServePlan wide, narrow;
+  st = serve_plan(ctx, ng, d, dtype, sc, false, &wide);
+  if (st == RERANK_OK) st = serve_plan(ctx, ng, d, dtype, sc, true, &narrow);
+  if (st != RERANK_OK) return st;
+  // The wide plan answers a request faster; the narrow one is taken where the wide
+  // one holds fewer slots, or has no room for itself or for the resident graph.
+  const size_t budget = ctx->cfg.hbm_budget;
+  const int asked = sc->slots ? std::min(sc->slots, kMaxSlots) : kMaxSlots;
+  const int nw = budget ? slots_in(wide, budget, asked) : asked;
+  const int nn = budget ? slots_in(narrow, budget, asked) : asked;
+  if (!nw && !nn) return RERANK_EBUDGET;
+  ServePlan* plan = nw < nn ? &narrow : &wide;
+  bool no_graph = false;
+  st = serve_build(*plan, xg, plan == &wide ? nw : nn, &no_graph);
+  if (plan == &wide && (st == RERANK_ENOMEM || (st == RERANK_OK && (no_graph || more_slots(wide, nw, narrow, nn))))) {
+    free_server(wide.srv.release());
+    plan = &narrow;
+    st = serve_build(narrow, xg, nn, &no_graph);
+  }
+  if (st != RERANK_OK) {
+    free_server(plan->srv.release());
+    return st;
+  }
+  Server* v = plan->srv.release();
   ctx->serve = reinterpret_cast<ServeHandle*>(v);
   v->worker = std::thread(worker_loop, v);
   return RERANK_OK;
