@@ -149,7 +149,9 @@ k7_dense_scores(const float* __restrict__ h, int64_t nq, int64_t ng, int dp, con
   const int t = threadIdx.x, lane = t & 31, wq = t >> 5;
   const int tr = (wq >> 1) * 32 + (lane >> 3) * 4;  // rows tr + i and tr + 16 + i, i < 4
   const int tc = (wq & 1) * 64 + (lane & 7) * 4;    // columns tc + j and tc + 32 + j, j < 4
-  const int64_t q0 = int64_t(blockIdx.y) * STM, g0 = int64_t(blockIdx.x) * STN;
+  // One grid dimension (the second one ends at 65,535 tiles of queries), gallery tiles first.
+  const unsigned gtiles = unsigned((ng + STN - 1) / STN);
+  const int64_t q0 = int64_t(blockIdx.x / gtiles) * STM, g0 = int64_t(blockIdx.x % gtiles) * STN;
   f32x2 hi[32], p[32];
 #pragma unroll
   for (int j = 0; j < 32; ++j) {
@@ -265,7 +267,7 @@ int launch_dense_layer(const Shape& sh, const float* hin, float* hout, const int
 int launch_dense_scores(const Shape& sh, const float* h, double* inv, float* S, cudaStream_t s) {
   const int T = 256;
   k7_dense_inv_norms<<<unsigned((sh.n * kWarp + T - 1) / T), T, 0, s>>>(h, sh.n, sh.dp, inv);
-  const dim3 grid(unsigned((sh.ng + STN - 1) / STN), unsigned((sh.nq + STM - 1) / STM));
+  const unsigned grid = unsigned(((sh.ng + STN - 1) / STN) * ((sh.nq + STM - 1) / STM));
   cudaFuncSetAttribute(k7_dense_scores, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SSMEM));
   k7_dense_scores<<<grid, STHREADS, SSMEM, s>>>(h, sh.nq, sh.ng, sh.dp, inv, S);
   return 2;
