@@ -523,11 +523,12 @@ rerank_status map_status(const long long* h, int precision, rerank_info* info, i
   return RERANK_OK;
 }
 
-// The same instance planned for the list kernels of the similarity stage.
-rerank_status plan_lists(const rerank_ctx* ctx, Shape* sh) {
+// The same instance planned with less memory for the similarity stage.
+rerank_status plan_smaller(const rerank_ctx* ctx, Shape* sh) {
   const Shape o = *sh;
+  const Side side = o.side == Side::kNone ? Side::kLean : Side::kNone;
   return plan_shape(ctx, o.nq, o.ng, o.d, o.dtype, o.k1, o.k2, o.layers, o.topk, o.knn_only, o.host_in, o.host_out,
-                    o.cap_h, sh, nullptr, Side::kNone);
+                    o.cap_h, sh, nullptr, side);
 }
 
 // One attempt of the pipeline.  Returns OK, or the mapped device error.
@@ -535,19 +536,18 @@ rerank_status run_once(rerank_ctx* ctx, const void* xq, const void* xg, int32_t*
                        cudaStream_t s) {
   JobRun j;
   j.sh = ctx->shape;
-  Carver dry;
-  size_t need = carve(dry, j.sh, j.b, ctx->sm_count, ctx->cfg.precision);
-  const bool wide = j.sh.segs > 0 || j.sh.smat;
-  rerank_status st = wide ? ensure_wide_workspace(ctx, need) : ensure_workspace(ctx, need);
-  if (wide && (st == RERANK_EBUDGET || st == RERANK_ENOMEM)) {
-    // No room for the append pass's segments (or the matrix): the list kernels need less.
-    st = plan_lists(ctx, &j.sh);
+  rerank_status st = RERANK_OK;
+  for (;;) {
+    Carver dry;
+    const size_t need = carve(dry, j.sh, j.b, ctx->sm_count, ctx->cfg.precision);
+    const bool smaller = j.sh.side != Side::kLean;  // there is a plan that needs less
+    st = smaller ? ensure_wide_workspace(ctx, need) : ensure_workspace(ctx, need);
+    if (!smaller || (st != RERANK_EBUDGET && st != RERANK_ENOMEM)) break;
+    // No room for the append pass's segments or the matrix, or for so many lists.
+    st = plan_smaller(ctx, &j.sh);
     if (st != RERANK_OK) return st;
     ctx->shape = j.sh;
     j.b = Buffers{};
-    Carver again;
-    need = carve(again, j.sh, j.b, ctx->sm_count, ctx->cfg.precision);
-    st = ensure_workspace(ctx, need);
   }
   if (st != RERANK_OK) return st;
   Carver real;
@@ -602,6 +602,7 @@ rerank_status plan_shape(const rerank_ctx* ctx, int64_t nq, int64_t ng, int d, i
                          int64_t topk, bool knn_only, bool host_in, bool host_out, int64_t cap_hint, Shape* out,
                          const Tuning* tune, Side side) {
   Shape sh;
+  sh.side = side;
   sh.nq = nq;
   sh.ng = ng;
   sh.n = nq + ng;
@@ -632,7 +633,8 @@ rerank_status plan_shape(const rerank_ctx* ctx, int64_t nq, int64_t ng, int d, i
   // tensor-core products over all columns in the recheck (market: 4,004 rows
   // with 42 places, 6 with 64; recheck 0.88 -> 0.19 ms).  Smaller margins that
   // the caller or the tuning table asks for are kept.
-  const bool may_append = tc && side != Side::kNone && tc_append_ok(sh.np, ctx->sm_count);
+  const bool may_side = side == Side::kBands || side == Side::kWhole;
+  const bool may_append = tc && may_side && tc_append_ok(sh.np, ctx->sm_count);
   const bool full = may_append && sh.tune.rescore_m < 0 && m >= 16;
   int64_t K = std::min<int64_t>(full ? kmax : int64_t(k1) + std::max(m, 0), sh.n);
   K = std::min<int64_t>(K, kmax);
@@ -647,15 +649,17 @@ rerank_status plan_shape(const rerank_ctx* ctx, int64_t nq, int64_t ng, int d, i
   const int irows = tc ? tc_item_rows() : 128;
   const int units = ctx->sm_count * 128 / irows;
   int chunks = choose_chunks(sh.np / irows, sh.np / (tc ? 256 : 128), units, sh.tune.sim_chunks);
-  // An item of the paired kernels spans at most tc_max_item_tiles() tiles.
-  if (tc) chunks = std::max<int>(chunks, int((sh.np / 256 + tc_max_item_tiles() - 1) / tc_max_item_tiles()));
+  // An item of the paired kernels spans at most tc_max_item_tiles() tiles (longer
+  // ones, where memory is too short for the lists of more, take single CTAs).
+  if (tc && side != Side::kLean)
+    chunks = std::max<int>(chunks, int((sh.np / 256 + tc_max_item_tiles() - 1) / tc_max_item_tiles()));
   sh.P = std::min(chunks, 32 / lpc) * lpc;
   if (may_append) {
     tc_append_plan(sh.n, sh.np, sh.dp, sh.K, chunks, &sh.segs, &sh.seg_cap, &sh.sample);
     sh.seg_rows = side == Side::kBands ? tc_append_band(sh.n, sh.segs, sh.seg_cap) : sh.n;
     sh.P = 1;
   }
-  if (!tc && side != Side::kNone && size_t(sh.np) * sh.np * 4 <= kSideBytes) {
+  if (!tc && may_side && size_t(sh.np) * sh.np * 4 <= kSideBytes) {
     sh.smat = true;
     sh.P = 1;
   }
@@ -848,9 +852,8 @@ rerank_status run_batch(rerank_ctx* ctx, rerank_job* jobs, int njobs, cudaStream
   const size_t inst_bytes = tc_batch_inst_bytes() * size_t(njobs);
   size_t inst_off = 0, total = 0;
   rerank_status st = RERANK_OK;
-  // With the append pass's segments; without them where they do not fit.
-  for (int attempt = 0; attempt < 2; ++attempt) {
-    bool append = false;
+  // With the append pass's segments; without them, or with fewer lists, where they do not fit.
+  for (const Side plan : {Side::kWhole, Side::kNone, Side::kLean}) {
     size_t side = batch_side_bytes();  // left for the instances to come
     total = 0;
     for (int i = 0; i < njobs; ++i) {
@@ -864,11 +867,10 @@ rerank_status run_batch(rerank_ctx* ctx, rerank_job* jobs, int njobs, cudaStream
         return plan_shape(ctx, jb.nq, jb.ng, jb.d, jb.dtype, jb.k1, jb.k2, jb.layers, topk, false, host_in, host_out,
                           0, &run.sh, nullptr, w);
       };
-      st = plan_side(attempt == 0 ? Side::kWhole : Side::kNone);
+      st = plan_side(plan);
       if (st == RERANK_OK && side_bytes(run.sh) > side) st = plan_side(Side::kNone);
       if (st != RERANK_OK) return st;
       side -= side_bytes(run.sh);
-      append = append || run.sh.segs > 0 || run.sh.smat;
       Carver dry;
       const size_t need = carve(dry, run.sh, run.b, ctx->sm_count, ctx->cfg.precision);
       total = (total + 255) & ~size_t(255);
@@ -878,8 +880,8 @@ rerank_status run_batch(rerank_ctx* ctx, rerank_job* jobs, int njobs, cudaStream
     total = (total + 255) & ~size_t(255);
     inst_off = total;
     if (tc_batch) total += inst_bytes;
-    st = append ? ensure_wide_workspace(ctx, total) : ensure_workspace(ctx, total);
-    if (!append || (st != RERANK_EBUDGET && st != RERANK_ENOMEM)) break;
+    st = plan != Side::kLean ? ensure_wide_workspace(ctx, total) : ensure_workspace(ctx, total);
+    if (st != RERANK_EBUDGET && st != RERANK_ENOMEM) break;
   }
   if (st != RERANK_OK) return st;
   st = ensure_streams(ctx);

@@ -139,6 +139,15 @@ struct Buffers {
   int64_t* scan_tmp = nullptr;
 };
 
+// The memory that the similarity stage may take to be faster: the append pass's
+// segments, or the FP32 matrix.
+enum class Side {
+  kBands,  // the segments of one band of rows after the other share theirs
+  kWhole,  // the segments of all rows at once (batched calls: one launch over all instances)
+  kNone,   // none: the list kernels
+  kLean    // nor more lists than the work split wants (pairs need one per 65,536 columns, single CTAs do not)
+};
+
 struct Shape {
   int64_t nq = 0, ng = 0, n = 0, np = 0;
   int d = 0, dp = 0, dtype = 0;
@@ -161,6 +170,7 @@ struct Shape {
   int hash_slots = 0;      // slots of each global hash table (big-row path)
   int rank_ctas = 0;
   int64_t rank_scratch_per_cta = 0;
+  Side side = Side::kBands;  // what it was planned with
   Tuning tune;             // launch shapes of this instance
 };
 
@@ -464,13 +474,6 @@ bool is_host_ptr(const void* p);
 size_t type_size(int dtype);
 int choose_chunks(int64_t row_blocks, int64_t col_tiles, int sm_count, int forced);
 size_t carve(Carver& c, const Shape& sh, Buffers& b, int sm_count, int precision);
-// The memory that the similarity stage may take to be faster: the append pass's
-// segments, or the FP32 matrix.
-enum class Side {
-  kNone,   // none: the list kernels
-  kBands,  // the segments of one band of rows after the other share theirs
-  kWhole   // the segments of all rows at once (batched calls: one launch over all instances)
-};
 rerank_status plan_shape(const rerank_ctx* ctx, int64_t nq, int64_t ng, int d, int dtype, int k1, int k2,
                          int layers, int64_t topk, bool knn_only, bool host_in, bool host_out, int64_t cap_hint,
                          Shape* out, const Tuning* tune = nullptr,  // tune: override of the table lookup

@@ -902,9 +902,12 @@ struct ServePlan {
   size_t gws = 0;  // the gallery's temporary workspace: it lives until the slots hold their copies
 };
 
-// narrow: with the context's rescore_m and the list kernels only (less memory).
-rerank_status serve_plan(rerank_ctx* ctx, int64_t ng, int d, int dtype, const rerank_serve_config* sc, bool narrow,
+// side: kBands with full lists and the append pass; else with the context's rescore_m
+// and the list kernels only (less memory).  The gallery's own lists come from the
+// list kernels in any case: they are lists of K entries, not bounded by a floor.
+rerank_status serve_plan(rerank_ctx* ctx, int64_t ng, int d, int dtype, const rerank_serve_config* sc, Side side,
                          ServePlan* out) {
+  const bool narrow = side != Side::kBands;
   const int prec = ctx->cfg.precision;
   const int64_t S = sc->max_query;
   const int k1 = sc->k1, k2 = sc->k2, layers = sc->layers;
@@ -927,7 +930,7 @@ rerank_status serve_plan(rerank_ctx* ctx, int64_t ng, int d, int dtype, const re
   Tuning tg = lookup_tuning(ctx, prec, ng, d);
   tg.rescore_m = v->margin;
   rerank_status st = plan_shape(ctx, ng, 0, d, dtype, k1, 1, 0, 0, true, false, false, 0, &out->shg, &tg,
-                                Side::kNone);  // lists of K entries, not bounded by a floor
+                                narrow ? side : Side::kNone);
   if (st != RERANK_OK) return st;
   v->dp = out->shg.dp;
   v->K = out->shg.K;
@@ -937,6 +940,7 @@ rerank_status serve_plan(rerank_ctx* ctx, int64_t ng, int d, int dtype, const re
   if (st != RERANK_OK) return st;
   out->shmax.K = v->K;  // a request's lists are as long as the resident ones (at most ng places)
   out->shmax.ext_feat = true;
+  out->shmax.P = 1;  // its lists are the slot's own (pa, pb, pm)
   if (!narrow && ng >= 4096 && tc_append_ok((ng + 255) / 256 * 256, ctx->sm_count)) {
     v->ap_chunks = int(std::min<int64_t>((ng + 255) / 256, tc_rows_append_segs() / 4));
     v->ap_cap = tc_rows_append_cap(ng + S, v->K, v->ap_chunks);
@@ -957,14 +961,14 @@ int slots_in(const ServePlan& p, size_t budget, int asked) {
   return int(std::min<size_t>(size_t(asked), (budget - other) / p.srv->slot_bytes));
 }
 
-// Whether `narrow` would hold more slots (up to nn) in the device's memory than
-// `wide` got of the nw it was to have.
-bool more_slots(const ServePlan& wide, int nw, const ServePlan& narrow, int nn) {
-  const size_t got = wide.srv->slots.size();
+// Whether `other` would hold more slots (up to no) in the device's memory than `p`
+// got of the np it was to have.
+bool more_slots(const ServePlan& p, int np, const ServePlan& other, int no) {
+  const size_t got = p.srv->slots.size();
   size_t free = 0, total = 0;
-  if (got >= size_t(nw) || cudaMemGetInfo(&free, &total) != cudaSuccess) return false;
-  const size_t room = free + wide.srv->resident_bytes + got * wide.srv->slot_bytes;
-  return size_t(slots_in(narrow, room, nn)) > got;
+  if (got >= size_t(np) || cudaMemGetInfo(&free, &total) != cudaSuccess) return false;
+  const size_t room = free + p.srv->resident_bytes + got * p.srv->slot_bytes;
+  return size_t(slots_in(other, room, no)) > got;
 }
 
 // Loads the gallery as planned, with up to nslots slots (fewer where the device has no
@@ -1094,30 +1098,32 @@ rerank_status serve_load(rerank_ctx* ctx, const void* xg, int64_t ng, int d, int
   if (st != RERANK_OK) return st;
   if (ng < int64_t(sc->k1) + ctx->cfg.rescore_m || sc->slots < 0 || sc->max_query > kMaxQuery) return RERANK_EINVAL;
   RR_CUDA(cudaSetDevice(ctx->device));
-  ServePlan wide, narrow;
-  st = serve_plan(ctx, ng, d, dtype, sc, false, &wide);
-  if (st == RERANK_OK) st = serve_plan(ctx, ng, d, dtype, sc, true, &narrow);
-  if (st != RERANK_OK) return st;
-  // The wide plan answers a request faster; the narrow one is taken where the wide
-  // one holds fewer slots, or has no room for itself or for the resident graph.
+  // The first plan answers a request fastest; a smaller one is taken where it holds
+  // more slots, or where the larger one has no room for itself or for the resident graph.
+  constexpr Side kSides[] = {Side::kBands, Side::kNone, Side::kLean};
+  constexpr int kPlans = 3;
+  ServePlan plans[kPlans];
+  int slots[kPlans];
   const size_t budget = ctx->cfg.hbm_budget;
   const int asked = sc->slots ? std::min(sc->slots, kMaxSlots) : kMaxSlots;
-  const int nw = budget ? slots_in(wide, budget, asked) : asked;
-  const int nn = budget ? slots_in(narrow, budget, asked) : asked;
-  if (!nw && !nn) return RERANK_EBUDGET;
-  ServePlan* plan = nw < nn ? &narrow : &wide;
-  bool no_graph = false;
-  st = serve_build(*plan, xg, plan == &wide ? nw : nn, &no_graph);
-  if (plan == &wide && (st == RERANK_ENOMEM || (st == RERANK_OK && (no_graph || more_slots(wide, nw, narrow, nn))))) {
-    free_server(wide.srv.release());
-    plan = &narrow;
-    st = serve_build(narrow, xg, nn, &no_graph);
+  int at = 0;
+  for (int k = 0; k < kPlans; ++k) {
+    st = serve_plan(ctx, ng, d, dtype, sc, kSides[k], &plans[k]);
+    if (st != RERANK_OK) return st;
+    slots[k] = budget ? slots_in(plans[k], budget, asked) : asked;
+    if (slots[k] > slots[at]) at = k;
   }
-  if (st != RERANK_OK) {
-    free_server(plan->srv.release());
-    return st;
+  if (!slots[at]) return RERANK_EBUDGET;
+  for (;; ++at) {
+    bool no_graph = false;
+    st = serve_build(plans[at], xg, slots[at], &no_graph);
+    const bool last = at + 1 == kPlans;
+    if (st == RERANK_OK && (last || (!no_graph && !more_slots(plans[at], slots[at], plans[kPlans - 1], slots[kPlans - 1]))))
+      break;
+    free_server(plans[at].srv.release());
+    if (last || (st != RERANK_OK && st != RERANK_ENOMEM)) return st;
   }
-  Server* v = plan->srv.release();
+  Server* v = plans[at].srv.release();
   ctx->serve = reinterpret_cast<ServeHandle*>(v);
   v->worker = std::thread(worker_loop, v);
   return RERANK_OK;

@@ -16,7 +16,7 @@
 namespace {
 
 constexpr int kDevices = 2;
-constexpr size_t kDefaultShared = 48 * 1024;
+constexpr size_t kDefaultShared = 48 * 1024, kMostShared = 227 * 1024;
 const int kSms[kDevices] = {152, 76};
 
 struct Block {
@@ -154,6 +154,7 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
 }
 cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {
   std::lock_guard<std::mutex> lk(S().mu);
+  if (v < 0 || size_t(v) > kMostShared) return fail(cudaErrorInvalidValue);
   if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) {
     size_t& limit = S().shared[{f, t_dev}];
     if (size_t(v) < limit) ++S().counts["lowered " + S().names[f]];
@@ -185,7 +186,7 @@ cudaError_t cudaGetDeviceProperties(cudaDeviceProp* p, int d) {
   p->major = 10;
   p->minor = 3;
   p->multiProcessorCount = kSms[d];
-  p->sharedMemPerBlockOptin = 227 * 1024;
+  p->sharedMemPerBlockOptin = kMostShared;
   return cudaSuccess;
 }
 const char* cudaGetErrorString(cudaError_t) { return "error of the stand-in runtime"; }

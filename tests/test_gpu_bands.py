@@ -55,3 +55,24 @@ def test_batch_with_and_without_segments_or_matrix(lib, monkeypatch, precision, 
     for res in out[1:]:
         for (i, d), (i0, d0) in zip(res, out[0]):
             assert torch.equal(i, i0) and torch.equal(d, d0)
+
+
+@pytest.mark.parametrize("precision", ["bf16", "fp8"])
+def test_large_lists_with_less_and_less_memory(lib, precision):
+    """304 column tiles in one chunk: the append pass, lists on pairs (two chunks of
+    columns), and lists on single CTAs (one) as the budget shrinks."""
+    n, d, k = 77800, 64, 10
+    g = torch.Generator(device="cuda").manual_seed(8)
+    c = torch.randn(n // 12, d, generator=g, device="cuda")
+    x = c[torch.randint(len(c), (n,), generator=g, device="cuda")]
+    x += 0.5 * torch.randn(n, d, generator=g, device="cuda")
+    budget, out, need = 0, [], []
+    for _ in range(4):  # (the first allocation within a new plan has an eighth to spare)
+        with lib.Reranker(device=0, precision=precision, hbm_budget=budget) as R:
+            out.append(R.knn(x, k))
+            torch.cuda.synchronize()
+            need.append(R.last_info()["workspace_bytes"])
+        budget = (need[-1] * 8 // 9 if len(need) == 1 else need[-1]) - 1
+    assert need == sorted(need, reverse=True) and len(set(need)) == 4
+    for i, s in out[1:]:
+        assert torch.equal(i, out[0][0]) and torch.equal(s, out[0][1])

@@ -92,3 +92,12 @@ def test_a_batch_takes_no_more_than_its_share_for_speed(lib, precision, n, jobs)
     """16 GB of matrices and segments for the call, not for each instance (64 and 82 GB here)."""
     c = Case(lib, precision, n=n, jobs=jobs)
     assert c.wide <= c.narrow + (16 << 30) + jobs * MB
+
+
+@pytest.mark.parametrize("n,d,k,m", [(724988, 7, 27, 0), (458472, 7, 38, 16)])
+def test_large_lists_in_little_memory(lib, n, d, k, m):
+    """8 GB hold these lists where a row has no more of them than the work split wants."""
+    lib.fake.fake_reset(1 << 40)
+    x, oi, os = (fake_cuda.device(lib, (n, w), t) for w, t in ((d, "f4"), (k, "i4"), (k, "f4")))
+    with lib.Reranker(device=0, precision="bf16", rescore_m=m, hbm_budget=8 << 30) as R:
+        R.knn(x, k, oi, os, stream=0)

@@ -1,5 +1,7 @@
 """How a gallery is loaded at the limits of memory, on a stand-in runtime with a set
 capacity: the plan with full lists and segments gives way to the one without."""
+import ctypes
+
 import pytest
 
 import fake_cuda
@@ -72,3 +74,18 @@ def test_the_resident_graph_is_not_given_up_for_the_larger_plan(gallery):
         assert info["reuse_layers"] == 1
         nbytes += MB
     assert info["reuse_layers"] == 1  # the first budget that the larger plan is taken with
+
+
+@pytest.mark.parametrize("precision,ng,d,m,k1,k2,layers,max_query,slots", [
+    ("fp8", 404302, 713, 0, 36, 2, 2, 64, 1), ("bf16", 503430, 187, 16, 2, 2, 4, 500, 2),
+    ("fp8", 228312, 335, 4, 32, 5, 3, 1024, 2), ("fp8", 225405, 1, 100, 7, 3, 0, 64, 3)])
+def test_large_galleries_in_32_gigabytes(gallery, precision, ng, d, m, k1, k2, layers, max_query, slots):
+    lib = gallery.lib
+    lib.fake.fake_reset(1 << 40)
+    x = fake_cuda.device(lib, (ng, d))
+    lib.fake.fake_reset(lib.fake.fake_used(0) + (32 << 30) - ng * d * 4)
+    with lib.Reranker(device=0, precision=precision, rescore_m=m) as R:
+        R.load_gallery(x, max_query, k1, k2, layers, slots=8)
+        info = R.serve_info()
+        assert info["slots"] >= slots and info["reuse_layers"] == 1
+    lib.fake.cudaFree(ctypes.c_void_p(x.ctypes.data))
