@@ -221,7 +221,9 @@ __device__ int merge_lists(WarpSmem& w, const float* ls, const int32_t* li, int 
   // score: it was either dropped from a full chunk list (below that list's
   // K-th, which the merged K-th cannot undercut), skipped by a floor (another
   // chunk's K-th, same argument) or not taken by the merge.  With fewer than K
-  // candidates nothing was dropped or skipped.
+  // candidates no list dropped anything, but columns below a floor that was there
+  // from the start (a sampled one, or the stage's before) were skipped: the callers
+  // replace B by that floor (RefineFloors::in).
   __syncwarp();
   B = cnt == K ? w.g[K - 1] : -FLT_MAX;
   return cnt;

@@ -390,7 +390,7 @@ __device__ __forceinline__ void zero_tail(const RankArgs& A, int64_t q, int cnt,
 // adding atomic returns the old score), and everything after works on that list
 // instead of on all scores: bucket counts, scatter, in-bucket places, and the
 // clean-up for the next query.  The keys are the listed 16-bit indices and the
-// scores themselves, so that a gallery of up to ~19,800 rows leaves room for two
+// scores themselves, so that a gallery of up to 20,072 rows leaves room for two
 // CTAs per SM: one writes its zero tail (7,300 cycles of HBM at the Market
 // shape) while the other computes.  Queries with more non-zeros, or with a bucket
 // too crowded for counting, are handed to k6_rank through `over`.
@@ -1133,7 +1133,7 @@ int launch_rank_queries(const Shape& sh, const Buffers& b, int src, int32_t* out
   int nl = 1;
   // Queries with few non-zeros first, where the scores fit the light kernel's
   // shared memory beside its lists: two CTAs of 512 threads per SM while they
-  // fit twice (up to ~19,800 gallery rows), else one of 1,024.
+  // fit twice (up to 20,072 gallery rows; 48,372 fit once), else one of 1,024.
   const size_t light = light_smem_bytes(ng);
   if (light <= kSmemMax && ng <= 65536 && A.sort_cap == SORT_CAP) {
     cudaMemsetAsync(A.over_count, 0, sizeof(int32_t), s);
