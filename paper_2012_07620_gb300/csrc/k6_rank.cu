@@ -70,10 +70,14 @@ __global__ void k5_fill(const int64_t* __restrict__ start, const int32_t* __rest
 // column to the total and keeps the old value (base, per CTA and column), the
 // filling pass starts its own places there.  An entry costs a shared-memory atomic
 // instead of a scattered global one: both passes 87 -> 57 us at Market (2.2 M entries),
-// 440 -> 315 at market_hard (14 M).  Not below 8,192 gallery rows or above 32,768
-// columns, where clearing, storing and loading every CTA's columns costs what the
-// entries save (50,000 vertices, 4 M entries: no gain), nor for a request
-// (rows_sel), which has few rows.
+// 440 -> 315 at market_hard (14 M).  Above 32,768 columns a CTA's counts leave
+// little L1 and dense layers lose, slightly from 28,000 on; both sides, the ranking
+// stage of 200 queries (us, without -> with):
+//   rows            9,400       23,100      28,000      32,700       45,000       55,000
+//   sparse layer    88 -> 70    158 -> 123  170 -> 139  225 -> 195   269 -> 236   270 -> 250
+//   dense layer     338 -> 244  708 -> 602  776 -> 799  1617 -> 1642 1928 -> 2278 2084 -> 2758
+// The lower line is on the safe side: 3,000 rows gain too (76 -> 51, dense 204 -> 137).
+// Not for a request (rows_sel), which has few rows.
 constexpr int K5T = 1024;
 constexpr int64_t kColsMax = 32768;  // 128 KB of shared memory; places fit 32 bits (n^2 < 2^32)
 constexpr int64_t kColsMinRows = 8192;
