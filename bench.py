@@ -248,10 +248,10 @@ def _config(args, w):
 
 # DRAM bytes (read + write) of one similarity launch, from ncu captures of the
 # current kernel (profiles/); None where no capture of it exists.
-SIM_TRAFFIC_BYTES = {("bf16", "market"): 996.1e6}  # profiles/k1_tc2_append_bf16_market_23k_d2048.md
+SIM_TRAFFIC_BYTES = {("bf16", "market"): 625.0e6}  # profiles/k1_tc2_append_bf16_market_23k_d2048.md
 # DRAM bytes read by the refinement's first pass, same source
 # (profiles/k2_refine_cta_bf16_market_23k_d2048.md).
-REFINE_DRAM_BYTES = {("bf16", "market"): 1.640e9}
+REFINE_DRAM_BYTES = {("bf16", "market"): 1.639e9}
 
 
 def _stage_rooflines(precision, stages, nq, ng, d, k1, k2, rescore_m, h_nnz, layers, workload):
