@@ -89,7 +89,7 @@ def test_segments_of_a_large_instance_are_bounded(lib, precision):
 
 @pytest.mark.parametrize("precision,n,jobs", [("fp32", 20000, 40), ("bf16", 8000, 160)])
 def test_a_batch_takes_no_more_than_its_share_for_speed(lib, precision, n, jobs):
-    """16 GB of matrices and segments for the call, not for each instance (64 and 82 GB here)."""
+    """16 GB of matrices and segments for the call, not for each instance (64 and 21 GB here)."""
     c = Case(lib, precision, n=n, jobs=jobs)
     assert c.wide <= c.narrow + (16 << 30) + jobs * MB
 
